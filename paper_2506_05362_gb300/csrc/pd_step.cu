@@ -242,13 +242,14 @@ __device__ __forceinline__ double3 wall_overlap_terms(const double *wall_pos, co
 // WX (the kernels launched when friction or inclusion-exclusion is on) also the
 // wall friction and the multi-wall terms, which other kernels do not carry.
 template <bool WX>
-__device__ __forceinline__ unsigned wall_force(const StepParams &p, const double *wp, double px, double py, double pz,
+__device__ __forceinline__ unsigned wall_force(const StepParams &p, const double *wp, unsigned near, double px, double py, double pz,
                                                double vol, double vx, double vy, double vz, double &fx,
                                                double &fy, double &fz, double *react)
 {
     unsigned e = 0;
     int touching = 0;
-    for (int l = 0; l < p.walls.nw; ++l) {
+    for (; near; near &= near - 1) {  // the walls that may touch, in ascending order
+        const int l = __ffs(near) - 1;
         const double nx = p.walls.n[l][0], ny = p.walls.n[l][1], nz = p.walls.n[l][2];
         const double *w = wp + 3 * l;
         double d = dadd(dadd(dmul(px - w[0], nx), dmul(py - w[1], ny)), dmul(pz - w[2], nz));
@@ -289,6 +290,29 @@ __device__ __forceinline__ unsigned wall_force(const StepParams &p, const double
         fx += o.x; fy += o.y; fz += o.z;
     }
     return e;
+}
+
+// The walls in FP32 relative to the domain centre, one per block in shared memory, for
+// the test that spares rows away from every wall the FP64 evaluation.  (Converted
+// per row, the doubles took a third of a packing's step on the narrow FP64 pipe.)
+struct WallF {
+    float n[3], q[3], m;  // normal, point - centre, the point's and the centre's part of the margin
+};
+
+// fills the table from the current wall points wp; a barrier must follow
+__device__ __forceinline__ void load_walls_f(const StepParams &p, const double *wp, WallF *wf)
+{
+    const int l = threadIdx.x;
+    if (l >= p.walls.nw) return;
+    WallF w;
+    w.m = 0.f;
+    for (int a = 0; a < 3; ++a) {
+        const float c = (float)p.centre[a];
+        w.n[a] = (float)p.walls.n[l][a];
+        w.q[a] = (float)wp[3 * l + a] - c;
+        w.m += fabsf(w.q[a]) + fabsf(c);
+    }
+    wf[l] = w;
 }
 
 // x_lo rides in the spare lanes of the u records as BF16: R1.w = (x_lo.x, x_lo.y),
@@ -580,7 +604,7 @@ __device__ __forceinline__ unsigned epilogue_component(const StepParams &p, int6
 // warp calls it (inactive rows included) so that the shuffles that broadcast a
 // wall force and sum |v|^2 are uniform.
 template <int G, bool WX>
-__device__ __forceinline__ unsigned epilogue_lanes(const StepParams &p, const double *wp, int64_t row, bool active,
+__device__ __forceinline__ unsigned epilogue_lanes(const StepParams &p, const double *wp, const WallF *wf, int64_t row, bool active,
                                                    int gl, float Fx,
                                                    float Fy, float Fz, const float4 &oxh, const float4 &uh,
                                                    const float4 &ul, const float4 &vh, const float4 &vl,
@@ -589,25 +613,26 @@ __device__ __forceinline__ unsigned epilogue_lanes(const StepParams &p, const do
     unsigned err = 0;
     if (p.walls.nw) {  // uniform: a kernel parameter
         float wx = 0.f, wy = 0.f, wz = 0.f;
-        if (active && gl == 0) {
+        // the group's lanes test the walls, lane l walls l, l + G, ...
+        unsigned near = 0;
+        if (active) {
             const float px = oxh.x + uh.x, py = oxh.y + uh.y, pz = oxh.z + uh.z;
-            const float cx = (float)p.centre[0], cy = (float)p.centre[1], cz = (float)p.centre[2];
-            bool near = false;
-            for (int l = 0; l < p.walls.nw; ++l) {
-                const double *w = wp + 3 * l;
-                const float qx = (float)w[0] - cx, qy = (float)w[1] - cy, qz = (float)w[2] - cz;
-                const float d = (px - qx) * (float)p.walls.n[l][0] + (py - qy) * (float)p.walls.n[l][1] +
-                                (pz - qz) * (float)p.walls.n[l][2];
-                const float margin = 1e-6f * (fabsf(px) + fabsf(py) + fabsf(pz) + fabsf(qx) + fabsf(qy) +
-                                              fabsf(qz) + fabsf(cx) + fabsf(cy) + fabsf(cz));
-                near |= d < p.Rc_f + margin;
+            const float pm = fabsf(px) + fabsf(py) + fabsf(pz);
+            for (int l = gl; l < p.walls.nw; l += G) {
+                const WallF &w = wf[l];
+                const float d = (px - w.q[0]) * w.n[0] + (py - w.q[1]) * w.n[1] + (pz - w.q[2]) * w.n[2];
+                if (d < p.Rc_f + 1e-6f * (pm + w.m)) near |= 1u << l;
             }
-            if (near) {
+        }
+        if (__any_sync(0xffffffffu, near != 0)) {
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) near |= __shfl_xor_sync(0xffffffffu, near, o);
+            if (near && gl == 0) {
                 const dbl4 ox = p.x4[row];
                 const double ux = df_to_double(df{uh.x, ul.x}), uy = df_to_double(df{uh.y, ul.y}),
                              uz = df_to_double(df{uh.z, ul.z});
                 double fx = 0.0, fy = 0.0, fz = 0.0;
-                err |= wall_force<WX>(p, wp, dadd(ox.x, ux), dadd(ox.y, uy), dadd(ox.z, uz), ox.w, df_to_double(df{vh.x, vl.x}),
+                err |= wall_force<WX>(p, wp, near, dadd(ox.x, ux), dadd(ox.y, uy), dadd(ox.z, uz), ox.w, df_to_double(df{vh.x, vl.x}),
                                   df_to_double(df{vh.y, vl.y}), df_to_double(df{vh.z, vl.z}), fx, fy, fz, react);
                 wx = (float)fx; wy = (float)fy; wz = (float)fz;
             }
@@ -631,14 +656,29 @@ __device__ __forceinline__ unsigned epilogue_lanes(const StepParams &p, const do
 // bonded; otherwise (gx, gy, gz) = its force density on i.  The predicate is
 // evaluated in FP64 without FMA, so contact pair sets are exact.
 template <bool MIXED>
-__device__ __forceinline__ bool contact_term(const StepParams &p, int64_t q, const dbl4 &ox, double pix, double piy,
-                                             double piz, int gi, double R2, double &gx, double &gy, double &gz)
+__device__ __forceinline__ bool contact_term(const StepParams &p, int64_t q, const float4 &o0, const float4 &o1,
+                                             const dbl4 &ox, double pix, double piy, double piz, int gi, double R2,
+                                             double &gx, double &gy, double &gz)
 {
     const int2 cj = p.cand[q];
     const int j = cj.x;
     if (cj.y >= 0) {
         const uint32_t w = *((volatile uint32_t *)(p.brk + (cj.y >> 5)));
         if (!((w >> (cj.y & 31)) & 1u)) return false;  // bond intact
+    }
+    if (MIXED) {
+        // FP32 first: a pair that is clearly apart needs no FP64 (that pipe is narrow).
+        // Each difference of the records' high halves is off by at most 2^-24 of itself,
+        // and the low halves left out are at most 2^-24 of x and u; the margins below are
+        // four times that
+        const float4 a0 = __ldg(p.xh4 + RECX * (int64_t)j), a1 = __ldg(p.uh_in + REC * (int64_t)j);
+        const float x0 = a0.x - o0.x, x1 = a0.y - o0.y, x2 = a0.z - o0.z;
+        const float u0 = a1.x - o1.x, u1 = a1.y - o1.y, u2 = a1.z - o1.z;
+        const float ex = x0 + u0, ey = x1 + u1, ez = x2 + u2;
+        const float lim = p.Rc_f * 1.00001f +
+                          5e-7f * (((fabsf(x0) + fabsf(x1)) + (fabsf(x2) + fabsf(u0))) + (fabsf(u1) + fabsf(u2))) +
+                          2.5e-7f * (((fabsf(o0.x) + fabsf(o0.y)) + (fabsf(o0.z) + fabsf(o1.x))) + (fabsf(o1.y) + fabsf(o1.z)));
+        if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > lim * lim) return false;
     }
     const dbl4 xj = p.x4[j], uj = load_u_t<MIXED>(p, j);
     const double dx = dadd(xj.x, uj.x) - pix;
@@ -648,10 +688,13 @@ __device__ __forceinline__ bool contact_term(const StepParams &p, int64_t q, con
     if (!(d2 < R2)) return false;
     const double dn = sqrt(d2);
     if (dn == 0.0) return false;
-    double mag;
-    const double xx = xj.x - ox.x, xy = xj.y - ox.y, xz = xj.z - ox.z;
-    const double L = sqrt(dadd(dadd(dmul(xx, xx), dmul(xy, xy)), dmul(xz, xz)));
-    if (p.grain[j] != gi || L >= p.Rc) {
+    double mag, L = 0.0;
+    const bool same = p.grain[j] == gi;
+    if (same) {
+        const double xx = xj.x - ox.x, xy = xj.y - ox.y, xz = xj.z - ox.z;
+        L = sqrt(dadd(dadd(dmul(xx, xx), dmul(xy, xy)), dmul(xz, xz)));
+    }
+    if (!same || L >= p.Rc) {
         mag = -p.Kn * (p.Rc - dn);
     } else {
         const double sr = (dn - L) / L;
@@ -695,7 +738,12 @@ __device__ __forceinline__ void contact_sum(const StepParams &p, int64_t row, bo
     dbl4 ox = dbl4{0.0, 0.0, 0.0, 0.0};
     double pix = 0.0, piy = 0.0, piz = 0.0;
     int gi = 0;
+    float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
     if (nch > 0) {
+        if (MIXED) {
+            o0 = __ldg(p.xh4 + RECX * row);
+            o1 = __ldg(p.uh_in + REC * row);
+        }
         ox = p.x4[row];
         const dbl4 ou = load_u_t<MIXED>(p, row);
         pix = dadd(ox.x, ou.x); piy = dadd(ox.y, ou.y); piz = dadd(ox.z, ou.z);
@@ -705,9 +753,16 @@ __device__ __forceinline__ void contact_sum(const StepParams &p, int64_t row, bo
     for (int t = 0; t < nmax; ++t) {
         const int64_t q = c0 + (int64_t)t * G + gl;
         double gx = 0.0, gy = 0.0, gz = 0.0;
-        if (q < c1 && !contact_term<MIXED>(p, q, ox, pix, piy, piz, gi, R2, gx, gy, gz)) gx = gy = gz = 0.0;
+        const bool touch = q < c1 && contact_term<MIXED>(p, q, o0, o1, ox, pix, piy, piz, gi, R2, gx, gy, gz);
+        if (!touch) gx = gy = gz = 0.0;
+        // in ascending order, passing over the places where no group of the warp touches
+        // (adding their zeros changes nothing)
+        unsigned m = __ballot_sync(0xffffffffu, touch);
 #pragma unroll
-        for (int l = 0; l < G; ++l) {
+        for (int o = 16; o >= G; o >>= 1) m |= m >> o;
+        m &= G == 32 ? 0xffffffffu : (1u << (G & 31)) - 1u;
+        for (; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
             cx += __shfl_sync(0xffffffffu, gx, l, G);
             cy += __shfl_sync(0xffffffffu, gy, l, G);
             cz += __shfl_sync(0xffffffffu, gz, l, G);
@@ -819,7 +874,7 @@ struct TileView {
 // Steps 1-4 for one row owned by a group of G lanes (all lanes call; inactive
 // groups pass active = false and still join the shuffles).
 template <int G, bool MIXED, bool WX = false, bool PAIRS = false>
-__device__ __forceinline__ void process_row(const StepParams &p, const double *wp, int64_t row, bool active, int gl,
+__device__ __forceinline__ void process_row(const StepParams &p, const double *wp, const WallF *wf, int64_t row, bool active, int gl,
                                             int lrow,
                                             const TileView &tv, double *react, unsigned &err, float &vmax2f,
                                             double &vmax2)
@@ -974,11 +1029,11 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
     // ---- 4. walls and Verlet update (group leader)
     if (MIXED) {
         float4 oxh = make_float4(0.f, 0.f, 0.f, 0.f), ouh = oxh, oul = oxh, ovh = oxh, ovl = oxh;
-        if (active && gl < 3) {
+        if (active && (gl < 3 || p.walls.nw)) {
             oxh = __ldg(p.xh4 + RECX * row); ouh = __ldg(p.uh_in + REC * row); oul = __ldg(p.ul_in + REC * row);
             ovh = p.vh[row]; ovl = p.vl[row];
         }
-        err |= epilogue_lanes<G, WX>(p, wp, row, active, gl, fbx, fby, fbz, oxh, ouh, oul, ovh, ovl, react, vmax2f);
+        err |= epilogue_lanes<G, WX>(p, wp, wf, row, active, gl, fbx, fby, fbz, oxh, ouh, oul, ovh, ovl, react, vmax2f);
     }
     if (!MIXED && active && gl == 0) {
         const double hdt = 0.5 * p.dt;
@@ -986,7 +1041,7 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
         const dbl4 ox = p.x4[row], ou = p.u_in[row];
         const dbl4 ov = p.v[row];
         if (p.walls.nw)
-            err |= wall_force<WX>(p, wp, dadd(ox.x, ou.x), dadd(ox.y, ou.y), dadd(ox.z, ou.z), ox.w, ov.x, ov.y, ov.z, Fx, Fy,
+            err |= wall_force<WX>(p, wp, (1u << p.walls.nw) - 1u, dadd(ox.x, ou.x), dadd(ox.y, ou.y), dadd(ox.z, ou.z), ox.w, ov.x, ov.y, ov.z, Fx, Fy,
                               Fz, react);
         if (!isfinite(Fx) || !isfinite(Fy) || !isfinite(Fz)) err |= PDE_NONFINITE;
         dbl4 a;
@@ -1100,6 +1155,8 @@ __global__ void __launch_bounds__(STEP_THREADS, MIXED ? PD_MINB_GLOBAL : 2) k_st
     if (gl == 0) {
         for (int q = 0; q < PD_MAX_WALLS * 3; ++q) s_react[grp][q] = 0.0;
     }
+    __shared__ WallF s_wf[PD_MAX_WALLS];
+    load_walls_f(p, p.wall_pos, s_wf);
     if (threadIdx.x == 0) {
         s_err = 0;
         if (blockIdx.x == 0 && p.contact && *p.stale) atomicOr(p.err, (unsigned)PDE_SKIN);
@@ -1112,7 +1169,7 @@ __global__ void __launch_bounds__(STEP_THREADS, MIXED ? PD_MINB_GLOBAL : 2) k_st
     const TileView tv{nullptr, nullptr, nullptr, false};
     for (int64_t r0 = (int64_t)blockIdx.x * GPB; r0 < p.n; r0 += (int64_t)gridDim.x * GPB) {
         const int64_t row = r0 + grp;
-        process_row<G, MIXED, WX, PAIRS>(p, p.wall_pos, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
+        process_row<G, MIXED, WX, PAIRS>(p, p.wall_pos, s_wf, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
     }
     if (gl == 0) s_vmax[grp] = MIXED ? (double)vmax2f : vmax2;
     block_finish<GPB>(p, s_react, s_vmax, s_err, s_last, err);
@@ -1209,6 +1266,8 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
     }
     if (gl == 0)
         for (int q = 0; q < PD_MAX_WALLS * 3; ++q) s_react[grp][q] = 0.0;
+    __shared__ WallF s_wf[PD_MAX_WALLS];
+    load_walls_f(p, s_wall, s_wf);
     if (threadIdx.x == 0) s_err = 0;
     __syncthreads();
     unsigned err = 0;
@@ -1217,7 +1276,7 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
     const TileView tv{nullptr, nullptr, nullptr, false};
     for (int64_t r0 = (int64_t)blockIdx.x * GPB; r0 < p.n; r0 += (int64_t)gridDim.x * GPB) {
         const int64_t row = r0 + grp;
-        process_row<G, MIXED, WX, false>(p, s_wall, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
+        process_row<G, MIXED, WX, false>(p, s_wall, s_wf, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
     }
     if (gl == 0) s_vmax[grp] = MIXED ? (double)vmax2f : vmax2;
     if (err) atomicOr(&s_err, err);
@@ -1335,6 +1394,8 @@ __global__ void __launch_bounds__(STEP_THREADS, PD_MINB_TILED) k_step_tiled(cons
     if (gl == 0) {
         for (int q = 0; q < PD_MAX_WALLS * 3; ++q) s_react[grp][q] = 0.0;
     }
+    __shared__ WallF s_wf[PD_MAX_WALLS];
+    load_walls_f(p, p.wall_pos, s_wf);
     if (threadIdx.x == 0) {
         s_err = 0;
         if (blockIdx.x == 0 && p.contact && *p.stale) atomicOr(p.err, (unsigned)PDE_SKIN);
@@ -1376,7 +1437,7 @@ __global__ void __launch_bounds__(STEP_THREADS, PD_MINB_TILED) k_step_tiled(cons
             const int64_t row = r0 + rr;
             const bool active = rr < rows;
             if (!on) {
-                process_row<G, true>(p, p.wall_pos, row, active, gl, 0, off, s_react[grp], err, vmax2f, vmax2);
+                process_row<G, true>(p, p.wall_pos, s_wf, row, active, gl, 0, off, s_react[grp], err, vmax2f, vmax2);
                 continue;
             }
             float fbx = 0.f, fby = 0.f, fbz = 0.f;
@@ -1414,7 +1475,7 @@ __global__ void __launch_bounds__(STEP_THREADS, PD_MINB_TILED) k_step_tiled(cons
             fby = group_sum<G>(fby) + (float)cy;
             fbz = group_sum<G>(fbz) + (float)cz;
             const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            err |= epilogue_lanes<G, false>(p, p.wall_pos, row, active, gl, fbx, fby, fbz, active ? o0 : z4, active ? o1 : z4,
+            err |= epilogue_lanes<G, false>(p, p.wall_pos, s_wf, row, active, gl, fbx, fby, fbz, active ? o0 : z4, active ? o1 : z4,
                                      active ? o2 : z4, active ? vhs[rr] : z4, active ? vls[rr] : z4, s_react[grp],
                                      vmax2f);
         }
