@@ -51,6 +51,7 @@ struct pd_ctx {
     int64_t *rowptr = nullptr, *crow = nullptr;
     int32_t *col = nullptr, *kc_of = nullptr;
     uint32_t *brk = nullptr;
+    double2 *blen = nullptr;  // FP64 path: per slot (|xi|, 1 / |xi|)
     int64_t nwords = 0;
 
     // contact candidates and grid
@@ -273,6 +274,7 @@ StepParams params(pd_ctx *c, int mode, int in, double dt)
         for (int a = 0; a < 3; ++a) p.bf[a] = (float)c->b[a];
         p.Rc_f = (float)c->mat.contact_radius;
     }
+    p.blen = c->blen;
     p.x4 = c->x4;
     p.u_in = c->u[in];
     p.u_out = c->u[in ^ 1];
@@ -854,6 +856,11 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     ALLOC(c->stage_bits, uint32_t, c->nwords);
     ALLOC(c->stage_b, uint8_t, B + 16);
     CK(cudaMemsetAsync(c->brk, 0, sizeof(uint32_t) * c->nwords, c->st));
+    release(c, c->blen);
+    if (c->opt.precision == PD_FP64) {
+        ALLOC(c->blen, double2, B + 1);
+        bond_lengths(c->x4, c->rowptr, c->col, n, c->blen, c->st);
+    }
     // mixed path: neighbour index with the broken flag in bit 31, one word per slot
     release(c, c->colf);
     if (c->opt.precision == PD_MIXED) {

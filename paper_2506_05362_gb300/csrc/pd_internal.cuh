@@ -81,6 +81,7 @@ struct StepParams {
     float4 *af;                    // a = (F + b)/rho, stored for the next drift
     float dt_hi, dt_lo, hdt_hi, hdt_lo, inv_rho_f, bf[3], Rc_f;
     // FP64 state
+    const double2 *blen;        // FP64 path: per slot (|xi|, 1 / |xi|), which never change
     const dbl4 *x4;             // (x, V)
     const dbl4 *u_in;           // u, current buffer
     dbl4 *u_out;                // u, next buffer

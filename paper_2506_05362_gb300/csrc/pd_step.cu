@@ -40,6 +40,31 @@ __device__ __forceinline__ int32_t ld_slot(const int32_t *a)
     return v;
 }
 
+// a slot's bond lengths on the FP64 path: streamed once per step, past L1
+__device__ __forceinline__ double2 ld_len(const double2 *a)
+{
+    double2 v;
+    asm("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(a));
+    return v;
+}
+
+// l = sqrt(a) and r = 1 / sqrt(a) from one approximate reciprocal root x0 (relative
+// error e0 below 2^-20): with e = 1 - a x0^2, 1 / sqrt(a) = x0 (1 - e)^(-1/2), and the
+// binomial series to second order leaves 5/16 e^3, below 2^-58; l = a r then takes one
+// Newton correction.  The FP64 bond loop is bound by the FP64 pipe (2 lanes a clock an
+// SM): with sqrt and two divisions, and the undeformed length computed again in every
+// step, a directed bond cost some 62 FP64 instructions, with this and the stored
+// lengths (16 bytes a slot) some 30.  Plate cut of 21,240 nodes: 654 -> 354 us a step.
+__device__ __forceinline__ void root64(double a, double &l, double &r)
+{
+    double x0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(a));
+    const double e = fma(-(a * x0), x0, 1.0);
+    r = fma(x0 * e, fma(0.375, e, 0.5), x0);
+    l = a * r;
+    l = fma(fma(-l, l, a), 0.5 * r, l);
+}
+
 constexpr int STEP_THREADS = 256;
 // bonds each lane keeps in flight per loop iteration, and the minimum resident
 // blocks per SM the compiler must allow (register budget)
@@ -986,21 +1011,24 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                 const uint32_t w = p.brk[k >> 5];
                 if ((w >> (k & 31)) & 1u) continue;
                 const int j = __ldg(p.col + k);
+                const double2 len = ld_len(p.blen + k);
                 const dbl4 a = p.x4[j], c = p.u_in[j];
-                const double xx = a.x - ox.x, xy = a.y - ox.y, xz = a.z - ox.z;
-                const double ex = c.x - ou.x, ey = c.y - ou.y, ez = c.z - ou.z;
-                const double yx = xx + ex, yy = xy + ey, yz = xz + ez;
-                const double L = sqrt(xx * xx + xy * xy + xz * xz);
-                const double l = sqrt(yx * yx + yy * yy + yz * yz);
-                const double s = (l - L) / L;
+                const double yx = (a.x - ox.x) + (c.x - ou.x), yy = (a.y - ox.y) + (c.y - ou.y),
+                             yz = (a.z - ox.z) + (c.z - ou.z);
+                const double l2 = fma(yx, yx, fma(yy, yy, yz * yz));
+                double l, rl;
+                root64(l2, l, rl);
+                const double s = (l - len.x) * len.y;
                 const bool brk = p.break_mode ? (fabs(s) > p.s0) : (s > p.s0);
                 if (brk) {
                     atomicOr(p.brk + (k >> 5), 1u << (k & 31));
                 } else {
-                    const double g = (p.conic ? p.c * (p.delta - L) : p.c) * s * a.w / l;
-                    fdx += g * yx; fdy += g * yy; fdz += g * yz;
+                    double g = s * rl * a.w;
+                    if (p.conic) g *= p.delta - len.x;
+                    fdx = fma(g, yx, fdx); fdy = fma(g, yy, fdy); fdz = fma(g, yz, fdz);
                 }
             }
+            fdx *= p.c; fdy *= p.c; fdz *= p.c;
         }
     }
     __syncwarp();
