@@ -55,16 +55,13 @@ struct pd_ctx {
     int64_t nwords = 0;
 
     // contact candidates and grid
-    int64_t *cand_ptr = nullptr, *cand_cnt = nullptr;
+    longlong2 *cand_rng = nullptr;
     int2 *cand = nullptr;
     int64_t cand_cap = 0;
     dbl4 *cand_fd = nullptr;  // pair damping + friction force per candidate (float4 view on the mixed path)
     double fric_dt = 0;       // time step the friction's stick branch sees (that of the latest pd_step)
     double *gl = nullptr;     // Gauss-Legendre table of the multi-wall overlap terms
-    uint32_t *gk = nullptr, *gk2 = nullptr, *gv = nullptr, *gv2 = nullptr, *gstart = nullptr, *gend = nullptr;
-    uint64_t *gcell = nullptr;
-    float4 *gpf = nullptr;  // FP32 positions of the grid's nodes (distance prefilter)
-    uint32_t nbuckets = 0;
+    GridBuf grid = {};
     int64_t *tmp = nullptr;  // scan / radix scratch for n-sized problems
 
     // reductions and device scalars
@@ -283,7 +280,7 @@ StepParams params(pd_ctx *c, int mode, int in, double dt)
     p.F_out = mode == MODE_FORCES ? c->F : nullptr;
     p.grain = c->grain;
     p.contact = c->opt.contact;
-    p.cand_ptr = c->cand_ptr;
+    p.cand_rng = c->cand_rng;
     p.cand = c->cand;
     p.c = c->c;
     p.s0 = c->s0;
@@ -352,22 +349,20 @@ const dbl4 *upos(pd_ctx *c, int in)
 // Contact candidate rebuild from u[in] (stream-ordered; capturable).
 void enqueue_rebuild(pd_ctx *c, int in)
 {
-    const dbl4 *u = upos(c, in);
+    const bool mixed = c->opt.precision == PD_MIXED;
     GridView g;
     for (int a = 0; a < 3; ++a) g.lo[a] = c->lo[a];
     const double cut = c->mat.contact_radius + skin_of(c);
-    grid_build(g, c->x4, u, c->n, cut * (1.0 + 1e-7), c->nbuckets, c->gk, c->gk2, c->gv, c->gv2, c->gstart,
-               c->gend, c->gcell, c->tmp, c->gpf, c->st);
-    cand_count(c->x4, u, c->grain, c->rowptr, c->col, c->n, g, cut, c->cand_cnt, c->st);
-    scan_exclusive_i64(c->cand_cnt, c->cand_ptr, c->n, c->tmp, c->st);
-    cand_fill(c->x4, u, c->grain, c->rowptr, c->col, c->n, g, cut, c->cand_ptr, c->cand, c->cand_cap,
-              c->derr, c->disp, c->stale, c->st);
+    grid_build(g, c->grid, c->x4, mixed ? nullptr : c->u[in], mixed ? c->uh[in] : nullptr, mixed ? c->ul[in] : nullptr,
+               REC, c->n, cut * (1.0 + 1e-7), c->st);
+    cand_build(c->grain, c->rowptr, c->col, c->n, g, c->grid, cut, c->cand_rng, c->cand, c->cand_cap, c->derr, c->disp,
+               c->stale, c->st);
 }
 
 pd_status grow_candidates(pd_ctx *c)
 {
     int64_t need = 0;
-    CK(cudaMemcpy(&need, c->cand_ptr + c->n, sizeof(int64_t), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(&need, c->grid.cand_cursor(), sizeof(int64_t), cudaMemcpyDeviceToHost));
     int64_t cap = std::max<int64_t>(2 * c->cand_cap, need + need / 2 + 1024);
     release(c, c->cand);
     ALLOC(c->cand, int2, cap);
@@ -564,18 +559,18 @@ static pd_status create_impl(pd_ctx *c, const double *x, const double *vol, cons
     // grid and contact buffers
     uint32_t nb = 1024;
     while ((int64_t)nb < 2 * n && nb < (1u << 26)) nb <<= 1;
-    c->nbuckets = nb;
-    ALLOC(c->gk, uint32_t, n);
-    ALLOC(c->gk2, uint32_t, n);
-    ALLOC(c->gv, uint32_t, n);
-    ALLOC(c->gv2, uint32_t, n);
-    ALLOC(c->gstart, uint32_t, nb);
-    ALLOC(c->gend, uint32_t, nb);
-    ALLOC(c->gcell, uint64_t, n);
-    ALLOC(c->gpf, float4, n);
-    ALLOC(c->cand_ptr, int64_t, n + 1);
-    ALLOC(c->cand_cnt, int64_t, n + 1);
-    CK(cudaMemsetAsync(c->cand_ptr, 0, sizeof(int64_t) * (n + 1), c->st));
+    c->grid.nbuckets = nb;
+    ALLOC(c->grid.count, uint32_t, nb + 4);
+    ALLOC(c->grid.range, uint2, nb);
+    ALLOC(c->grid.key, uint32_t, n);
+    ALLOC(c->grid.rank, uint32_t, n);
+    ALLOC(c->grid.node, uint32_t, n);
+    ALLOC(c->grid.cell, uint64_t, n);
+    ALLOC(c->grid.ecell, uint64_t, n);
+    ALLOC(c->grid.pf, float4, n);
+    ALLOC(c->grid.epf, float4, n);
+    ALLOC(c->cand_rng, longlong2, n);
+    CK(cudaMemsetAsync(c->cand_rng, 0, sizeof(longlong2) * n, c->st));
     c->cand_cap = c->opt.cand_capacity > 0 ? c->opt.cand_capacity : std::max<int64_t>(1024, 8 * n);
     ALLOC(c->cand, int2, c->cand_cap);
     if (c->mat.beta_d > 0 || c->mat.mu > 0) ALLOC(c->cand_fd, dbl4, c->cand_cap);  // damping + friction per candidate
@@ -746,8 +741,7 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     // grid over the reference positions, cell = horizon
     GridView g;
     for (int a = 0; a < 3; ++a) g.lo[a] = c->lo[a];
-    grid_build(g, c->x4, nullptr, n, horizon * (1.0 + 1e-7), c->nbuckets, c->gk, c->gk2, c->gv, c->gv2, c->gstart,
-               c->gend, c->gcell, c->tmp, c->gpf, c->st);
+    grid_build(g, c->grid, c->x4, nullptr, nullptr, nullptr, 0, n, horizon * (1.0 + 1e-7), c->st);
     int64_t *cnt;
     ALLOC(cnt, int64_t, n + 1);
     ALLOC(c->rowptr, int64_t, n + 1);
@@ -1007,7 +1001,7 @@ static int64_t enqueue_chunk(pd_ctx *c, int steps, int k, int parity, double dt,
     for (int s = 0; s < steps;) {
         if (c->opt.contact && s % k == 0 && !(skip0 && s == 0)) {
             enqueue_rebuild(c, in);
-            launches += 12;
+            launches += 4;
         }
         if (pgrid > 0) {
             // the steps up to the next rebuild, all MODE_FULL, in one launch; the
@@ -1524,7 +1518,7 @@ pd_status pd_contacts(pd_ctx *c, int64_t *npairs, int32_t *ij)
     int64_t *off = (int64_t *)pd_dev_alloc(c, sizeof(int64_t) * (n + 1));
     if (!cnt || !off) { pd_dev_free(c, cnt); pd_dev_free(c, off); return fail(c, PD_ENOMEM, "pd_contacts staging"); }
     const dbl4 *upc = upos(c, c->cur);
-    pairs_count(c->x4, upc, c->perm, c->brk, c->cand_ptr, c->cand, n, c->mat.contact_radius, cnt, c->st);
+    pairs_count(c->x4, upc, c->perm, c->brk, c->cand_rng, c->cand, n, c->mat.contact_radius, cnt, c->st);
     scan_exclusive_i64(cnt, off, n, c->tmp, c->st);
     int64_t total = 0;
     cudaMemcpyAsync(&total, off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c->st);
@@ -1537,7 +1531,7 @@ pd_status pd_contacts(pd_ctx *c, int64_t *npairs, int32_t *ij)
             if (!out) {
                 s = fail(c, PD_ENOMEM, "pd_contacts output");
             } else {
-                pairs_fill(c->x4, upc, c->perm, c->brk, c->cand_ptr, c->cand, n, c->mat.contact_radius, off,
+                pairs_fill(c->x4, upc, c->perm, c->brk, c->cand_rng, c->cand, n, c->mat.contact_radius, off,
                            out, c->st);
                 cudaMemcpyAsync(ij, out, sizeof(int32_t) * 2 * total, cudaMemcpyDeviceToHost, c->st);
                 s = sync(c);

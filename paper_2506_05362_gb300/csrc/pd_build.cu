@@ -78,32 +78,91 @@ __global__ void k_gather_nodes(const uint32_t *__restrict__ perm, int64_t n, con
 }
 
 // ---- grid --------------------------------------------------------------------
-__global__ void k_cell_keys(const dbl4 *__restrict__ x4, const dbl4 *__restrict__ u4, int64_t n, double lx,
-                            double ly, double lz, double cs, uint32_t mask, uint32_t *key, uint32_t *val,
-                            uint64_t *cell, float4 *pf)
+// Cell, FP32 position and bucket of every node; the bucket's counter gives the node's
+// place in it.
+__global__ void k_cell_keys(const dbl4 *__restrict__ x4, const dbl4 *__restrict__ u4, const float4 *__restrict__ hi,
+                            const float4 *__restrict__ lo, int stride, int64_t n, double lx, double ly, double lz,
+                            double inv, uint32_t mask, uint32_t *key, uint32_t *rank, uint32_t *count, uint64_t *cell,
+                            float4 *pf)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        dbl4 a = x4[i];
+        const dbl4 a = x4[i];
         double px = a.x, py = a.y, pz = a.z;
         if (u4) {
-            dbl4 u = u4[i];
+            const dbl4 u = u4[i];
             px = dadd(px, u.x); py = dadd(py, u.y); pz = dadd(pz, u.z);
+        } else if (hi) {
+            const float4 h = hi[stride * i], l = lo[stride * i];
+            px = dadd(px, df_to_double(df{h.x, l.x}));
+            py = dadd(py, df_to_double(df{h.y, l.y}));
+            pz = dadd(pz, df_to_double(df{h.z, l.z}));
         }
-        int cx = grid_coord(px, lx, cs), cy = grid_coord(py, ly, cs), cz = grid_coord(pz, lz, cs);
+        const int cx = grid_coord(px, lx, inv), cy = grid_coord(py, ly, inv), cz = grid_coord(pz, lz, inv);
         cell[i] = grid_pack(cx, cy, cz);
         const float fx = (float)dsub(px, lx), fy = (float)dsub(py, ly), fz = (float)dsub(pz, lz);
         pf[i] = make_float4(fx, fy, fz, fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz))));
-        key[i] = grid_hash(cx, cy, cz, mask);
-        val[i] = (uint32_t)i;
+        const uint32_t b = grid_hash(cx, cy, cz, mask);
+        key[i] = b;
+        rank[i] = atomicAdd(count + b, 1u);
     }
 }
 
-__global__ void k_bucket_ranges(const uint32_t *__restrict__ key, int64_t n, uint32_t *start, uint32_t *end)
+// sum over the threads of lower index in the block, and the block's total
+template <int THREADS>
+__device__ __forceinline__ unsigned block_prefix(unsigned v, unsigned &total)
 {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t b = key[e];
-        if (e == 0 || key[e - 1] != b) start[b] = (uint32_t)e;
-        if (e == n - 1 || key[e + 1] != b) end[b] = (uint32_t)(e + 1);
+    __shared__ unsigned ws[THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[warp] = x;
+    __syncthreads();
+    unsigned before = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) {
+        if (w < warp) before += ws[w];
+        total += ws[w];
+    }
+    __syncthreads();
+    return before + x - v;
+}
+
+// Entry ranges of the buckets: a block lays its 1024 buckets out one after another from
+// where the cursor stands (which block comes first does not matter).
+__global__ void __launch_bounds__(256) k_bucket_ranges(const uint32_t *__restrict__ count, uint32_t nbuckets,
+                                                       unsigned *cursor, uint2 *range)
+{
+    __shared__ unsigned s_base;
+    const uint32_t b = blockIdx.x * 1024 + threadIdx.x * 4;  // nbuckets is a multiple of 1024
+    const uint4 c = *(const uint4 *)(count + b);
+    unsigned total;
+    unsigned s = block_prefix<256>(c.x + c.y + c.z + c.w, total);
+    if (threadIdx.x == 0) s_base = atomicAdd(cursor, total);
+    __syncthreads();
+    s += s_base;
+    range[b] = make_uint2(s, s + c.x);
+    s += c.x;
+    range[b + 1] = make_uint2(s, s + c.y);
+    s += c.y;
+    range[b + 2] = make_uint2(s, s + c.z);
+    s += c.z;
+    range[b + 3] = make_uint2(s, s + c.w);
+}
+
+__global__ void k_bucket_fill(const uint32_t *__restrict__ key, const uint32_t *__restrict__ rank,
+                              const uint2 *__restrict__ range, const uint64_t *__restrict__ cell,
+                              const float4 *__restrict__ pf, int64_t n, uint32_t *node, uint64_t *ecell, float4 *epf)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t e = range[key[i]].x + rank[i];
+        node[e] = (uint32_t)i;
+        ecell[e] = cell[i];
+        epf[e] = pf[i];
     }
 }
 
@@ -157,15 +216,13 @@ __global__ void k_bonds(const dbl4 *__restrict__ x4, const int32_t *__restrict__
                 for (int dx = -1; dx <= 1; ++dx) {
                     const uint64_t want = grid_pack(cx + dx, cy + dy, cz + dz);
                     const uint32_t b = grid_hash(cx + dx, cy + dy, cz + dz, g.mask);
-                    const uint32_t s = g.start[b];
-                    if (s == 0xffffffffu) continue;
-                    const uint32_t e = g.end[b];
-                    for (uint32_t t = s; t < e; ++t) {
+                    const uint2 range = g.range[b];
+                    for (uint32_t t = range.x; t < range.y; ++t) {
                         const int32_t j = (int32_t)g.node[t];
-                        if (j == i || g.cell[j] != want || grain[j] != gi) continue;
+                        if (j == i || g.ecell[t] != want || grain[j] != gi) continue;
                         // FP32 decides pairs clearly inside or outside the horizon;
                         // the exact FP64 predicate decides the band between
-                        const float4 pj = g.pf[j];
+                        const float4 pj = g.epf[t];
                         const float d2f = pf_dist2(pi, pj), sl = pf_slack(deltaf, pi, pj);
                         const float hi = deltaf + sl, lo = deltaf - sl;
                         if (!(d2f < hi * hi)) continue;
@@ -205,68 +262,97 @@ __device__ __forceinline__ int64_t find_slot(const int64_t *rowptr, const int32_
     return (lo < rowptr[i + 1] && col[lo] == j) ? lo : -1;
 }
 
-template <bool FILL>
-__global__ void k_cand(const dbl4 *__restrict__ x4, const dbl4 *__restrict__ u4, const int32_t *__restrict__ grain,
-                       const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col, int64_t n, GridView g,
-                       double cut2, int64_t *cnt, const int64_t *__restrict__ off, int2 *cand, int64_t cap,
-                       unsigned *err, double *disp, int *stale)
+// Visits the nodes closer to node i than the search distance (a superset of them: the
+// step kernel applies the exact FP64 contact predicate).
+template <typename F>
+__device__ __forceinline__ void near_nodes(const GridView &g, int64_t i, float cutf, F f)
 {
-    if (FILL && blockIdx.x == 0 && threadIdx.x == 0) {
+    const float4 pi = g.pf[i];
+    const uint64_t pc = g.cell[i];
+    const int cx = (int)((pc >> 42) & 0x1fffff) - 1048576, cy = (int)((pc >> 21) & 0x1fffff) - 1048576,
+              cz = (int)(pc & 0x1fffff) - 1048576;
+    for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy) {
+            uint2 range[3];  // three cells' ranges in flight
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx)
+                range[dx] = __ldg(g.range + grid_hash(cx + dx - 1, cy + dy, cz + dz, g.mask));
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+                const uint64_t want = grid_pack(cx + dx - 1, cy + dy, cz + dz);
+                for (uint32_t t = range[dx].x; t < range[dx].y; ++t) {
+                    const uint64_t ce = __ldg(g.ecell + t);
+                    const float4 pj = __ldg(g.epf + t);
+                    if (ce != want) continue;
+                    const float lim = cutf + pf_slack(cutf, pi, pj);
+                    if (!(pf_dist2(pi, pj) < lim * lim)) continue;
+                    const int32_t j = (int32_t)__ldg(g.node + t);
+                    if (j != i) f(j);
+                }
+            }
+        }
+}
+
+// Contact candidates in one walk: a thread collects its node's candidates in ascending
+// partner order (so that the step kernels add contact terms in an order that does not
+// depend on the grid's), the block takes room for its rows from the cursor, and every
+// row's range goes to rng.  A row of more than CAND_LOCAL candidates is walked again.
+// (Counting, scanning and filling in separate passes walked the grid twice and took five
+// launches.  With the counting sort above in place of a three-pass radix sort a rebuild on
+// the 178,200-node plate is 4 launches and 78 us instead of 25 launches and 270 us, bound
+// by the latency of the 27 cells' scattered entries.)  Lists that outgrow cap set PDE_CAPACITY; the cursor holds the room needed.
+constexpr int CAND_LOCAL = 16;
+
+__global__ void __launch_bounds__(128) k_cand(const int32_t *__restrict__ grain, const int64_t *__restrict__ rowptr,
+                                              const int32_t *__restrict__ col, int64_t n, GridView g, float cutf,
+                                              longlong2 *rng, int2 *cand, int64_t cap, unsigned long long *cursor,
+                                              unsigned *err, double *disp, int *stale)
+{
+    __shared__ unsigned long long s_base;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         *disp = 0.0;
         *stale = 0;
-        if (off[n] > cap) atomicOr(err, (unsigned)PDE_CAPACITY);
     }
-    if (FILL && off[n] > cap) return;
-    const float cutf = (float)sqrt(cut2);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 pi = g.pf[i];
+    for (int64_t i0 = (int64_t)blockIdx.x * 128; i0 < n; i0 += (int64_t)gridDim.x * 128) {
+        const int64_t i = i0 + threadIdx.x;
+        int32_t hit[CAND_LOCAL];
+        unsigned k = 0;
+        if (i < n)
+            near_nodes(g, i, cutf, [&](int32_t j) {
+                if (k < CAND_LOCAL) {
+                    unsigned b = k;
+                    for (; b > 0 && hit[b - 1] > j; --b) hit[b] = hit[b - 1];
+                    hit[b] = j;
+                }
+                ++k;
+            });
+        unsigned total;
+        const unsigned before = block_prefix<128>(k, total);
+        if (threadIdx.x == 0) s_base = total ? atomicAdd(cursor, (unsigned long long)total) : 0ull;
+        __syncthreads();
+        const int64_t base = (int64_t)s_base;
+        __syncthreads();
+        const bool fits = base + total <= cap;  // uniform over the block
+        if (!fits && threadIdx.x == 0) atomicOr(err, (unsigned)PDE_CAPACITY);
+        if (i >= n) continue;
+        const int64_t c0 = base + before;
+        rng[i] = fits ? make_longlong2(c0, c0 + k) : make_longlong2(0, 0);
+        if (!fits) continue;
         const int gi = grain[i];
-        const uint64_t pc = g.cell[i];
-        const int cx = (int)((pc >> 42) & 0x1fffff) - 1048576, cy = (int)((pc >> 21) & 0x1fffff) - 1048576,
-                  cz = (int)(pc & 0x1fffff) - 1048576;
-        int64_t k = 0;
-        const int64_t base = FILL ? off[i] : 0;
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const uint64_t want = grid_pack(cx + dx, cy + dy, cz + dz);
-                    const uint32_t b = grid_hash(cx + dx, cy + dy, cz + dz, g.mask);
-                    const uint32_t s = g.start[b];
-                    if (s == 0xffffffffu) continue;
-                    const uint32_t e = g.end[b];
-                    for (uint32_t t = s; t < e; ++t) {
-                        const int32_t j = (int32_t)g.node[t];
-                        if (j == i || g.cell[j] != want) continue;
-                        // a superset of the pairs closer than cut: the step kernel
-                        // applies the exact FP64 contact predicate
-                        const float4 pj = g.pf[j];
-                        const float lim = cutf + pf_slack(cutf, pi, pj);
-                        if (!(pf_dist2(pi, pj) < lim * lim)) continue;
-                        if (FILL) {
-                            int2 c;
-                            c.x = j;
-                            c.y = (grain[j] == gi) ? (int)find_slot(rowptr, col, i, j) : -1;
-                            cand[base + k] = c;
-                        }
-                        ++k;
-                    }
-                }
-        if (!FILL) {
-            cnt[i] = k;
+        auto entry = [&](int32_t j) {
+            return make_int2(j, grain[j] == gi ? (int)find_slot(rowptr, col, i, j) : -1);
+        };
+        int2 *row = cand + c0;
+        if (k <= CAND_LOCAL) {
+            for (unsigned q = 0; q < k; ++q) row[q] = entry(hit[q]);
         } else {
-            // ascending partner index (insertion sort; rows hold few candidates), so
-            // that the step kernels add contact terms in an order that does not
-            // depend on the grid's bucket order
-            int2 *row = cand + base;
-            for (int64_t a = 1; a < k; ++a) {
-                const int2 c = row[a];
-                int64_t b = a - 1;
-                while (b >= 0 && row[b].x > c.x) {
-                    row[b + 1] = row[b];
-                    --b;
-                }
-                row[b + 1] = c;
-            }
+            unsigned m = 0;
+            near_nodes(g, i, cutf, [&](int32_t j) {
+                const int2 c = entry(j);
+                unsigned b = m++;
+                for (; b > 0 && row[b - 1].x > j; --b) row[b] = row[b - 1];
+                row[b] = c;
+            });
         }
     }
 }
@@ -274,14 +360,15 @@ __global__ void k_cand(const dbl4 *__restrict__ x4, const dbl4 *__restrict__ u4,
 // Exact contact pairs from the candidate lists at the current state (for output).
 template <bool FILL>
 __global__ void k_pairs(const dbl4 *__restrict__ x4, const dbl4 *__restrict__ u4, const int32_t *__restrict__ perm,
-                        const uint32_t *__restrict__ brk, const int64_t *__restrict__ cp, const int2 *__restrict__ cand,
-                        int64_t n, double R2, int64_t *cnt, const int64_t *__restrict__ off, int32_t *out)
+                        const uint32_t *__restrict__ brk, const longlong2 *__restrict__ cp,
+                        const int2 *__restrict__ cand, int64_t n, double R2, int64_t *cnt, const int64_t *__restrict__ off, int32_t *out)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const dbl4 a = x4[i], ua = u4[i];
         const double px = dadd(a.x, ua.x), py = dadd(a.y, ua.y), pz = dadd(a.z, ua.z);
         int64_t k = 0;
-        for (int64_t q = cp[i]; q < cp[i + 1]; ++q) {
+        const longlong2 rng = cp[i];
+        for (int64_t q = rng.x; q < rng.y; ++q) {
             const int2 c = cand[q];
             if (c.y >= 0 && !((brk[c.y >> 5] >> (c.y & 31)) & 1u)) continue;
             const dbl4 bj = x4[c.x], uj = u4[c.x];
@@ -692,26 +779,22 @@ void gather_nodes(const uint32_t *order, int64_t n, const double *x, const doubl
                                                centre[0], centre[1], centre[2]);
 }
 
-void grid_build(GridView &g, const dbl4 *x4, const dbl4 *u4, int64_t n, double cs, uint32_t nbuckets,
-                uint32_t *keys, uint32_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, uint32_t *start,
-                uint32_t *end, uint64_t *cell, int64_t *tmp, float4 *pf, cudaStream_t st)
+void grid_build(GridView &g, const GridBuf &w, const dbl4 *x4, const dbl4 *u4, const float4 *hi, const float4 *lo,
+                int stride, int64_t n, double cs, cudaStream_t st)
 {
-    g.cs = cs;
-    g.mask = nbuckets - 1;
-    k_cell_keys<<<grid_of(n), 256, 0, st>>>(x4, u4, n, g.lo[0], g.lo[1], g.lo[2], cs, g.mask, keys, vals, cell,
-                                            pf);
-    int bits = 0;
-    while ((1u << bits) < nbuckets) ++bits;
-    uint32_t *k = keys, *ka = keys_alt, *v = vals, *va = vals_alt;
-    radix_sort_u32(&k, &ka, &v, &va, n, ((bits + 7) / 8) * 8, tmp, st);
-    cudaMemsetAsync(start, 0xff, sizeof(uint32_t) * nbuckets, st);
-    cudaMemsetAsync(end, 0, sizeof(uint32_t) * nbuckets, st);
-    k_bucket_ranges<<<grid_of(n), 256, 0, st>>>(k, n, start, end);
-    g.start = start;
-    g.end = end;
-    g.node = v;
-    g.cell = cell;
-    g.pf = pf;
+    g.inv = 1.0 / cs;
+    g.mask = w.nbuckets - 1;
+    cudaMemsetAsync(w.count, 0, sizeof(uint32_t) * (w.nbuckets + 4), st);
+    k_cell_keys<<<grid_of(n), 256, 0, st>>>(x4, u4, hi, lo, stride, n, g.lo[0], g.lo[1], g.lo[2], g.inv, g.mask, w.key,
+                                            w.rank, w.count, w.cell, w.pf);
+    k_bucket_ranges<<<w.nbuckets / 1024, 256, 0, st>>>(w.count, w.nbuckets, w.bucket_cursor(), w.range);
+    k_bucket_fill<<<grid_of(n), 256, 0, st>>>(w.key, w.rank, w.range, w.cell, w.pf, n, w.node, w.ecell, w.epf);
+    g.range = w.range;
+    g.node = w.node;
+    g.ecell = w.ecell;
+    g.epf = w.epf;
+    g.cell = w.cell;
+    g.pf = w.pf;
 }
 
 void bonds_count(const dbl4 *x4, const int32_t *grain, const int32_t *perm, int64_t n, const GridView &g,
@@ -731,28 +814,21 @@ void bonds_keys_to_col(const uint64_t *keys, int64_t B, int sh, int32_t *col, cu
     k_keys_to_col<<<grid_of(B), 256, 0, st>>>(keys, B, (1ull << sh) - 1ull, col);
 }
 
-void cand_count(const dbl4 *x4, const dbl4 *u4, const int32_t *grain, const int64_t *rowptr, const int32_t *col,
-                int64_t n, const GridView &g, double cut, int64_t *cnt, cudaStream_t st)
+void cand_build(const int32_t *grain, const int64_t *rowptr, const int32_t *col, int64_t n, const GridView &g,
+                const GridBuf &w, double cut, longlong2 *rng, int2 *cand, int64_t cap, unsigned *err, double *disp,
+                int *stale, cudaStream_t st)
 {
-    k_cand<false><<<grid_of(n, 128), 128, 0, st>>>(x4, u4, grain, rowptr, col, n, g, cut * cut, cnt, nullptr,
-                                                   nullptr, 0, nullptr, nullptr, nullptr);
+    k_cand<<<grid_of(n, 128), 128, 0, st>>>(grain, rowptr, col, n, g, (float)cut, rng, cand, cap, w.cand_cursor(), err,
+                                            disp, stale);
 }
 
-void cand_fill(const dbl4 *x4, const dbl4 *u4, const int32_t *grain, const int64_t *rowptr, const int32_t *col,
-               int64_t n, const GridView &g, double cut, const int64_t *off, int2 *cand, int64_t cap, unsigned *err,
-               double *disp, int *stale, cudaStream_t st)
-{
-    k_cand<true><<<grid_of(n, 128), 128, 0, st>>>(x4, u4, grain, rowptr, col, n, g, cut * cut, nullptr, off, cand,
-                                                  cap, err, disp, stale);
-}
-
-void pairs_count(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const int64_t *cp,
+void pairs_count(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const longlong2 *cp,
                  const int2 *cand, int64_t n, double Rc, int64_t *cnt, cudaStream_t st)
 {
     k_pairs<false><<<grid_of(n), 256, 0, st>>>(x4, u4, perm, brk, cp, cand, n, Rc * Rc, cnt, nullptr, nullptr);
 }
 
-void pairs_fill(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const int64_t *cp,
+void pairs_fill(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const longlong2 *cp,
                 const int2 *cand, int64_t n, double Rc, const int64_t *off, int32_t *out, cudaStream_t st)
 {
     k_pairs<true><<<grid_of(n), 256, 0, st>>>(x4, u4, perm, brk, cp, cand, n, Rc * Rc, nullptr, off, out);

@@ -23,14 +23,13 @@ void bonds_count(const dbl4 *x4, const int32_t *grain, const int32_t *perm, int6
 void bonds_fill(const dbl4 *x4, const int32_t *grain, const int32_t *perm, int64_t n, const GridView &g,
                 double delta, const FilterSet &f, const int64_t *off, uint64_t *keys, int sh, cudaStream_t st);
 void bonds_keys_to_col(const uint64_t *keys, int64_t B, int sh, int32_t *col, cudaStream_t st);
-void cand_count(const dbl4 *x4, const dbl4 *u4, const int32_t *grain, const int64_t *rowptr, const int32_t *col,
-                int64_t n, const GridView &g, double cut, int64_t *cnt, cudaStream_t st);
-void cand_fill(const dbl4 *x4, const dbl4 *u4, const int32_t *grain, const int64_t *rowptr, const int32_t *col,
-               int64_t n, const GridView &g, double cut, const int64_t *off, int2 *cand, int64_t cap, unsigned *err,
-               double *disp, int *stale, cudaStream_t st);
-void pairs_count(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const int64_t *cp,
+// contact candidates closer than cut: per row the range rng in cand
+void cand_build(const int32_t *grain, const int64_t *rowptr, const int32_t *col, int64_t n, const GridView &g,
+                const GridBuf &w, double cut, longlong2 *rng, int2 *cand, int64_t cap, unsigned *err, double *disp,
+                int *stale, cudaStream_t st);
+void pairs_count(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const longlong2 *cp,
                  const int2 *cand, int64_t n, double Rc, int64_t *cnt, cudaStream_t st);
-void pairs_fill(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const int64_t *cp,
+void pairs_fill(const dbl4 *x4, const dbl4 *u4, const int32_t *perm, const uint32_t *brk, const longlong2 *cp,
                 const int2 *cand, int64_t n, double Rc, const int64_t *off, int32_t *out, cudaStream_t st);
 void damage(const int64_t *rowptr, const uint32_t *brk, const int32_t *perm, int64_t n, double *phi,
             cudaStream_t st);

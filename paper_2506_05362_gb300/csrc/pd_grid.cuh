@@ -1,24 +1,39 @@
 // Uniform hashed cell grid shared by the bond builder and the contact search.
 //
 // A node at p falls in the integer cell c = floor((p - lo) / cs) (FP64), clamped
-// to +-2^20 cells per axis.  Cells hash into a power-of-two bucket table; nodes
-// are radix-sorted by bucket (stable, so each bucket lists its nodes in
-// ascending index order) and a query walks the 27 cells around a node, keeping
-// only nodes whose own cell is the visited cell.  The exact distance predicate
-// is applied by the caller, so hashing and clamping never change a result.
+// to +-2^20 cells per axis.  Cells hash into a power-of-two bucket table; the nodes are
+// counted into the buckets (a counting sort whose order inside a bucket and of the
+// buckets is arbitrary) with copies of their cells and FP32 positions, and a query walks
+// the 27 cells around a node, keeping only nodes whose own cell is the visited cell.
+// The exact distance predicate is applied by the caller, who also orders what it finds,
+// so hashing, clamping and the order never change a result.
 #pragma once
 
 #include "pd_internal.cuh"
 
 struct GridView {
     double lo[3];
-    double cs;                    // cell size
+    double inv;                   // 1 / cell size
     uint32_t mask;                // bucket table size - 1
-    const uint32_t *start;        // bucket -> first sorted entry (0xffffffff = empty)
-    const uint32_t *end;          // bucket -> one past last
-    const uint32_t *node;         // sorted entries -> node index
+    const uint2 *range;           // bucket -> first entry, one past last
+    const uint32_t *node;         // entry -> node index
+    const uint64_t *ecell;        // entry -> packed cell coordinates
+    const float4 *epf;            // entry -> FP32 position (as pf)
     const uint64_t *cell;         // node -> packed cell coordinates
     const float4 *pf;             // node -> FP32 (p - lo), .w = max |component| (prefilter)
+};
+
+// Device buffers of the grid: n entries or nodes each, nbuckets counts and ranges.  The
+// two cursors follow the counts, so that one memset clears them all.
+struct GridBuf {
+    uint32_t nbuckets;
+    uint32_t *count;              // nbuckets + 4 words
+    uint2 *range;
+    uint32_t *key, *rank, *node;
+    uint64_t *cell, *ecell;
+    float4 *pf, *epf;
+    unsigned *bucket_cursor() const { return count + nbuckets; }
+    unsigned long long *cand_cursor() const { return (unsigned long long *)(count + nbuckets + 2); }
 };
 
 // Conservative FP32 distance test.  pf = fl32(p - lo) carries an error of at
@@ -35,11 +50,11 @@ __device__ __forceinline__ float pf_dist2(const float4 &a, const float4 &b)
     return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
 }
 
-__device__ __forceinline__ int grid_coord(double p, double lo, double cs)
+// (p - lo) / cs rounds to within 2^-31 of a cell over the clamped range, far below the
+// 1e-7 by which every cell is wider than its search distance
+__device__ __forceinline__ int grid_coord(double p, double lo, double inv)
 {
-    double q = floor(__ddiv_rn(__dsub_rn(p, lo), cs));
-    q = fmin(fmax(q, -1048576.0), 1048575.0);
-    return (int)q;
+    return min(max(__double2int_rd(__dmul_rn(__dsub_rn(p, lo), inv)), -1048576), 1048575);
 }
 
 __device__ __forceinline__ uint64_t grid_pack(int cx, int cy, int cz)
@@ -54,7 +69,7 @@ __device__ __forceinline__ uint32_t grid_hash(int cx, int cy, int cz, uint32_t m
     return (((uint32_t)cx * 73856093u) ^ ((uint32_t)cy * 19349663u) ^ ((uint32_t)cz * 83492791u)) & mask;
 }
 
-// Build step kernels (pd_grid.cu).
-void grid_build(GridView &g, const dbl4 *x4, const dbl4 *u4, int64_t n, double cs, uint32_t nbuckets,
-                uint32_t *keys, uint32_t *keys_alt, uint32_t *vals, uint32_t *vals_alt, uint32_t *start,
-                uint32_t *end, uint64_t *cell, int64_t *tmp, float4 *pf, cudaStream_t st);
+// Buckets the nodes at x4 + u: u as FP64 (u4), as double-float pairs (hi, lo, element
+// stride `stride`), or none.  Clears both cursors.
+void grid_build(GridView &g, const GridBuf &w, const dbl4 *x4, const dbl4 *u4, const float4 *hi, const float4 *lo,
+                int stride, int64_t n, double cs, cudaStream_t st);

@@ -89,9 +89,9 @@ struct StepParams {
     dbl4 *acc;                  // acceleration (F + b)/rho, stored
     dbl4 *F_out;                // force density (MODE_FORCES), may be null
     const int32_t *grain;
-    // contact candidates (CSR; each entry = (j, bond slot or -1))
+    // contact candidates (each entry = (j, bond slot or -1))
     int contact;
-    const int64_t *cand_ptr;
+    const longlong2 *cand_rng;     // per row: first entry, one past last
     const int2 *cand;
     // constants
     double c, s0, Kn, Rc, rho, dt;

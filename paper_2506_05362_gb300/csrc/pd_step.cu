@@ -754,8 +754,9 @@ __device__ __forceinline__ void contact_sum(const StepParams &p, int64_t row, bo
     cx = cy = cz = 0.0;
     int64_t c0 = 0, c1 = 0;
     if (active && p.contact) {
-        c0 = p.cand_ptr[row];
-        c1 = p.cand_ptr[row + 1];
+        const longlong2 r = p.cand_rng[row];
+        c0 = r.x;
+        c1 = r.y;
     }
     const int nch = (int)((c1 - c0 + G - 1) / G);
     const int nmax = __reduce_max_sync(0xffffffffu, nch);  // warp-uniform trip count
@@ -825,7 +826,8 @@ __device__ __forceinline__ void pair_damping_rows(const StepParams &p, int64_t f
 {
     const double R2 = dmul(p.Rc, p.Rc);
     for (int64_t i = first; i < p.n; i += stride) {
-        const int64_t c0 = p.cand_ptr[i], c1 = p.cand_ptr[i + 1];
+        const longlong2 rng = p.cand_rng[i];
+        const int64_t c0 = rng.x, c1 = rng.y;
         if (c1 <= c0) continue;
         const dbl4 ox = p.x4[i], ou = load_u_t<MIXED>(p, i);
         const double pix = dadd(ox.x, ou.x), piy = dadd(ox.y, ou.y), piz = dadd(ox.z, ou.z);
