@@ -743,9 +743,11 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     for (int a = 0; a < 3; ++a) g.lo[a] = c->lo[a];
     grid_build(g, c->grid, c->x4, nullptr, nullptr, nullptr, 0, n, horizon * (1.0 + 1e-7), c->st);
     int64_t *cnt;
+    uint16_t *sides;
     ALLOC(cnt, int64_t, n + 1);
+    ALLOC(sides, uint16_t, n);
     ALLOC(c->rowptr, int64_t, n + 1);
-    bonds_count(c->x4, c->grain, c->perm, n, g, horizon, f, cnt, c->st);
+    bonds_count(c->x4, c->grain, c->perm, n, g, horizon, f, sides, cnt, c->st);
     scan_exclusive_i64(cnt, c->rowptr, n, c->tmp, c->st);
     int64_t B = 0;
     CK(cudaMemcpyAsync(&B, c->rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c->st));
@@ -753,33 +755,16 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     if (s) return s;
     if (B > 0x7fffffffLL) return fail(c, PD_ECAPACITY, "more than 2^31-1 directed bonds");
     c->B = B;
-    uint64_t *k1, *k2;
-    uint32_t *v1, *v2;
-    int64_t *btmp;
-    ALLOC(k1, uint64_t, B + 1);
-    ALLOC(k2, uint64_t, B + 1);
-    ALLOC(v1, uint32_t, B + 1);
-    ALLOC(v2, uint32_t, B + 1);
-    ALLOC(btmp, int64_t, std::max(radix_tmp_size(B + 1), scan_tmp_size(n + 1) + 8));
+    // canonical numbering (caller rows, ascending caller columns), rows in ascending order
+    int32_t *found;
+    ALLOC(found, int32_t, B + 1);
     ALLOC(c->col, int32_t, B + 1);
-    bonds_fill(c->x4, c->grain, c->perm, n, g, horizon, f, c->rowptr, k1, c->sh, c->st);
-    {
-        uint64_t *k = k1, *ka = k2;
-        radix_sort_u64(&k, &ka, nullptr, nullptr, B, 2 * c->sh, btmp, c->st);
-        bonds_keys_to_col(k, B, c->sh, c->col, c->st);
-    }
-    // canonical numbering (caller rows, ascending caller columns)
     ALLOC(c->kc_of, int32_t, B + 1);
     ALLOC(c->crow, int64_t, n + 1);
-    {
-        canon_keys(c->rowptr, c->col, c->perm, n, c->sh, k1, v1, c->st);
-        uint64_t *k = k1, *ka = k2;
-        uint32_t *v = v1, *va = v2;
-        radix_sort_u64(&k, &ka, &v, &va, B, 2 * c->sh, btmp, c->st);
-        canon_invert(v, B, c->kc_of, c->st);
-        row_len_caller(c->rowptr, c->inv, n, cnt, c->st);
-        scan_exclusive_i64(cnt, c->crow, n, c->tmp, c->st);
-    }
+    bonds_fill(c->x4, c->grain, c->perm, n, g, horizon, f, sides, c->rowptr, found, c->st);
+    row_len_caller(c->rowptr, c->inv, n, cnt, c->st);
+    scan_exclusive_i64(cnt, c->crow, n, c->tmp, c->st);
+    order_rows(found, c->rowptr, c->perm, c->crow, n, c->col, c->kc_of, c->st);
     // shared-memory tiles (mixed path): the largest tile (64, 32 or 16 rows) whose
     // staging fits two blocks per SM.  A material with friction or multi-wall terms
     // runs the global-gather kernels that carry the wall extras, so it has no tiles.
@@ -881,7 +866,7 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     CK(cudaGetLastError());
     s = sync(c);
     if (s) return s;
-    release(c, k1); release(c, k2); release(c, v1); release(c, v2); release(c, btmp); release(c, cnt);
+    release(c, found); release(c, cnt); release(c, sides);
     c->bonds_ready = true;
     c->list_ok = false;
     // several steps per launch: on request, or by default for problems small enough

@@ -167,87 +167,203 @@ __global__ void k_bucket_fill(const uint32_t *__restrict__ key, const uint32_t *
 }
 
 // ---- bonds -------------------------------------------------------------------
-// Filter test with the endpoints in canonical order (smaller caller index first).
-__device__ bool filter_drops(const double *x1, const double *x2, const FilterSet &f)
+// What the filters say of a node alone, two bits a filter.  Inner sphere: both bits
+// when the node is not strictly inside, so a bond is kept when its ends share a bit.
+// Notch: the side of the plane (bit 0 above, bit 1 below) when the node is clearly off it:
+// a bond whose ends share a bit does not cross the plane, whatever the rounding of the
+// exact test (the margin is 10^6 times the error of the plane's FP64 value); a bond whose
+// ends share none is tested by notch_drops.  Decided per bond, the spheres alone took
+// four fifths of the bond search's time (FP64 on a few lanes of every warp).
+__global__ void k_filter_sides(const dbl4 *__restrict__ x4, int64_t n, FilterSet f, uint16_t *sides)
 {
-    for (int q = 0; q < f.nf; ++q) {
-        const double *p = f.a[q];
-        if (f.kind[q] == 1) {
-            double dx = dsub(x2[0], x1[0]), dy = dsub(x2[1], x1[1]), dz = dsub(x2[2], x1[2]);
-            double num = dadd(dadd(dadd(dmul(p[0], x1[0]), dmul(p[1], x1[1])), dmul(p[2], x1[2])), p[3]);
-            double den = dadd(dadd(dmul(p[0], dx), dmul(p[1], dy)), dmul(p[2], dz));
-            if (den != 0.0) {
-                double t = __ddiv_rn(-num, den);
-                if (t > 0.0 && t < 1.0) {
-                    double r0 = dadd(x1[0], dmul(t, dx)), r1 = dadd(x1[1], dmul(t, dy)), r2 = dadd(x1[2], dmul(t, dz));
-                    if (r0 >= p[4] && r0 <= p[7] && r1 >= p[5] && r1 <= p[8] && r2 >= p[6] && r2 <= p[9]) return true;
-                }
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const dbl4 x = x4[i];
+        unsigned m = 0;
+        for (int q = 0; q < f.nf; ++q) {
+            const double *p = f.a[q];
+            if (f.kind[q] == 1) {
+                const double a = p[0] * x.x, b = p[1] * x.y, c = p[2] * x.z;
+                const double v = ((a + b) + c) + p[3], tol = 1e-9 * (((fabs(a) + fabs(b)) + fabs(c)) + fabs(p[3]));
+                if (v > tol) m |= 1u << (2 * q);
+                if (v < -tol) m |= 2u << (2 * q);
+            } else {
+                const double d = sq3(dsub(x.x, p[0]), dsub(x.y, p[1]), dsub(x.z, p[2]));
+                if (!(d < dmul(p[3], p[3]))) m |= 3u << (2 * q);
             }
-        } else if (f.kind[q] == 2) {
-            double R2 = dmul(p[3], p[3]);
-            double d1 = sq3(dsub(x1[0], p[0]), dsub(x1[1], p[1]), dsub(x1[2], p[2]));
-            double d2 = sq3(dsub(x2[0], p[0]), dsub(x2[1], p[1]), dsub(x2[2], p[2]));
-            if (d1 < R2 || d2 < R2) return true;
         }
+        sides[i] = (uint16_t)m;
+    }
+}
+
+// Notch test of one bond with the endpoints in canonical order (smaller caller index first).
+__device__ bool notch_drops(const double *x1, const double *x2, const double *p)
+{
+    double dx = dsub(x2[0], x1[0]), dy = dsub(x2[1], x1[1]), dz = dsub(x2[2], x1[2]);
+    double num = dadd(dadd(dadd(dmul(p[0], x1[0]), dmul(p[1], x1[1])), dmul(p[2], x1[2])), p[3]);
+    double den = dadd(dadd(dmul(p[0], dx), dmul(p[1], dy)), dmul(p[2], dz));
+    if (den == 0.0) return false;
+    double t = __ddiv_rn(-num, den);
+    if (!(t > 0.0 && t < 1.0)) return false;
+    double r0 = dadd(x1[0], dmul(t, dx)), r1 = dadd(x1[1], dmul(t, dy)), r2 = dadd(x1[2], dmul(t, dz));
+    return r0 >= p[4] && r0 <= p[7] && r1 >= p[5] && r1 <= p[8] && r2 >= p[6] && r2 <= p[9];
+}
+
+// Whether a filter drops the bond between nodes i and j of sides si and sj.
+__device__ __forceinline__ bool filters_drop(const FilterSet &f, unsigned si, unsigned sj, const dbl4 *x4,
+                                             const int32_t *perm, int64_t i, int32_t j)
+{
+    const unsigned m = si & sj;
+    unsigned open = ~(m | (m >> 1)) & 0x5555u & ((1u << (2 * f.nf)) - 1u);  // filters whose ends share no bit
+    for (; open; open &= open - 1) {
+        const int q = (__ffs(open) - 1) >> 1;
+        if (f.kind[q] == 2) return true;
+        const dbl4 a = x4[i], b = x4[j];
+        const double pa[3] = {a.x, a.y, a.z}, pb[3] = {b.x, b.y, b.z};
+        if (perm[i] < perm[j] ? notch_drops(pa, pb, f.a[q]) : notch_drops(pb, pa, f.a[q])) return true;
     }
     return false;
 }
 
-// Visits the bond partners of node i; FILL = false counts them, FILL = true
-// writes keys (row << sh) | j.
+// The exact horizon test.  Out of line: inlined, its FP64 arithmetic is executed for
+// every candidate with the result discarded (980 us instead of 270).
+__device__ __noinline__ bool within64(const dbl4 *x4, int64_t i, int32_t j, double d2max)
+{
+    const dbl4 a = x4[i], b = x4[j];
+    return sq3(dsub(b.x, a.x), dsub(b.y, a.y), dsub(b.z, a.z)) < d2max;
+}
+
+// The bond partners of node i, found by a warp: each of the 27 cells' entries is read by
+// consecutive lanes (a cell one horizon wide holds some 27 lattice nodes).  FILL = false
+// counts them; FILL = true writes them in the order they are found (k_order_rows sorts
+// the rows).  A thread a node, walking all 700 entries by itself, took 2.4 ms for the
+// 74,290 nodes of a hollow sphere (2,300 warps), this 0.27 (and 0.35 to fill).
 template <bool FILL>
-__global__ void k_bonds(const dbl4 *__restrict__ x4, const int32_t *__restrict__ grain,
-                        const int32_t *__restrict__ perm, int64_t n, GridView g, double delta2, FilterSet f,
-                        int64_t *cnt, const int64_t *__restrict__ off, uint64_t *keys, int sh)
+__global__ void __launch_bounds__(256) k_bonds(const dbl4 *__restrict__ x4, const int32_t *__restrict__ grain,
+                                               const int32_t *__restrict__ perm, int64_t n, GridView g, double delta2,
+                                               FilterSet f, const uint16_t *__restrict__ sides, int64_t *cnt,
+                                               const int64_t *__restrict__ off, int32_t *found)
 {
     const float deltaf = (float)sqrt(delta2);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const dbl4 a = x4[i];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nwarps) {
         const float4 pi = g.pf[i];
         const int gi = grain[i];
-        const int32_t ci = perm[i];
+        const unsigned si = f.nf ? sides[i] : 0u;
         const uint64_t pc = g.cell[i];
         const int cx = (int)((pc >> 42) & 0x1fffff) - 1048576, cy = (int)((pc >> 21) & 0x1fffff) - 1048576,
                   cz = (int)(pc & 0x1fffff) - 1048576;
-        int64_t k = 0;
-        int64_t base = FILL ? off[i] : 0;
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const uint64_t want = grid_pack(cx + dx, cy + dy, cz + dz);
-                    const uint32_t b = grid_hash(cx + dx, cy + dy, cz + dz, g.mask);
-                    const uint2 range = g.range[b];
-                    for (uint32_t t = range.x; t < range.y; ++t) {
-                        const int32_t j = (int32_t)g.node[t];
-                        if (j == i || g.ecell[t] != want || grain[j] != gi) continue;
-                        // FP32 decides pairs clearly inside or outside the horizon;
-                        // the exact FP64 predicate decides the band between
-                        const float4 pj = g.epf[t];
-                        const float d2f = pf_dist2(pi, pj), sl = pf_slack(deltaf, pi, pj);
-                        const float hi = deltaf + sl, lo = deltaf - sl;
-                        if (!(d2f < hi * hi)) continue;
-                        const dbl4 bj = x4[j];
-                        if (!(d2f < lo * lo)) {
-                            const double r2 = sq3(dsub(bj.x, a.x), dsub(bj.y, a.y), dsub(bj.z, a.z));
-                            if (!(r2 < delta2)) continue;
-                        }
-                        if (f.nf) {
-                            const double pa[3] = {a.x, a.y, a.z}, pb[3] = {bj.x, bj.y, bj.z};
-                            const bool drop = (ci < perm[j]) ? filter_drops(pa, pb, f) : filter_drops(pb, pa, f);
-                            if (drop) continue;
-                        }
-                        if (FILL) keys[base + k] = ((uint64_t)i << sh) | (uint64_t)j;
-                        ++k;
-                    }
+        uint2 range = make_uint2(0u, 0u);  // lane c holds the entries of cell c
+        uint64_t want = 0;
+        if (lane < 27) {
+            const int x = cx + lane % 3 - 1, y = cy + lane / 3 % 3 - 1, z = cz + lane / 9 - 1;
+            range = __ldg(g.range + grid_hash(x, y, z, g.mask));
+            want = grid_pack(x, y, z);
+        }
+        int64_t k = FILL ? off[i] : 0;
+        for (int c = 0; c < 27; ++c) {
+            const uint32_t e = __shfl_sync(0xffffffffu, range.y, c);
+            const uint64_t w = __shfl_sync(0xffffffffu, want, c);
+            for (uint32_t t0 = __shfl_sync(0xffffffffu, range.x, c); t0 < e; t0 += 32) {
+                const uint32_t t = t0 + lane;
+                bool ok = false;
+                int32_t j = 0;
+                if (t < e && __ldg(g.ecell + t) == w) {
+                    // FP32 decides pairs clearly inside or outside the horizon; the exact
+                    // FP64 predicate decides the band between
+                    const float4 pj = __ldg(g.epf + t);
+                    const float d2f = pf_dist2(pi, pj), sl = pf_slack(deltaf, pi, pj);
+                    const float hi = deltaf + sl, lo = deltaf - sl;
+                    j = (int32_t)__ldg(g.node + t);
+                    ok = d2f < hi * hi && j != i && grain[j] == gi;
+                    if (ok && !(d2f < lo * lo)) ok = within64(x4, i, j, delta2);
+                    if (ok && f.nf) ok = !filters_drop(f, si, sides[j], x4, perm, i, j);
                 }
-        if (!FILL) cnt[i] = k;
+                const unsigned m = __ballot_sync(0xffffffffu, ok);
+                if (FILL && ok) found[k + __popc(m & lt)] = j;
+                k += __popc(m);
+            }
+        }
+        if (!FILL && lane == 0) cnt[i] = k;
     }
 }
 
-__global__ void k_keys_to_col(const uint64_t *__restrict__ keys, int64_t B, uint64_t mask, int32_t *col)
+// Rows into ascending order, and the canonical (caller-order) slot of every bond, by
+// counting: a warp takes a row, and an element's place is the number of elements below
+// it, its canonical place the number whose caller index is below its own.  Rows of up to
+// ORDER_ROW elements are staged in shared memory, longer ones read where they are.  Two
+// radix sorts of all B bonds by 64-bit keys did this before, in 14 passes over 24 bytes
+// a bond.
+constexpr int ORDER_ROW = 512, ORDER_WARPS = 8;
+
+// places of the elements q0 + 32 u + lane, u < U, of a row (row: staged, or null)
+template <int U, typename E>
+__device__ __forceinline__ void place(E element, const int2 *row, int q0, int len, int lane, int64_t k0, int64_t c0,
+                                      int32_t *col, int32_t *kc_of)
 {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < B; k += (int64_t)gridDim.x * blockDim.x)
-        col[k] = (int32_t)(keys[k] & mask);
+    int2 e[U];
+    int a[U], c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int q = q0 + 32 * u + lane;
+        e[u] = q < len ? element(q) : make_int2(-1, -1);
+        a[u] = c[u] = 0;
+    }
+    auto count = [&](int2 r) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            a[u] += r.x < e[u].x;
+            c[u] += r.y < e[u].y;
+        }
+    };
+    if (row) {
+#pragma unroll 4
+        for (int q = 0; q < len; ++q) count(row[q]);
+    } else {
+        for (int q = 0; q < len; ++q) count(element(q));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (q0 + 32 * u + lane < len) {
+            col[k0 + a[u]] = e[u].x;
+            kc_of[k0 + a[u]] = (int32_t)(c0 + c[u]);
+        }
+}
+
+__global__ void __launch_bounds__(32 * ORDER_WARPS) k_order_rows(const int32_t *__restrict__ found,
+                                                                 const int64_t *__restrict__ rowptr,
+                                                                 const int32_t *__restrict__ perm,
+                                                                 const int64_t *__restrict__ crow, int64_t n,
+                                                                 int32_t *col, int32_t *kc_of)
+{
+    __shared__ int2 s_row[ORDER_WARPS][ORDER_ROW];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int2 *row = s_row[warp];
+    const int64_t nwarps = (int64_t)gridDim.x * ORDER_WARPS;
+    for (int64_t i = (int64_t)blockIdx.x * ORDER_WARPS + warp; i < n; i += nwarps) {
+        const int64_t k0 = rowptr[i];
+        const int len = (int)(rowptr[i + 1] - k0);
+        const int64_t c0 = crow[perm[i]];
+        const bool staged = len <= ORDER_ROW;
+        if (staged) {
+            for (int q = lane; q < len; q += 32) {
+                const int32_t j = found[k0 + q];
+                row[q] = make_int2(j, perm[j]);
+            }
+            __syncwarp();
+        }
+        auto element = [&](int q) {
+            if (staged) return row[q];
+            const int32_t j = found[k0 + q];
+            return make_int2(j, perm[j]);
+        };
+        int q0 = 0;
+        for (; len - q0 > 64; q0 += 128) place<4>(element, staged ? row : nullptr, q0, len, lane, k0, c0, col, kc_of);
+        if (len - q0 > 32) place<2>(element, staged ? row : nullptr, q0, len, lane, k0, c0, col, kc_of);
+        else if (len > q0) place<1>(element, staged ? row : nullptr, q0, len, lane, k0, c0, col, kc_of);
+        __syncwarp();
+    }
 }
 
 // ---- contact candidates ---------------------------------------------------------
@@ -425,25 +541,6 @@ __global__ void k_stable_dt(const dbl4 *__restrict__ x4, const int64_t *__restri
 }
 
 // ---- canonical (caller-order) bond numbering ------------------------------------
-// keys (caller row << sh | caller col), values = internal slot
-__global__ void k_canon_keys(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-                             const int32_t *__restrict__ perm, int64_t n, int sh, uint64_t *keys, uint32_t *vals)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t ri = (uint64_t)(uint32_t)perm[i] << sh;
-        for (int64_t k = rowptr[i]; k < rowptr[i + 1]; ++k) {
-            keys[k] = ri | (uint64_t)(uint32_t)perm[col[k]];
-            vals[k] = (uint32_t)k;
-        }
-    }
-}
-
-__global__ void k_canon_invert(const uint32_t *__restrict__ vals, int64_t B, int32_t *kc_of)
-{
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < B; q += (int64_t)gridDim.x * blockDim.x)
-        kc_of[vals[q]] = (int32_t)q;
-}
-
 __global__ void k_row_len_caller(const int64_t *__restrict__ rowptr, const int32_t *__restrict__ inv, int64_t n,
                                  int64_t *len)
 {
@@ -798,20 +895,23 @@ void grid_build(GridView &g, const GridBuf &w, const dbl4 *x4, const dbl4 *u4, c
 }
 
 void bonds_count(const dbl4 *x4, const int32_t *grain, const int32_t *perm, int64_t n, const GridView &g,
-                 double delta, const FilterSet &f, int64_t *cnt, cudaStream_t st)
+                 double delta, const FilterSet &f, uint16_t *sides, int64_t *cnt, cudaStream_t st)
 {
-    k_bonds<false><<<grid_of(n, 128), 128, 0, st>>>(x4, grain, perm, n, g, delta * delta, f, cnt, nullptr, nullptr, 0);
+    if (f.nf) k_filter_sides<<<grid_of(n), 256, 0, st>>>(x4, n, f, sides);
+    k_bonds<false><<<grid_of(32 * n), 256, 0, st>>>(x4, grain, perm, n, g, delta * delta, f, sides, cnt, nullptr, nullptr);
 }
 
 void bonds_fill(const dbl4 *x4, const int32_t *grain, const int32_t *perm, int64_t n, const GridView &g,
-                double delta, const FilterSet &f, const int64_t *off, uint64_t *keys, int sh, cudaStream_t st)
+                double delta, const FilterSet &f, const uint16_t *sides, const int64_t *off, int32_t *found,
+                cudaStream_t st)
 {
-    k_bonds<true><<<grid_of(n, 128), 128, 0, st>>>(x4, grain, perm, n, g, delta * delta, f, nullptr, off, keys, sh);
+    k_bonds<true><<<grid_of(32 * n), 256, 0, st>>>(x4, grain, perm, n, g, delta * delta, f, sides, nullptr, off, found);
 }
 
-void bonds_keys_to_col(const uint64_t *keys, int64_t B, int sh, int32_t *col, cudaStream_t st)
+void order_rows(const int32_t *found, const int64_t *rowptr, const int32_t *perm, const int64_t *crow, int64_t n,
+                int32_t *col, int32_t *kc_of, cudaStream_t st)
 {
-    k_keys_to_col<<<grid_of(B), 256, 0, st>>>(keys, B, (1ull << sh) - 1ull, col);
+    k_order_rows<<<grid_of(n, ORDER_WARPS), 32 * ORDER_WARPS, 0, st>>>(found, rowptr, perm, crow, n, col, kc_of);
 }
 
 void cand_build(const int32_t *grain, const int64_t *rowptr, const int32_t *col, int64_t n, const GridView &g,
@@ -846,17 +946,6 @@ void stable_dt(const dbl4 *x4, const int64_t *rowptr, const int32_t *col, int64_
                double delta, int conic, double *partial, cudaStream_t st)
 {
     k_stable_dt<<<grid_of(n), 256, 0, st>>>(x4, rowptr, col, n, c, rho, delta, conic, partial);
-}
-
-void canon_keys(const int64_t *rowptr, const int32_t *col, const int32_t *perm, int64_t n, int sh, uint64_t *keys,
-                uint32_t *vals, cudaStream_t st)
-{
-    k_canon_keys<<<grid_of(n, 128), 128, 0, st>>>(rowptr, col, perm, n, sh, keys, vals);
-}
-
-void canon_invert(const uint32_t *vals, int64_t B, int32_t *kc_of, cudaStream_t st)
-{
-    k_canon_invert<<<grid_of(B), 256, 0, st>>>(vals, B, kc_of);
 }
 
 void row_len_caller(const int64_t *rowptr, const int32_t *inv, int64_t n, int64_t *len, cudaStream_t st)

@@ -18,11 +18,17 @@ void build_morton(const double *x_dev, int64_t n, const double lo[3], const doub
 void gather_nodes(const uint32_t *order, int64_t n, const double *x, const double *vol, const int32_t *grain,
                   const double *v0, int32_t *perm, int32_t *inv, dbl4 *x4, int32_t *grain_out, dbl4 *v,
                   float4 *xh4, float4 *xl4, const double centre[3], cudaStream_t st);
+// bonds of every node (sides: n words of scratch for the filters, kept for bonds_fill)
 void bonds_count(const dbl4 *x4, const int32_t *grain, const int32_t *perm, int64_t n, const GridView &g,
-                 double delta, const FilterSet &f, int64_t *cnt, cudaStream_t st);
+                 double delta, const FilterSet &f, uint16_t *sides, int64_t *cnt, cudaStream_t st);
+// the partners of every node in the order they are found, rows at off
 void bonds_fill(const dbl4 *x4, const int32_t *grain, const int32_t *perm, int64_t n, const GridView &g,
-                double delta, const FilterSet &f, const int64_t *off, uint64_t *keys, int sh, cudaStream_t st);
-void bonds_keys_to_col(const uint64_t *keys, int64_t B, int sh, int32_t *col, cudaStream_t st);
+                double delta, const FilterSet &f, const uint16_t *sides, const int64_t *off, int32_t *found,
+                cudaStream_t st);
+// rows sorted (col), and the canonical slot (caller rows at crow, ascending caller
+// columns) of every internal slot
+void order_rows(const int32_t *found, const int64_t *rowptr, const int32_t *perm, const int64_t *crow, int64_t n,
+                int32_t *col, int32_t *kc_of, cudaStream_t st);
 // contact candidates closer than cut: per row the range rng in cand
 void cand_build(const int32_t *grain, const int64_t *rowptr, const int32_t *col, int64_t n, const GridView &g,
                 const GridBuf &w, double cut, longlong2 *rng, int2 *cand, int64_t cap, unsigned *err, double *disp,
@@ -36,9 +42,6 @@ void damage(const int64_t *rowptr, const uint32_t *brk, const int32_t *perm, int
 int stable_dt_blocks(int64_t n);
 void stable_dt(const dbl4 *x4, const int64_t *rowptr, const int32_t *col, int64_t n, double c, double rho,
                double delta, int conic, double *partial, cudaStream_t st);
-void canon_keys(const int64_t *rowptr, const int32_t *col, const int32_t *perm, int64_t n, int sh, uint64_t *keys,
-                uint32_t *vals, cudaStream_t st);
-void canon_invert(const uint32_t *vals, int64_t B, int32_t *kc_of, cudaStream_t st);
 void row_len_caller(const int64_t *rowptr, const int32_t *inv, int64_t n, int64_t *len, cudaStream_t st);
 void col_caller(const int32_t *col, const int32_t *perm, const int32_t *kc_of, int64_t B, int32_t *out,
                 cudaStream_t st);
