@@ -125,14 +125,16 @@ typedef struct {
     int lanes_per_node;                  /* lanes sharing one node's bonds: 4, 8, 16, 32; 0 = autotune */
     int graph_chunk;                     /* steps per captured CUDA graph; 0 = 64 */
     int tiles;                           /* mixed path: shared-memory tiles 1 = on, -1 = off,
-                                            0 = chosen by the autotuner (on when lanes are fixed) */
+                                            0 = chosen by the library (off: slower on every body
+                                            measured) */
     int64_t cand_capacity;               /* initial capacity of the contact-candidate list
                                             (entries); 0 = max(1024, 8 n).  A rebuild that
                                             overflows it rolls its segment back and grows it. */
     int pairs;                           /* mixed path: each bond evaluated once, from its
                                             lower-index end, in two passes (Eq. pmb is pairwise
                                             antisymmetric): 1 = on, -1 = off, 0 = chosen by the
-                                            autotuner; pairs = 1 with tiles = 1 is PD_EINVAL */
+                                            library (off, as for tiles); pairs = 1 with tiles = 1
+                                            is PD_EINVAL */
     int persistent;                      /* pd_step runs the steps between two contact-list
                                             rebuilds in one cooperative launch (a grid-wide
                                             barrier between steps; same results bit for bit):
@@ -168,7 +170,7 @@ typedef struct {
 } pd_bond_filter;
 
 /* Fills *opt with defaults: device 0, default stream, cudaMalloc, PD_MIXED,
- * contact on, automatic rebuild period and skin, autotuned lanes and tiles,
+ * contact on, automatic rebuild period and skin, autotuned lanes,
  * chunk 64. */
 void pd_default_options(pd_options *opt);
 
@@ -331,14 +333,14 @@ pd_status pd_get_state_packed(pd_ctx *ctx, double *u, double *v, uint32_t *broke
 pd_status pd_set_state_packed(pd_ctx *ctx, const double *u, const double *v, const uint32_t *broken_bits,
                               const double *t);
 
-/* Autotuning record of the bond loop: lanes per node chosen, the kernel chosen
- * (0 = every directed slot gathers its neighbour from global memory, 1 =
- * shared-memory tiles, 2 = each bond once in two passes) and the measured time
- * (ms) of one force evaluation per candidate: ms[0..3] kernel 0 with 4, 8, 16, 32
- * lanes, ms[4..7] kernel 1, ms[8..11] kernel 2 (0 = not run).  The kernel is the
- * one with the fastest evaluation; its lane count the smallest within 3% of that
- * time (a full step's per-node work favours fewer lanes).  Any pointer may be
- * NULL. */
+/* Autotuning record of the bond loop: lanes per node chosen, the kernel in use (0 =
+ * every directed slot gathers its neighbour from global memory, 1 = shared-memory
+ * tiles, 2 = each bond once in two passes; 1 and 2 only on request, pd_options) and
+ * the measured time (ms) of one force evaluation per candidate: ms[0..3] kernel 0 with
+ * 4, 8, 16, 32 lanes, ms[4..7] kernel 1, ms[8..11] kernel 2 (0 = not run: another
+ * kernel, or more lanes than a count that lost clearly).  The lane count is the
+ * smallest within 3% of the fastest evaluation (a full step's per-node work favours
+ * fewer lanes).  Any pointer may be NULL. */
 pd_status pd_tuning(pd_ctx *ctx, int *lanes, int *kernel, double ms[12]);
 
 /* Profiling switch.  When on, pd_step launches its kernels one by one (no CUDA

@@ -663,37 +663,33 @@ static int step_grid(const pd_ctx *c, int lanes)
 
 static pd_status autotune(pd_ctx *c)
 {
-    // time a force evaluation (idempotent at a fixed state) for each lane count and
-    // each kernel the context can run: per-slot gathers from global memory (0),
-    // shared-memory tiles (1), each bond once in two passes (2)
+    // time a force evaluation (idempotent at a fixed state) for each lane count of the
+    // context's kernel: per-slot gathers from global memory (0), shared-memory tiles (1),
+    // each bond once in two passes (2)
     const int cand[4] = {4, 8, 16, 32};
     const bool mixed = c->opt.precision == PD_MIXED;
-    bool use[3] = {c->opt.tiles != 1 && c->opt.pairs != 1, c->tiled && c->opt.tiles != -1 && c->opt.pairs != 1,
-                   c->pairs_ok && c->opt.pairs != -1 && c->opt.tiles != 1};
-    if (!use[0] && !use[1] && !use[2]) use[0] = true;
+    const int kind = c->pairs ? 2 : (c->tiled ? 1 : 0);
     double best = INFINITY;
-    int bestl = 16, bestk = 0;
+    int bestl = 16;
     if (c->opt.contact) enqueue_rebuild(c, c->cur);
     for (int q = 0; q < 12; ++q) c->tune_ms[q] = 0;
     for (int q = 0; q < 4; ++q) {
-        for (int kind = 0; kind < 3; ++kind) {
-            if (!use[kind]) continue;
-            const int l = cand[q];
-            c->tiled = kind == 1;
-            c->pairs = kind == 2;
-            const int blocks = step_grid(c, l);
-            StepParams p = params(c, MODE_FORCES, c->cur, 0.0);
-            launch_step(p, l, blocks, c->st);  // warm-up; applies any breaking once
-            CK(cudaEventRecord(c->ev0, c->st));
-            for (int r = 0; r < 5; ++r) launch_step(p, l, blocks, c->st);
-            CK(cudaEventRecord(c->ev1, c->st));
-            CK(cudaEventSynchronize(c->ev1));
-            float ms = 0;
-            CK(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
-            const double t = ms / 5.0;
-            c->tune_ms[4 * kind + q] = t;
-            if (t < best) { best = t; bestl = l; bestk = kind; }
-        }
+        const int l = cand[q];
+        const int blocks = step_grid(c, l);
+        StepParams p = params(c, MODE_FORCES, c->cur, 0.0);
+        launch_step(p, l, blocks, c->st);  // warm-up; applies any breaking once
+        CK(cudaEventRecord(c->ev0, c->st));
+        for (int r = 0; r < 5; ++r) launch_step(p, l, blocks, c->st);
+        CK(cudaEventRecord(c->ev1, c->st));
+        CK(cudaEventSynchronize(c->ev1));
+        float ms = 0;
+        CK(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
+        const double t = ms / 5.0;
+        c->tune_ms[4 * kind + q] = t;
+        if (t < best) { best = t; bestl = l; }
+        // the time has one minimum over the lane counts: more lanes are not tried once
+        // they lose clearly
+        if (t > 1.2 * best) break;
     }
     // A full step adds per-node work to the force evaluation timed here (the Verlet
     // update on three lanes of each group, the grid rule of the state), which a
@@ -701,12 +697,10 @@ static pd_status autotune(pd_ctx *c)
     // the fewest lanes within 3% of its best force evaluation are taken (on the
     // plate 4 and 8 lanes tie within 0.5% here, and 4 lanes are 4% faster a step).
     for (int q = 0; q < 4 && cand[q] < bestl; ++q) {
-        const double t = c->tune_ms[4 * bestk + q];
+        const double t = c->tune_ms[4 * kind + q];
         if (t > 0 && t <= 1.03 * best) { bestl = cand[q]; break; }
     }
     CK(cudaMemsetAsync(c->derr, 0, sizeof(unsigned), c->st));
-    c->tiled = bestk == 1;
-    c->pairs = bestk == 2;
     c->lanes = bestl;
     c->blocks = step_grid(c, bestl);
     clear_graphs(c);
@@ -765,13 +759,19 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     row_len_caller(c->rowptr, c->inv, n, cnt, c->st);
     scan_exclusive_i64(cnt, c->crow, n, c->tmp, c->st);
     order_rows(found, c->rowptr, c->perm, c->crow, n, c->col, c->kc_of, c->st);
-    // shared-memory tiles (mixed path): the largest tile (64, 32 or 16 rows) whose
+    // Shared-memory tiles and the each-bond-once lists are built on request only: the
+    // per-slot kernel on global memory was the faster one on every body measured (force
+    // evaluation in ms, per-slot / tiles / each bond once, best lane count each: sphere of
+    // 4,139 nodes 0.012 / 0.021 / 0.020, plate of 178,200 0.145 / 0.240 / 0.269, hollow
+    // sphere of 343,846 0.159 / 0.271 / 0.310, packing of 2.1 M 0.93 / 1.8 / 2.1), and
+    // building and timing the other two took half of this call.
+    // Tiles (mixed path): the largest tile (64, 32 or 16 rows) whose
     // staging fits two blocks per SM.  A material with friction or multi-wall terms
     // runs the global-gather kernels that carry the wall extras, so it has no tiles.
     release(c, c->tile_ptr); release(c, c->ulist); release(c, c->lcol); release(c, c->lrow);
     c->tiled = false;
     c->tile_cap = 0;
-    if (c->opt.precision == PD_MIXED && c->opt.tiles >= 0 && !(c->mat.mu > 0) && !c->mat.wall_overlap) {
+    if (c->opt.precision == PD_MIXED && c->opt.tiles == 1 && !(c->mat.mu > 0) && !c->mat.wall_overlap) {
         const int64_t m = B + n;
         const size_t smem_max = 110 * 1024;
         std::vector<int64_t> rp(n + 1);
@@ -848,7 +848,7 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     }
     // each bond once (mixed path; materials whose walls need the extra terms run the
     // per-slot kernels that carry them)
-    if (c->opt.precision == PD_MIXED && c->opt.pairs >= 0 && !(c->mat.mu > 0) && !c->mat.wall_overlap) {
+    if (c->opt.precision == PD_MIXED && c->opt.pairs == 1 && !(c->mat.mu > 0) && !c->mat.wall_overlap) {
         ALLOC(c->split, int32_t, n + 1);
         ALLOC(c->mir, int32_t, B + 16);
         ALLOC(c->tb, float, B + 16);
@@ -860,8 +860,7 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
         s = sync(c);
         if (s) return s;
         if (bad) return fail(c, PD_ECUDA, "bond list is not symmetric");
-        c->pairs_ok = true;
-        c->pairs = c->opt.pairs == 1;
+        c->pairs_ok = c->pairs = true;
     }
     CK(cudaGetLastError());
     s = sync(c);

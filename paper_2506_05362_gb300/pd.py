@@ -341,7 +341,7 @@ def pack_broken(broken):
 
 
 def pd_tuning(h):
-    """(lanes per node, kernel: 0 global gathers / 1 tiles / 2 each bond once,
+    """(lanes per node, kernel: 0 global gathers / 1 tiles / 2 each bond once (on request),
     ms per candidate: 4 lane counts for each kernel in that order)."""
     lanes, kernel = ctypes.c_int(), ctypes.c_int()
     ms = np.zeros(12)
