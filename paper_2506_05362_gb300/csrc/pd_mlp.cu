@@ -17,7 +17,7 @@
 #include <string>
 #include <vector>
 
-#include "pd_internal.cuh"
+#include "pd_mlp.cuh"
 
 typedef __nv_bfloat16 bf16;
 
@@ -277,7 +277,7 @@ __global__ void k_to_bf16_pad(const float *__restrict__ X, int64_t rows, int col
 
 // dY = bf16(2 (Y - T) / (B * nout)), padded to ldo; per-block loss partials
 __global__ void k_loss(const float *__restrict__ Y, const float *__restrict__ T, int64_t rows, int nout, int ldo,
-                       bf16 *dY, float *partial, bf16 *dYT, int64_t ldT)
+                       bf16 *dY, float *partial)
 {
     __shared__ float s[256];
     float acc = 0.f;
@@ -292,7 +292,6 @@ __global__ void k_loss(const float *__restrict__ Y, const float *__restrict__ T,
             acc += d * d;
         }
         dY[q] = __float2bfloat16_rn(d * scale);
-        if (dYT) dYT[(int64_t)c * ldT + r] = dY[q];  // transposed copy for the weight gradient
     }
     s[threadIdx.x] = acc;
     __syncthreads();
@@ -316,49 +315,6 @@ __global__ void k_loss_final(const float *__restrict__ partial, int nb, int64_t 
         __syncthreads();
     }
     if (threadIdx.x == 0) *loss = (float)(s[0] / (double)count);
-}
-
-// row sums of dZ^T (bf16 [n x ld], first `rows` columns) into gb: the bias
-// gradient from the transposed copy, with coalesced reads; fixed order
-constexpr int RS_THREADS = 1024;  // one block per column; two blocks fit an SM, so the columns take one wave
-__global__ void __launch_bounds__(RS_THREADS) k_rowsum(const bf16 *__restrict__ dZT, int64_t rows, int64_t ld,
-                                                       int n_valid, float *gb)
-{
-    __shared__ float s[RS_THREADS];
-    const int c = blockIdx.x;
-    float acc = 0.f;
-    const bf16 *r = dZT + (int64_t)c * ld;  // ld is a multiple of 8: rows start 16-byte aligned
-    const int64_t r8 = rows / 8;
-    // RS_BATCH 16-byte loads of a thread are issued before any is added (one block
-    // per column leaves few loads in flight otherwise); the additions keep the
-    // order of a plain strided loop
-    constexpr int RS_BATCH = 8;
-    for (int64_t q0 = threadIdx.x; q0 < r8; q0 += (int64_t)RS_BATCH * blockDim.x) {
-        uint4 w[RS_BATCH];
-#pragma unroll
-        for (int b = 0; b < RS_BATCH; ++b) {
-            const int64_t q = q0 + (int64_t)b * blockDim.x;
-            w[b] = q < r8 ? *(const uint4 *)(r + 8 * q) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int b = 0; b < RS_BATCH; ++b) {
-            if (q0 + (int64_t)b * blockDim.x >= r8) break;
-            const __nv_bfloat162 *h = (const __nv_bfloat162 *)&w[b];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float2 f = __bfloat1622float2(h[e]);
-                acc += f.x + f.y;
-            }
-        }
-    }
-    for (int64_t q = 8 * r8 + threadIdx.x; q < rows; q += blockDim.x) acc += __bfloat162float(r[q]);
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = RS_THREADS / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && c < n_valid) gb[c] = s[0];
 }
 
 // fixed-order sum of split-K partials into the gradient vector; rows < n_valid,
@@ -427,6 +383,83 @@ __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float
     }
 }
 
+// Everything after the last GEMM of a tcgen05 training step in one launch: the split-K
+// partials of every layer's weight and bias gradients summed in a fixed order into the
+// gradient vector, and, for a training step, Adam on them and the new weights and biases
+// in the layouts the GEMMs read (their padding stays as it was set); block 0 also sums the
+// loss.  A thread takes one parameter, its partials eight loads at a time: bound by the
+// latency of those loads (16 partials of 0.9 MB each, from L2).  16 launches (reductions,
+// bias row sums, Adam, repacking) did this before: 135 us a step of the surrogate at batch
+// 65,536, this 8.9 us; one warp per 32 parameters and part of the splits, as in
+// k_reduce_dw, took 20.
+struct UpdateLayer {
+    const float *part, *partb;  // [splits x N x K], [splits x N]
+    int N, K, k_valid;
+    int64_t w0, b0;             // offsets of W and b in the parameter vector (b follows W)
+    bf16 *Wb, *WT;
+    float *bias;
+};
+struct Update {
+    int L, splits;
+    int64_t nparams;
+    UpdateLayer l[8];
+    float *w, *m, *v, *g;
+    int adam;
+    float lr, b1, b2, eps, c1, c2;
+    const float *lpart;
+    int nlp;
+    int64_t lcount;
+    float *loss, *loss2;        // loss2 nullable
+};
+
+__global__ void __launch_bounds__(256) k_update(const __grid_constant__ Update U)
+{
+    __shared__ double sd[256];
+    if (blockIdx.x == 0) {
+        double acc = 0.0;
+        for (int b = threadIdx.x; b < U.nlp; b += 256) acc += U.lpart[b];
+        sd[threadIdx.x] = acc;
+        __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if ((int)threadIdx.x < o) sd[threadIdx.x] += sd[threadIdx.x + o];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            const float loss = (float)(sd[0] / (double)U.lcount);
+            *U.loss = loss;
+            if (U.loss2) *U.loss2 = loss;
+        }
+    }
+    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (p >= U.nparams) return;
+    int l = 0;
+    while (l + 1 < U.L && p >= U.l[l + 1].w0) ++l;
+    const UpdateLayer &Y = U.l[l];
+    const bool isw = p < Y.b0;
+    const int q = (int)(p - (isw ? Y.w0 : Y.b0));
+    const int r = isw ? q / Y.k_valid : q, c = isw ? q - r * Y.k_valid : 0;
+    const float *src = isw ? Y.part + (size_t)r * Y.K + c : Y.partb + r;
+    const size_t zs = isw ? (size_t)Y.N * Y.K : (size_t)Y.N;
+    float g = 0.f;
+#pragma unroll 8
+    for (int z = 0; z < U.splits; ++z) g += __ldcs(src + (size_t)z * zs);
+    U.g[p] = g;
+    if (!U.adam) return;
+    const float mq = U.b1 * U.m[p] + (1.f - U.b1) * g;
+    const float vq = U.b2 * U.v[p] + (1.f - U.b2) * g * g;
+    U.m[p] = mq;
+    U.v[p] = vq;
+    const float w = U.w[p] - U.lr * (mq / U.c1) / (sqrtf(vq / U.c2) + U.eps);
+    U.w[p] = w;
+    if (isw) {
+        const bf16 h = __float2bfloat16_rn(w);
+        Y.Wb[(size_t)r * Y.K + c] = h;
+        Y.WT[(size_t)c * Y.N + r] = h;
+    } else {
+        Y.bias[r] = w;
+    }
+}
+
 // masters (layout W [out x in] then b) -> padded bf16 W [out_pad x in_pad] and fp32 bias [out_pad]
 __global__ void k_pack_layer(const float *__restrict__ W, const float *__restrict__ b, int out, int in, int out_pad,
                              int in_pad, bf16 *Wb, float *bp, bf16 *WT)
@@ -475,16 +508,6 @@ struct pd_mlp {
     int path = 0;                // 0: tcgen05 forward when the shapes allow; 1: mma.sync only
     std::vector<void *> owned;
 };
-
-int mlp_forward_tc(int L, const int *dims, const int *pad, void *const *W, const float *const *bias, const float *X,
-                   int64_t rows, float *Y, unsigned *err, int device, cudaStream_t st);
-int mlp_forward_train_tc(int L, const int *dims, const int *pad, void *const *W, const float *const *bias,
-                         const float *X, int64_t rows, float *Y, void *const *Z, void *const *HT, int64_t ldT,
-                         unsigned *err, int device, cudaStream_t st);
-int mlp_dgelu_tc(const void *dZ, const void *WT, const void *z, int64_t rows, int N, int K, void *out, void *outT,
-                 int64_t ldT, unsigned *err, int device, cudaStream_t st);
-int mlp_dw_tc(const void *dZT, const void *HT, int64_t rows, int64_t ldT, int M, int N, float *part, int max_splits,
-              unsigned *err, int device, cudaStream_t st);
 
 namespace {
 
@@ -586,7 +609,7 @@ pd_status forward_dev(pd_mlp *m, const float *X, int64_t rows, float *Y, bool ke
         void *W[8];
         const float *b[8];
         for (int l = 0; l < m->L; ++l) { W[l] = m->Wb[l]; b[l] = m->bias[l]; }
-        if (mlp_forward_tc(m->L, m->dims, m->pad, W, b, X, rows, Y, m->tc_err, m->device, m->st) == 0)
+        if (mlp_forward_tc(m->L, m->dims, m->pad, W, b, X, rows, Y, nullptr, m->tc_err, m->device, m->st) > 0)
             return PD_OK;
         if (m->path == 2) return mfail(m, PD_EINVAL, "the tcgen05 forward cannot run this network or GPU");
     }
@@ -615,6 +638,17 @@ pd_status forward_dev(pd_mlp *m, const float *X, int64_t rows, float *Y, bool ke
     return PD_OK;
 }
 
+// one more Adam step: its constants
+void adam_constants(pd_mlp *m, float *b1, float *b2, float *eps, float *c1, float *c2)
+{
+    m->t += 1;
+    *b1 = 0.9f;
+    *b2 = 0.999f;
+    *eps = 1e-8f;
+    *c1 = (float)(1.0 - pow(0.9, (double)m->t));
+    *c2 = (float)(1.0 - pow(0.999, (double)m->t));
+}
+
 pd_status ensure_part(pd_mlp *m, int64_t need)
 {
     if (need <= m->part_cap) return PD_OK;
@@ -626,11 +660,13 @@ pd_status ensure_part(pd_mlp *m, int64_t need)
     return PD_OK;
 }
 
-// The same gradient on the tcgen05 kernels: the fused forward stores Z and the
-// transposed layer inputs; dW = dZ^T H and dZ_{l-1} = (dZ_l W_l) GELU'(Z_{l-1})
-// are tcgen05 GEMMs with K-major operands.  Returns -1 (nothing enqueued that
-// changes results) when the kernels cannot run this network.
-int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float *dloss)
+// The gradient on the tcgen05 kernels: the fused forward stores Z and the transposed
+// layer inputs and ends in the loss gradient; dW = dZ^T H and dZ_{l-1} = (dZ_l W_l)
+// GELU'(Z_{l-1}) are tcgen05 GEMMs with K-major operands; one launch sums the partials
+// into m->grad, and with lr > 0 takes the Adam step.  loss2 (nullable) also receives the
+// loss.  Returns -1 (nothing enqueued that changes results) when the kernels cannot run
+// this network.
+int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float lr, float *loss2)
 {
     const int L = m->L, nout = m->dims[L];
     for (int l = 0; l + 1 < L; ++l)
@@ -639,33 +675,64 @@ int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float *
     const float *b[8];
     void *Z[8];
     for (int l = 0; l < L; ++l) { W[l] = m->Wb[l]; b[l] = m->bias[l]; HT[l] = m->HT[l]; Z[l] = m->Z[l]; }
-    if (mlp_forward_train_tc(L, m->dims, m->pad, W, b, X, rows, m->Y, Z, HT, m->ldT, m->tc_err, m->device, m->st))
-        return -1;
-    const int nb = std::min(grid1(rows * m->pad[L]), 8192);
-    k_loss<<<nb, 256, 0, m->st>>>(m->Y, T, rows, nout, m->pad[L], m->dZ[L - 1], m->lpart, m->dZT[L - 1], m->ldT);
-    k_loss_final<<<1, 256, 0, m->st>>>(m->lpart, nb, rows * nout, dloss);
-    const int max_splits = 128;
-    for (int l = L - 1; l >= 0; --l) {
-        const int N = m->pad[l + 1], K = m->pad[l];
-        if (ensure_part(m, (int64_t)max_splits * ((N + 127) / 128 * 128) * K)) return -2;
-        const int splits = mlp_dw_tc(m->dZT[l], m->HT[l], rows, m->ldT, N, K, m->part, max_splits, m->tc_err,
-                                     m->device, m->st);
-        if (splits <= 0) return -2;
-        k_reduce_dw<<<rd_blocks((int64_t)m->dims[l + 1] * m->dims[l]), 32 * RD_PARTS, 0, m->st>>>(
-            m->part, splits, N, K, m->dims[l + 1], m->dims[l], m->grad + m->woff[l]);
-        k_rowsum<<<m->dims[l + 1], RS_THREADS, 0, m->st>>>(m->dZT[l], rows, m->ldT, m->dims[l + 1], m->grad + m->boff[l]);
-        if (l > 0 && mlp_dgelu_tc(m->dZ[l], m->WT[l], m->Z[l - 1], rows, K, N, m->dZ[l - 1], m->dZT[l - 1], m->ldT,
-                                  m->tc_err, m->device, m->st))
-            return -2;
+    MlpTrain tr;
+    tr.Z = Z;
+    tr.HT = HT;
+    tr.ldT = m->ldT;
+    tr.T = T;
+    tr.scale = 2.0f / (float)(rows * nout);
+    tr.dY = m->dZ[L - 1];
+    tr.dYT = m->dZT[L - 1];
+    tr.lpart = m->lpart;
+    // room for every layer's partials
+    int64_t need = 0, at[8];
+    const int splits = mlp_dw_splits(L, m->pad, rows, m->device);
+    for (int l = 0; l < L; ++l) {
+        at[l] = need;
+        need += (int64_t)splits * m->pad[l + 1] * (m->pad[l] + 1);
+        need = (need + 31) / 32 * 32;
     }
+    const int nlp = mlp_forward_tc(L, m->dims, m->pad, W, b, X, rows, nullptr, &tr, m->tc_err, m->device, m->st);
+    if (nlp < 0) return -1;
+    if (ensure_part(m, need)) return -2;
+    void *WT[8], *dZT[8];
+    for (int l = 0; l < L; ++l) { WT[l] = m->WT[l]; dZT[l] = m->dZT[l]; }
+    if (mlp_backward_tc(L, m->pad, WT, &tr, dZT, rows, m->tc_err, m->device, m->st) < 0) return -2;
+    Update U;
+    memset(&U, 0, sizeof(U));
+    U.L = L;
+    float *part[8], *partb[8];
+    for (int l = 0; l < L; ++l) {
+        const int N = m->pad[l + 1], K = m->pad[l];
+        part[l] = m->part + at[l];
+        partb[l] = part[l] + (int64_t)splits * N * K;
+        UpdateLayer &Y = U.l[l];
+        Y.part = part[l]; Y.partb = partb[l]; Y.N = N; Y.K = K;
+        Y.k_valid = m->dims[l];
+        Y.w0 = m->woff[l]; Y.b0 = m->boff[l];
+        Y.Wb = m->Wb[l]; Y.WT = m->WT[l]; Y.bias = m->bias[l];
+    }
+    if (mlp_dw_tc(L, m->pad, dZT, HT, rows, m->ldT, part, partb, m->tc_err, m->device, m->st)) return -2;
+    U.splits = splits;
+    U.nparams = m->nparams;
+    U.w = m->master; U.m = m->m; U.v = m->v; U.g = m->grad;
+    if (lr > 0) {
+        U.adam = 1;
+        adam_constants(m, &U.b1, &U.b2, &U.eps, &U.c1, &U.c2);
+        U.lr = lr;
+    }
+    U.lpart = m->lpart; U.nlp = nlp; U.lcount = rows * nout;
+    U.loss = m->dloss; U.loss2 = loss2;
+    k_update<<<(unsigned)((m->nparams + 255) / 256), 256, 0, m->st>>>(U);
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
-// gradient of the MSE loss into m->grad (parameter layout); loss to dloss (device)
-pd_status backward_dev(pd_mlp *m, const float *X, const float *T, int64_t rows, float *dloss)
+// gradient of the MSE loss into m->grad (parameter layout), the loss into m->dloss and
+// loss2 (device, nullable); with lr > 0 one Adam step
+pd_status backward_dev(pd_mlp *m, const float *X, const float *T, int64_t rows, float lr, float *loss2)
 {
     if (m->path != 1) {
-        const int r = backward_tc(m, X, T, rows, dloss);
+        const int r = backward_tc(m, X, T, rows, lr, loss2);
         if (r == 0) return PD_OK;
         if (r == -2) return mfail(m, PD_ECUDA, "tcgen05 training kernels failed to launch");
         if (m->path == 2) return mfail(m, PD_EINVAL, "the tcgen05 kernels cannot train this network or GPU");
@@ -674,8 +741,9 @@ pd_status backward_dev(pd_mlp *m, const float *X, const float *T, int64_t rows, 
     if (s) return s;
     const int L = m->L, nout = m->dims[L];
     const int nb = std::min(grid1(rows * m->pad[L]), 8192);
-    k_loss<<<nb, 256, 0, m->st>>>(m->Y, T, rows, nout, m->pad[L], m->dZ[L - 1], m->lpart, nullptr, 0);
-    k_loss_final<<<1, 256, 0, m->st>>>(m->lpart, nb, rows * nout, dloss);
+    k_loss<<<nb, 256, 0, m->st>>>(m->Y, T, rows, nout, m->pad[L], m->dZ[L - 1], m->lpart);
+    k_loss_final<<<1, 256, 0, m->st>>>(m->lpart, nb, rows * nout, m->dloss);
+    if (loss2) MCK(cudaMemcpyAsync(loss2, m->dloss, sizeof(float), cudaMemcpyDeviceToDevice, m->st));
     for (int l = L - 1; l >= 0; --l) {
         const int N = m->pad[l + 1], K = m->pad[l];
         // weight gradient: dW = dZ^T H, batch split across CTAs
@@ -715,6 +783,13 @@ pd_status backward_dev(pd_mlp *m, const float *X, const float *T, int64_t rows, 
         }
     }
     MCK(cudaGetLastError());
+    if (lr > 0) {
+        float b1, b2, eps, c1, c2;
+        adam_constants(m, &b1, &b2, &eps, &c1, &c2);
+        k_adam<<<grid1(m->nparams), 256, 0, m->st>>>(m->master, m->grad, m->m, m->v, m->nparams, lr, b1, b2, eps, c1,
+                                                     c2);
+        return pack_all(m);
+    }
     return PD_OK;
 }
 
@@ -859,11 +934,11 @@ pd_status pd_mlp_set_forward_path(pd_mlp *m, int path)
     return PD_OK;
 }
 
-static pd_status grad_impl(pd_mlp *m, const float *Xd, const float *Td, int64_t batch)
+static pd_status grad_impl(pd_mlp *m, const float *Xd, const float *Td, int64_t batch, float lr, float *loss2)
 {
     pd_status s = ensure_cap(m, batch, true);
     if (s) return s;
-    return backward_dev(m, Xd, Td, batch, m->dloss);
+    return backward_dev(m, Xd, Td, batch, lr, loss2);
 }
 
 pd_status pd_mlp_grad(pd_mlp *m, const float *X, const float *T, int64_t batch, float *grad, float *loss)
@@ -874,7 +949,7 @@ pd_status pd_mlp_grad(pd_mlp *m, const float *X, const float *T, int64_t batch, 
     if (s) return s;
     MCK(cudaMemcpyAsync(m->Xf, X, sizeof(float) * batch * m->dims[0], cudaMemcpyHostToDevice, m->st));
     MCK(cudaMemcpyAsync(m->Tf, T, sizeof(float) * batch * m->dims[m->L], cudaMemcpyHostToDevice, m->st));
-    s = grad_impl(m, m->Xf, m->Tf, batch);
+    s = grad_impl(m, m->Xf, m->Tf, batch, 0.f, nullptr);
     if (s) return s;
     MCK(cudaMemcpyAsync(grad, m->grad, sizeof(float) * m->nparams, cudaMemcpyDeviceToHost, m->st));
     if (loss) MCK(cudaMemcpyAsync(loss, m->dloss, sizeof(float), cudaMemcpyDeviceToHost, m->st));
@@ -882,24 +957,11 @@ pd_status pd_mlp_grad(pd_mlp *m, const float *X, const float *T, int64_t batch, 
     return PD_OK;
 }
 
-static pd_status adam(pd_mlp *m, float lr)
-{
-    m->t += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = (float)(1.0 - pow(0.9, (double)m->t)), c2 = (float)(1.0 - pow(0.999, (double)m->t));
-    k_adam<<<grid1(m->nparams), 256, 0, m->st>>>(m->master, m->grad, m->m, m->v, m->nparams, lr, b1, b2, 1e-8f,
-                                                 c1, c2);
-    return pack_all(m);
-}
-
 pd_status pd_mlp_train_step_device(pd_mlp *m, const float *X, const float *T, int64_t batch, float lr, float *loss)
 {
     if (!m || !X || !T || batch < 1 || batch > 0x7fffffff || !(lr > 0)) return PD_EINVAL;
     MCK(cudaSetDevice(m->device));
-    pd_status s = grad_impl(m, X, T, batch);
-    if (s) return s;
-    if (loss) MCK(cudaMemcpyAsync(loss, m->dloss, sizeof(float), cudaMemcpyDeviceToDevice, m->st));
-    return adam(m, lr);
+    return grad_impl(m, X, T, batch, lr, loss);
 }
 
 pd_status pd_mlp_train_step(pd_mlp *m, const float *X, const float *T, int64_t batch, float lr, float *loss)
@@ -910,11 +972,9 @@ pd_status pd_mlp_train_step(pd_mlp *m, const float *X, const float *T, int64_t b
     if (s) return s;
     MCK(cudaMemcpyAsync(m->Xf, X, sizeof(float) * batch * m->dims[0], cudaMemcpyHostToDevice, m->st));
     MCK(cudaMemcpyAsync(m->Tf, T, sizeof(float) * batch * m->dims[m->L], cudaMemcpyHostToDevice, m->st));
-    s = grad_impl(m, m->Xf, m->Tf, batch);
+    s = grad_impl(m, m->Xf, m->Tf, batch, lr, nullptr);
     if (s) return s;
     if (loss) MCK(cudaMemcpyAsync(loss, m->dloss, sizeof(float), cudaMemcpyDeviceToHost, m->st));
-    s = adam(m, lr);
-    if (s) return s;
     MCK(cudaStreamSynchronize(m->st));
     return PD_OK;
 }

@@ -16,6 +16,14 @@
 //               bias, exact-erf GELU, round to BF16 and write the next layer's A
 //               tile in the swizzled layout; the last layer writes FP32 outputs.
 //               They also stage the input tile with coalesced reads.
+// The same kernel runs a training step's forward (it also stores what the backward needs
+// and ends in the loss) and, over the layers in reverse with the transposed weights, its
+// backward: dZ_{l-1} = (dZ_l W_l) GELU'(Z_{l-1}) stays in shared memory from layer to layer
+// and only its transposed copy, the operand of the weight gradient, is stored.  Both are
+// bound by the epilogue's instructions (GELU or GELU', the transposition by lane pairs, the
+// stores of 283 MB forward and 149 MB backward): 142 and 129 us at batch 65,536 of the
+// surrogate, 45 and 40 us at 4,096.  The forward with two-byte transposed stores and the
+// loss in two launches of its own took 175 and 59 us.
 // Every mbarrier wait is bounded; on timeout the kernel records an error word,
 // stops issuing, frees its TMEM and returns.
 #include <cuda.h>
@@ -24,7 +32,7 @@
 
 #include <string.h>
 
-#include "pd_internal.cuh"
+#include "pd_mlp.cuh"
 
 namespace tc {
 
@@ -62,7 +70,17 @@ struct Params {
     __nv_bfloat16 *Z[MAX_LAYERS];
     __nv_bfloat16 *HT[MAX_LAYERS];
     int64_t ldT;
+    // and the MSE loss: targets [rows x out_cols], dY = scale (Y - T) as BF16 [rows x
+    // N_last] and transposed [N_last x ldT], and one partial sum of (Y - T)^2 a CTA
+    const float *T;
+    float scale;
+    __nv_bfloat16 *dY, *dYT;
+    float *lpart;
+    // backward: the input is dY [rows x K_0]; layer i multiplies by GELU' of Z[i] [rows x
+    // N_i] and stores its transposed result to HT[i] [N_i x ldT]
 };
+
+enum Mode { INFER, TRAIN_FWD, TRAIN_BWD };
 
 // ---- PTX wrappers -------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -169,6 +187,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
     for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
 }
 
+// 8 accumulator columns, as the 16-column pair below
+__device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait8(uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+                 :
+                 : "memory");
+}
+
 // 16 accumulator columns of this thread's TMEM lane, issued without waiting:
 // the registers hold the values only after tmem_wait16 on them
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16])
@@ -234,6 +267,35 @@ __device__ __forceinline__ float2 gelu2(float2 z)
     return __ffma2_rn(n, phi, make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f)));
 }
 
+// The training forward's GELU: the function whose derivative gelu_grad() takes, in the
+// same form (the special-function unit does not bound that epilogue).  Same method as
+// gelu() below (Abramowitz & Stegun eq. 7.1.26 for erf, odd extension):
+//   x = |z|/sqrt2, t = 1/(1 + p x), e = erf(x) = 1 - t P(t) exp(-x^2),
+//   GELU = z/2 (1 + sign(z) e); the Horner coefficients carry the minus sign so
+//   that e is one fused multiply-add, and sign(z) e is e with z's sign bit
+//   (e >= 0).  exp(-x^2) = 2^(-x^2 log2 e) on the hardware ex2.
+__device__ __forceinline__ float2 gelu2_train(float2 z)
+{
+    const float2 c = make_float2(0.70710678118654752f, 0.70710678118654752f);
+    float2 x = __fmul2_rn(z, c);
+    x.x = fabsf(x.x);
+    x.y = fabsf(x.y);
+    const float2 d = __ffma2_rn(make_float2(0.3275911f, 0.3275911f), x, make_float2(1.0f, 1.0f));
+    const float2 t = make_float2(rcp_approx(d.x), rcp_approx(d.y));
+    float2 q = __ffma2_rn(t, make_float2(-1.061405429f, -1.061405429f), make_float2(1.453152027f, 1.453152027f));
+    q = __ffma2_rn(t, q, make_float2(-1.421413741f, -1.421413741f));
+    q = __ffma2_rn(t, q, make_float2(0.284496736f, 0.284496736f));
+    q = __ffma2_rn(t, q, make_float2(-0.254829592f, -0.254829592f));
+    q = __fmul2_rn(t, q);  // -t P(t)
+    const float2 w = __fmul2_rn(x, __fmul2_rn(x, make_float2(-1.4426950408889634f, -1.4426950408889634f)));
+    const float2 ex = make_float2(ex2_approx(w.x), ex2_approx(w.y));
+    const float2 e = __ffma2_rn(q, ex, make_float2(1.0f, 1.0f));
+    const float2 es = make_float2(__uint_as_float(__float_as_uint(e.x) | (__float_as_uint(z.x) & 0x80000000u)),
+                                  __uint_as_float(__float_as_uint(e.y) | (__float_as_uint(z.y) & 0x80000000u)));
+    const float2 hz = __fmul2_rn(z, make_float2(0.5f, 0.5f));
+    return __ffma2_rn(hz, es, hz);
+}
+
 // two floats rounded to BF16 (nearest-even), packed low = a, high = b, in registers
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b)
 {
@@ -256,6 +318,19 @@ __device__ __forceinline__ float gelu(float z)
     return 0.5f * z * (1.0f + copysignf(e, z));
 }
 
+// GELU'(z) = Phi(z) + z phi(z); Phi from the Abramowitz-Stegun erf of gelu(),
+// and exp(-z^2/2) is the exp(-x^2) of that erf
+__device__ __forceinline__ float gelu_grad(float z)
+{
+    const float x = fabsf(z) * 0.70710678118654752f;
+    const float t = rcp_approx(fmaf(0.3275911f, x, 1.0f));
+    const float poly =
+        t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f), 0.254829592f);
+    const float ex = ex2_approx(-1.4426950408889634f * x * x);
+    const float e = 1.0f - poly * ex;
+    return 0.5f * (1.0f + copysignf(e, z)) + z * ex * 0.3989422804014327f;
+}
+
 // byte offset of element (m, k) of a 128-row K-major BF16 tile in the 128-byte
 // swizzled layout: atoms of 64 columns (16 KiB), 8-row groups of 1024 bytes,
 // 16-byte chunk index XOR-ed with the row within its group
@@ -265,19 +340,35 @@ __device__ __forceinline__ uint32_t sw128_offset(int m, int k)
     return (uint32_t)(atom * (TILE_M * 128) + g * 1024 + r * 128 + ((c ^ r) << 4) + ((k & 7) << 1));
 }
 
-// bias + GELU + BF16 of the 16 accumulator columns [c, c + 16) of row m, written
-// to the next layer's swizzled A tile: the arithmetic of the whole-chunk path,
-// element for element (c is a multiple of 16, so the bias loads are aligned)
-__device__ __forceinline__ void epi16(const float *bias, const uint32_t (&r)[16], int c, unsigned char *sA, int m)
+// Two columns of this lane's row and its neighbour's (lane ^ 1), held as one packed word
+// a lane, stored to a transposed array [column x ld]: the even lane takes the first
+// column of both rows, the odd lane the second, so that a warp's store writes 64
+// consecutive bytes of each column in words of two rows.  All lanes call it.
+__device__ __forceinline__ void store_pair_T(__nv_bfloat16 *T, int64_t ld, int c, int64_t row, bool valid, uint32_t w)
 {
-    float bb[16];
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, w, 1);
+    const bool odd = row & 1;
+    const uint32_t v = odd ? __byte_perm(o, w, 0x7632) : __byte_perm(w, o, 0x5410);
+    if (valid) *(uint32_t *)(T + (int64_t)(c + odd) * ld + (row & ~(int64_t)1)) = v;
+}
+
+template <int N>
+__device__ __forceinline__ void load_bias(const float *bias, float (&b)[N])
+{
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float4 t4 = __ldg((const float4 *)(bias + c) + i);
-        bb[4 * i] = t4.x; bb[4 * i + 1] = t4.y; bb[4 * i + 2] = t4.z; bb[4 * i + 3] = t4.w;
+    for (int i = 0; i < N / 4; ++i) {
+        const float4 t4 = __ldg((const float4 *)bias + i);
+        b[4 * i] = t4.x; b[4 * i + 1] = t4.y; b[4 * i + 2] = t4.z; b[4 * i + 3] = t4.w;
     }
+}
+
+// bias + GELU + BF16 of the N accumulator columns [c, c + N) of row m, written to the next
+// layer's swizzled A tile
+template <int N>
+__device__ __forceinline__ void epi_hidden(const float (&bb)[N], const uint32_t (&r)[N], int c, unsigned char *sA, int m)
+{
 #pragma unroll
-    for (int c8 = 0; c8 < 16; c8 += 8) {
+    for (int c8 = 0; c8 < N; c8 += 8) {
         uint32_t pk[4];
 #pragma unroll
         for (int e = 0; e < 8; e += 2) {
@@ -287,6 +378,45 @@ __device__ __forceinline__ void epi16(const float *bias, const uint32_t (&r)[16]
             pk[e / 2] = pack_bf16x2(g2.x, g2.y);
         }
         *(uint4 *)(sA + sw128_offset(m, c + c8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
+}
+
+// the same for 8 columns in training (row of the batch): also the transposed activations,
+// and the pre-activations in zw
+__device__ __forceinline__ void epi_train8(const float (&bb)[8], const uint32_t (&r)[8], int c, unsigned char *sA, int m,
+                                           const Params &P, int l, int64_t row, uint4 &zw)
+{
+    uint32_t pk[4], z[4];
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) {
+        const float2 zz = __fadd2_rn(make_float2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])),
+                                     make_float2(bb[e], bb[e + 1]));
+        z[e / 2] = pack_bf16x2(zz.x, zz.y);
+        const float2 g2 = gelu2_train(zz);
+        pk[e / 2] = pack_bf16x2(g2.x, g2.y);
+        store_pair_T(P.HT[l + 1], P.ldT, c + e, row, (row & ~(int64_t)1) < P.rows, pk[e / 2]);
+    }
+    *(uint4 *)(sA + sw128_offset(m, c)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    zw = make_uint4(z[0], z[1], z[2], z[3]);
+}
+
+// 16 columns [c, c + 16) of the data gradient of row m (row of the batch): times GELU' of
+// the pre-activations z0, z1, rounded, written to the next layer's A tile (unless it is
+// the last) and to the transposed copy
+__device__ __forceinline__ void dgelu16(const Params &P, const uint32_t (&r)[16], const uint4 &z0, const uint4 &z1, int c,
+                                        unsigned char *sA, int m, int l, int64_t row, bool last)
+{
+    const uint32_t zw[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+    uint32_t pk[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float2 z = __bfloat1622float2(*(const __nv_bfloat162 *)&zw[i]);
+        pk[i] = pack_bf16x2(__uint_as_float(r[2 * i]) * gelu_grad(z.x), __uint_as_float(r[2 * i + 1]) * gelu_grad(z.y));
+        store_pair_T(P.HT[l], P.ldT, c + 2 * i, row, (row & ~(int64_t)1) < P.rows, pk[i]);
+    }
+    if (!last) {
+        *(uint4 *)(sA + sw128_offset(m, c)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *(uint4 *)(sA + sw128_offset(m, c + 8)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
     }
 }
 
@@ -308,34 +438,50 @@ struct Maps {
 // epilogue warps finish the other slot's previous item.
 __device__ __forceinline__ int64_t pair_tile(int64_t r, int b) { return blockIdx.x + (2 * r + b) * (int64_t)gridDim.x; }
 
-// input tile -> BF16 swizzled A tile (zero beyond the input width and the batch);
-// consecutive threads take consecutive 8-column chunks of a row (coalesced reads)
-__device__ __forceinline__ void stage_input(const Params &P, int64_t t, unsigned char *sA, int et)
+// input tile -> BF16 swizzled A tile (zero beyond the input width and the batch).  A warp
+// takes 16 rows of 64 columns, a lane two neighbouring columns (coalesced reads); in
+// training the lane's 16 rows of a column are 32 consecutive bytes of the transposed
+// input that the first weight gradient reads.
+template <int MODE>
+__device__ __forceinline__ void stage_input(const Params &P, int64_t t, unsigned char *sA, int warp, int lane)
 {
-    const int cpr = P.layer[0].kchunks * KCHUNK / 8;
-    for (int ci = et; ci < TILE_M * cpr; ci += EPI_THREADS) {
-        const int mm = ci / cpr, k0 = (ci - mm * cpr) * 8;
-        const int64_t rr = t * TILE_M + mm;
-        float xv[8];
+    const int m0 = (warp >> 1) * 16;
+    const int64_t r0 = t * TILE_M + m0;
+    for (int k = 64 * (warp & 1) + 2 * lane; k < P.layer[0].kchunks * KCHUNK; k += 128) {
+        uint32_t w[16];
+        const float *x = P.X + r0 * P.in_cols + k;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int k = k0 + e;
-            xv[e] = (rr < P.rows && k < P.in_cols) ? P.X[rr * P.in_cols + k] : 0.f;
+        for (int i = 0; i < 16; ++i) {
+            const bool in = r0 + i < P.rows;
+            if (MODE == TRAIN_BWD) {  // the loss gradient as it is (its width is a multiple of 16)
+                w[i] = in && k < P.layer[0].K ? *(const uint32_t *)(P.dY + (r0 + i) * P.layer[0].K + k) : 0u;
+                continue;
+            }
+            const float a = in && k < P.in_cols ? __ldg(x + (int64_t)i * P.in_cols) : 0.f;
+            const float b = in && k + 1 < P.in_cols ? __ldg(x + (int64_t)i * P.in_cols + 1) : 0.f;
+            w[i] = pack_bf16x2(a, b);
         }
-        const uint4 pk = make_uint4(pack_bf16x2(xv[0], xv[1]), pack_bf16x2(xv[2], xv[3]), pack_bf16x2(xv[4], xv[5]),
-                                    pack_bf16x2(xv[6], xv[7]));
-        *(uint4 *)(sA + sw128_offset(mm, k0)) = pk;
-        if (P.HT[0] && rr < P.rows) {  // training: the input transposed, for the first weight gradient
-            const __nv_bfloat16 *hb = (const __nv_bfloat16 *)&pk;
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (k0 + e < P.layer[0].K) P.HT[0][(int64_t)(k0 + e) * P.ldT + rr] = hb[e];
+        for (int i = 0; i < 16; ++i) *(uint32_t *)(sA + sw128_offset(m0 + i, k)) = w[i];
+        if (MODE == TRAIN_FWD && k < P.layer[0].K && r0 < P.rows) {  // K is a multiple of 16: both columns exist
+            __nv_bfloat16 *h = P.HT[0] + (int64_t)k * P.ldT + r0;
+#pragma unroll
+            for (int c = 0; c < 2; ++c, h += P.ldT) {
+                uint32_t v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = __byte_perm(w[2 * i], w[2 * i + 1], c ? 0x7632 : 0x5410);
+                *(uint4 *)h = make_uint4(v[0], v[1], v[2], v[3]);
+                // ldT is the batch rounded up to 8 rows at least
+                if (r0 + 8 < P.ldT) *((uint4 *)h + 1) = make_uint4(v[4], v[5], v[6], v[7]);
+            }
         }
     }
 }
 
-__global__ void __launch_bounds__(THREADS, 1) k_mlp_fwd_tc(const __grid_constant__ Maps maps, const Params P)
+template <int MODE>
+__global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ Maps maps, const Params P)
 {
+    constexpr bool TRAIN = MODE == TRAIN_FWD;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment for the swizzle atoms
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -347,6 +493,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_fwd_tc(const __grid_constant
     uint64_t *done = a_ready + 2;
     uint32_t *tmem_slot = (uint32_t *)(done + 1);
     __shared__ volatile int s_abort;
+    __shared__ float s_loss[EPI_THREADS / 32];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -435,10 +582,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_fwd_tc(const __grid_constant
         const int q = warp & 3;
         const int part = (warp - 2) >> 2;  // 0..3
         const int m = q * 32 + lane;       // row of the tile owned by this thread
-        const int et = threadIdx.x - 64;
+        const int ew = warp - 2;
+        float loss = 0.f;  // training: this thread's part of the sum of (Y - T)^2
         uint32_t accph[2] = {0u, 0u};
         bool stopped = false;
-        for (int b = 0; b < 2 && b < my; ++b) stage_input(P, pair_tile(0, b), base + b * A_BYTES, et);
+        for (int b = 0; b < 2 && b < my; ++b) stage_input<MODE>(P, pair_tile(0, b), base + b * A_BYTES, ew, lane);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         for (int b = 0; b < 2 && b < my; ++b) mbar_arrive(a_ready + b);
@@ -460,25 +608,92 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_fwd_tc(const __grid_constant
                     const int hw = ((Ly.N / 4 + 31) / 32) * 32;  // columns per part, whole 32-column loads
                     const int cend = min(Ly.N, (part + 1) * hw);
                     const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * MAX_N);
-                    // inference on whole 32-column chunks: the TMEM load of the next
-                    // 16 columns is in flight while the current 16 go through GELU
-                    const bool piped = !last && (Ly.N % 32) == 0 && !P.Z[l];
-                    if (piped && part * hw < cend) {
+                    // hidden layers of whole 32-column chunks (training has no others): the
+                    // TMEM load and the biases of the next 16 columns are in flight while
+                    // the current 16 go through GELU
+                    const bool piped = MODE == TRAIN_BWD || (!last && (TRAIN || (Ly.N % 32) == 0));
+                    if (MODE == TRAIN_BWD) {  // as below, with the pre-activations instead of the biases
+                        if (part * hw < cend) {
+                            uint32_t ra[16], rb[16];
+                            uint4 za0, za1, zb0, zb1;
+                            const bool in = row < P.rows;
+                            auto load_z = [&](int c, uint4 &a, uint4 &b) {
+                                const uint4 *zr = (const uint4 *)(P.Z[l] + row * Ly.N + c);
+                                a = in ? __ldg(zr) : make_uint4(0u, 0u, 0u, 0u);
+                                b = in ? __ldg(zr + 1) : make_uint4(0u, 0u, 0u, 0u);
+                            };
+                            __syncwarp();
+                            tmem_ld16_issue(tacc + (uint32_t)(part * hw), ra);
+                            load_z(part * hw, za0, za1);
+                            tmem_wait16(ra);
+                            for (int c0 = part * hw; c0 < cend; c0 += 32) {
+                                __syncwarp();
+                                tmem_ld16_issue(tacc + (uint32_t)(c0 + 16), rb);
+                                load_z(c0 + 16, zb0, zb1);
+                                dgelu16(P, ra, za0, za1, c0, sA, m, l, row, last);
+                                tmem_wait16(rb);
+                                const bool more = c0 + 32 < cend;
+                                if (more) {
+                                    __syncwarp();
+                                    tmem_ld16_issue(tacc + (uint32_t)(c0 + 32), ra);
+                                    load_z(c0 + 32, za0, za1);
+                                }
+                                dgelu16(P, rb, zb0, zb1, c0 + 16, sA, m, l, row, last);
+                                if (more) tmem_wait16(ra);
+                            }
+                        }
+                    } else if (TRAIN && piped) {
+                        // 8 columns at a time, which leaves the registers for the biases ahead;
+                        // 16 pre-activations (32 bytes, a whole sector a lane) are stored together
+                        if (part * hw < cend) {
+                            uint32_t ra[8], rb[8];
+                            float ba[8], bb[8];
+                            __syncwarp();  // tcgen05.ld is warp-collective
+                            tmem_ld8_issue(tacc + (uint32_t)(part * hw), ra);
+                            load_bias(Ly.bias + part * hw, ba);
+                            tmem_wait8(ra);
+                            for (int c0 = part * hw; c0 < cend; c0 += 16) {  // bounds uniform in the warp
+                                uint4 za, zb;
+                                __syncwarp();
+                                tmem_ld8_issue(tacc + (uint32_t)(c0 + 8), rb);
+                                load_bias(Ly.bias + c0 + 8, bb);
+                                epi_train8(ba, ra, c0, sA, m, P, l, row, za);
+                                tmem_wait8(rb);
+                                const bool more = c0 + 16 < cend;
+                                if (more) {
+                                    __syncwarp();
+                                    tmem_ld8_issue(tacc + (uint32_t)(c0 + 16), ra);
+                                    load_bias(Ly.bias + c0 + 16, ba);
+                                }
+                                epi_train8(bb, rb, c0 + 8, sA, m, P, l, row, zb);
+                                if (row < P.rows) {
+                                    uint4 *zp = (uint4 *)(P.Z[l] + row * Ly.N + c0);
+                                    zp[0] = za;
+                                    zp[1] = zb;
+                                }
+                                if (more) tmem_wait8(ra);
+                            }
+                        }
+                    } else if (piped && part * hw < cend) {
                         uint32_t ra[16], rb[16];
+                        float ba[16], bb[16];
                         __syncwarp();  // tcgen05.ld is warp-collective
                         tmem_ld16_issue(tacc + (uint32_t)(part * hw), ra);
+                        load_bias(Ly.bias + part * hw, ba);
                         tmem_wait16(ra);
                         for (int c0 = part * hw; c0 < cend; c0 += 32) {  // bounds uniform in the warp
                             __syncwarp();
                             tmem_ld16_issue(tacc + (uint32_t)(c0 + 16), rb);
-                            epi16(Ly.bias, ra, c0, sA, m);
+                            load_bias(Ly.bias + c0 + 16, bb);
+                            epi_hidden(ba, ra, c0, sA, m);
                             tmem_wait16(rb);
                             const bool more = c0 + 32 < cend;
                             if (more) {
                                 __syncwarp();
                                 tmem_ld16_issue(tacc + (uint32_t)(c0 + 32), ra);
+                                load_bias(Ly.bias + c0 + 32, ba);
                             }
-                            epi16(Ly.bias, rb, c0 + 16, sA, m);
+                            epi_hidden(bb, rb, c0 + 16, sA, m);
                             if (more) tmem_wait16(ra);
                         }
                     }
@@ -486,38 +701,28 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_fwd_tc(const __grid_constant
                         float v[32];
                         __syncwarp();  // tcgen05.ld is warp-collective
                         tmem_ld32(tacc + (uint32_t)c0, v);
-                        if (!last && c0 + 32 <= Ly.N) {
-                            // a whole chunk: its 32 biases in 8 vector loads (the bias
-                            // array is 128-byte aligned at every 32-column boundary)
-                            float bb[32];
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float4 t4 = __ldg((const float4 *)(Ly.bias + c0) + i);
-                                bb[4 * i] = t4.x; bb[4 * i + 1] = t4.y; bb[4 * i + 2] = t4.z; bb[4 * i + 3] = t4.w;
-                            }
+                        if (TRAIN) {
+                            // the loss and its gradient, row-major and transposed
 #pragma unroll
                             for (int c8 = 0; c8 < 32; c8 += 8) {
+                                if (c0 + c8 >= Ly.N) break;  // uniform
                                 uint32_t pk[4];
-                                float zs[8];
 #pragma unroll
                                 for (int e = 0; e < 8; e += 2) {
-                                    const float2 zz = __fadd2_rn(make_float2(v[c8 + e], v[c8 + e + 1]),
-                                                                 make_float2(bb[c8 + e], bb[c8 + e + 1]));
-                                    zs[e] = zz.x;
-                                    zs[e + 1] = zz.y;
-                                    const float2 g2 = gelu2(zz);
-                                    pk[e / 2] = pack_bf16x2(g2.x, g2.y);
-                                }
-                                *(uint4 *)(sA + sw128_offset(m, c0 + c8)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                                if (P.Z[l] && row < P.rows) {  // training: Z for GELU', H^T for dW
-                                    *(uint4 *)(P.Z[l] + row * Ly.N + c0 + c8) =
-                                        make_uint4(pack_bf16x2(zs[0], zs[1]), pack_bf16x2(zs[2], zs[3]),
-                                                   pack_bf16x2(zs[4], zs[5]), pack_bf16x2(zs[6], zs[7]));
-                                    const __nv_bfloat16 *hb = (const __nv_bfloat16 *)pk;
+                                    float d[2] = {0.f, 0.f};
 #pragma unroll
-                                    for (int e = 0; e < 8; ++e)
-                                        P.HT[l + 1][(int64_t)(c0 + c8 + e) * P.ldT + row] = hb[e];
+                                    for (int u = 0; u < 2; ++u) {
+                                        const int c = c0 + c8 + e + u;
+                                        if (c < P.out_cols && row < P.rows) {
+                                            d[u] = (v[c8 + e + u] + __ldg(Ly.bias + c)) - __ldg(P.T + row * P.out_cols + c);
+                                            loss += d[u] * d[u];
+                                        }
+                                    }
+                                    pk[e / 2] = pack_bf16x2(d[0] * P.scale, d[1] * P.scale);
+                                    store_pair_T(P.dYT, P.ldT, c0 + c8 + e, row, (row & ~(int64_t)1) < P.rows, pk[e / 2]);
                                 }
+                                if (row < P.rows)
+                                    *(uint4 *)(P.dY + row * Ly.N + c0 + c8) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                             }
                         } else if (!last) {
 #pragma unroll
@@ -545,15 +750,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_fwd_tc(const __grid_constant
                     } else if (2 * (r + 1) + b < my) {
                         // this slot's next tile; the accumulator has been read, and
                         // its last MMAs (which read sA) have completed
-                        stage_input(P, pair_tile(r + 1, b), sA, et);
+                        stage_input<MODE>(P, pair_tile(r + 1, b), sA, ew, lane);
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         mbar_arrive(a_ready + b);
                     }
                 }
+        if (TRAIN) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+            if (lane == 0) s_loss[ew] = loss;
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (TRAIN && threadIdx.x == 0) {
+        float sum = 0.f;
+        for (int w = 0; w < EPI_THREADS / 32; ++w) sum += s_loss[w];
+        P.lpart[blockIdx.x] = sum;
+    }
     __syncwarp();
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * MAX_N));
 }
@@ -580,61 +795,59 @@ encode_fn_t encoder()
 
 }  // namespace
 
-// ---- generic GEMM for training: C[M x N] = A[M x K] * B[N x K]^T ---------------
-// Both operands K-major and fed by TMA (same 128-byte swizzle as above); one
-// 128-row tile of C per CTA and one split of K (blockIdx.y); N <= 256.
-//   GEMM_DGELU:   d = acc * GELU'(z) -> BF16 out[m][n] (ld N) and outT[n][m] (ld ldT)
-//   GEMM_PARTIAL: acc -> FP32 part[split][m][n] (split-K partial sums)
+// ---- weight gradients: C[M x N] = A[M x K] * B[N x K]^T over the batch K ----------
+// Both operands K-major and fed by TMA (same 128-byte swizzle as above).  All layers in
+// one launch: blockIdx.x is one 128-row tile of one layer's C (N <= 256), blockIdx.y one
+// split of the batch, and the splits are as many as give every SM one CTA, so that a
+// layer's FP32 partial sums part[split][m][n] are few (16 splits for the five layers of
+// the surrogate; a launch a layer wanted 76 to fill the SMs, 80 MB of partials to write and
+// read again).  The row sums of A over the split (the bias gradient) go to partb[split][m]:
+// the epilogue warps, idle until the end, read them from the stages.  Bound by the 290 MB
+// of operands it reads at batch 65,536: 52 us, 5.6 TB/s (12 us at batch 4,096).  The nine
+// GEMM launches of the data and weight gradients and the row sums took 348 us (129 us)
+// before; this and the fused data gradients take 181 us (52 us).
 namespace {
 
 constexpr int G_EPI = 256;  // 8 epilogue warps, 2 per TMEM lane quarter
 constexpr int G_THREADS = 64 + G_EPI;
 constexpr int G_A_STAGE = TILE_M * KCHUNK * 2;  // 16 KiB
-enum { GEMM_DGELU = 0, GEMM_PARTIAL = 1 };
+constexpr int G_STAGES = 4;
+constexpr int G_SUM_WARPS = 4;                  // warps that also read the A stages
 
-struct GemmP {
-    int M, N, kchunks, kcs;   // kcs: K chunks per split
-    int mode;
-    int64_t m_valid;          // rows of C that exist
-    const __nv_bfloat16 *z;   // DGELU: pre-activation [M x N], BF16
-    __nv_bfloat16 *out, *outT;
-    int64_t ldT;
-    float *part;              // PARTIAL
+struct DwLayer {
+    CUtensorMap ma, mb;
+    int M, N;            // rows of C that exist, columns
+    int tile0;           // the layer's first tile of 128 rows
+    float *part, *partb;
+};
+struct DwArgs {
+    DwLayer l[MAX_LAYERS];
+    int L, kchunks, kcs;  // kcs: K chunks per split
     unsigned *err;
 };
 
-// GELU'(z) = Phi(z) + z phi(z); Phi from the Abramowitz-Stegun erf of gelu(),
-// and exp(-z^2/2) is the exp(-x^2) of that erf
-__device__ __forceinline__ float gelu_grad(float z)
+__global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ DwArgs A)
 {
-    const float x = fabsf(z) * 0.70710678118654752f;
-    const float t = rcp_approx(fmaf(0.3275911f, x, 1.0f));
-    const float poly =
-        t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f), 0.254829592f);
-    const float ex = ex2_approx(-1.4426950408889634f * x * x);
-    const float e = 1.0f - poly * ex;
-    return 0.5f * (1.0f + copysignf(e, z)) + z * ex * 0.3989422804014327f;
-}
-
-__global__ void __launch_bounds__(G_THREADS, 1) k_gemm_tc(const __grid_constant__ CUtensorMap ma,
-                                                          const __grid_constant__ CUtensorMap mb, const GemmP P)
-{
+    constexpr int S = G_STAGES;
+    int layer = 0;
+    while (layer + 1 < A.L && (int)blockIdx.x >= A.l[layer + 1].tile0) ++layer;
+    const DwLayer &P = A.l[layer];
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char *sA = base;                                  // STAGES x 16 KiB
-    unsigned char *sB = base + STAGES * G_A_STAGE;             // STAGES x 32 KiB
-    uint64_t *full = (uint64_t *)(sB + STAGES * W_STAGE_BYTES);
-    uint64_t *empty = full + STAGES;
-    uint64_t *acc_full = empty + STAGES;
+    unsigned char *sA = base;                      // S x 16 KiB
+    unsigned char *sB = base + S * G_A_STAGE;      // S x 32 KiB
+    uint64_t *full = (uint64_t *)(sB + S * W_STAGE_BYTES);
+    uint64_t *empty = full + S;
+    uint64_t *acc_full = empty + S;
     uint64_t *done = acc_full + 1;
     uint32_t *tmem_slot = (uint32_t *)(done + 1);
     __shared__ volatile int s_abort;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int q = 0; q < STAGES; ++q) {
+        for (int q = 0; q < S; ++q) {
             mbar_init(full + q, 1);
-            mbar_init(empty + q, 1);
+            mbar_init(empty + q, 1 + G_SUM_WARPS);
         }
         mbar_init(acc_full, 1);
         mbar_init(done, 1);
@@ -650,25 +863,25 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_gemm_tc(const __grid_constant_
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
-    const int m0 = blockIdx.x * TILE_M;
-    const int kc0 = blockIdx.y * P.kcs, kc1 = min(P.kchunks, kc0 + P.kcs);
+    const int m0 = ((int)blockIdx.x - P.tile0) * TILE_M;
+    const int kc0 = blockIdx.y * A.kcs, kc1 = min(A.kchunks, kc0 + A.kcs);
 
     if (warp == 0) {
         if (lane == 0) {
             int s = 0;
             uint32_t ph = 0;
-            int last_ph[STAGES];
-            for (int q = 0; q < STAGES; ++q) last_ph[q] = -1;
-            for (int kc = kc0; kc < kc1; ++kc) {
-                if (!mbar_wait(empty + s, ph ^ 1)) { atomicOr(P.err, 1u); s_abort = 1; break; }
+            int last_ph[S];
+            for (int q = 0; q < S; ++q) last_ph[q] = -1;
+            for (int kc = kc0; kc < kc1 && !s_abort; ++kc) {
+                if (!mbar_wait(empty + s, ph ^ 1)) { atomicOr(A.err, 1u); s_abort = 1; break; }
                 mbar_expect_tx(full + s, (uint32_t)(G_A_STAGE + P.N * KCHUNK * 2));
-                tma_load_2d(sA + s * G_A_STAGE, &ma, full + s, kc * KCHUNK, m0);
-                tma_load_2d(sB + s * W_STAGE_BYTES, &mb, full + s, kc * KCHUNK, 0);
+                tma_load_2d(sA + s * G_A_STAGE, &P.ma, full + s, kc * KCHUNK, m0);
+                tma_load_2d(sB + s * W_STAGE_BYTES, &P.mb, full + s, kc * KCHUNK, 0);
                 last_ph[s] = (int)ph;
-                if (++s == STAGES) { s = 0; ph ^= 1; }
+                if (++s == S) { s = 0; ph ^= 1; }
             }
-            for (int q = 0; q < STAGES; ++q)
-                if (last_ph[q] >= 0 && !mbar_wait(full + q, (uint32_t)last_ph[q])) atomicOr(P.err, 1u);
+            for (int q = 0; q < S; ++q)
+                if (last_ph[q] >= 0 && !mbar_wait(full + q, (uint32_t)last_ph[q])) atomicOr(A.err, 1u);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -676,7 +889,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_gemm_tc(const __grid_constant_
             uint32_t ph = 0;
             const uint32_t idesc = idesc_bf16(TILE_M, P.N);
             for (int kc = kc0; kc < kc1 && !s_abort; ++kc) {
-                if (!mbar_wait(full + s, ph)) { atomicOr(P.err, 1u); s_abort = 1; break; }
+                if (!mbar_wait(full + s, ph)) { atomicOr(A.err, 1u); s_abort = 1; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t a0 = smem_u32(sA + s * G_A_STAGE);
                 const uint32_t b0 = smem_u32(sB + s * W_STAGE_BYTES);
@@ -684,56 +897,60 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_gemm_tc(const __grid_constant_
                 for (int kk = 0; kk < KCHUNK / 16; ++kk)
                     mma_bf16(tmem, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), idesc, (kc != kc0 || kk != 0));
                 mma_commit(empty + s);
-                if (++s == STAGES) { s = 0; ph ^= 1; }
+                if (++s == S) { s = 0; ph ^= 1; }
             }
             mma_commit(acc_full);
             mma_commit(done);
-            if (!mbar_wait(done, 0)) atomicOr(P.err, 1u);
+            if (!mbar_wait(done, 0)) atomicOr(A.err, 1u);
         }
     } else {
         const int q = warp & 3;
         const int part = (warp - 2) >> 2;  // 0..1
         const int m = q * 32 + lane;
         const int64_t row = (int64_t)m0 + m;
+        if (part == 0) {
+            // row sums of A: this thread's row of every stage (128 swizzled bytes)
+            int s = 0;
+            uint32_t ph = 0;
+            float sum = 0.f;
+            for (int kc = kc0; kc < kc1; ++kc) {
+                const bool ok = mbar_wait(full + s, ph);
+                if (!ok) { atomicOr(A.err, 1u); s_abort = 1; }
+                if (__any_sync(0xffffffffu, !ok || s_abort)) break;
+                const unsigned char *a = sA + s * G_A_STAGE + (m >> 3) * 1024 + (m & 7) * 128;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint4 w = *(const uint4 *)(a + ((c ^ (m & 7)) << 4));
+                    const uint32_t h[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 f = __bfloat1622float2(*(const __nv_bfloat162 *)&h[e]);
+                        sum += f.x + f.y;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty + s);
+                if (++s == S) { s = 0; ph ^= 1; }
+            }
+            if (row < P.M) P.partb[(int64_t)blockIdx.y * P.M + row] = sum;
+        }
         __syncwarp();
         const bool ok = mbar_wait(acc_full, 0);
-        if (!ok) { atomicOr(P.err, 1u); s_abort = 1; }
+        if (!ok) { atomicOr(A.err, 1u); s_abort = 1; }
         if (!__any_sync(0xffffffffu, !ok || s_abort)) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int hw = ((P.N / 2 + 31) / 32) * 32;
             const int cend = min(P.N, (part + 1) * hw);
+            const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16);
             for (int c0 = part * hw; c0 < cend; c0 += 32) {
                 float v[32];
                 __syncwarp();
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
-                if (row >= P.m_valid) continue;
-                if (P.mode == GEMM_PARTIAL) {
-                    float *dst = P.part + ((int64_t)blockIdx.y * P.M + row) * P.N + c0;
+                tmem_ld32(tacc + (uint32_t)c0, v);
+                if (row >= P.M) continue;
+                float *dst = P.part + ((int64_t)blockIdx.y * P.M + row) * P.N + c0;
 #pragma unroll
-                    for (int e = 0; e < 32; e += 4)
-                        if (c0 + e < P.N) *(float4 *)(dst + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-                } else {
-                    const __nv_bfloat16 *zr = P.z + row * P.N + c0;
-#pragma unroll
-                    for (int e = 0; e < 32; e += 8) {
-                        if (c0 + e >= P.N) break;
-                        const uint4 zw = *(const uint4 *)(zr + e);  // 8 BF16 pre-activations
-                        const float2 z01 = __bfloat1622float2(*(const __nv_bfloat162 *)&zw.x);
-                        const float2 z23 = __bfloat1622float2(*(const __nv_bfloat162 *)&zw.y);
-                        const float2 z45 = __bfloat1622float2(*(const __nv_bfloat162 *)&zw.z);
-                        const float2 z67 = __bfloat1622float2(*(const __nv_bfloat162 *)&zw.w);
-                        const float d0 = v[e] * gelu_grad(z01.x), d1 = v[e + 1] * gelu_grad(z01.y);
-                        const float d2 = v[e + 2] * gelu_grad(z23.x), d3 = v[e + 3] * gelu_grad(z23.y);
-                        const float d4 = v[e + 4] * gelu_grad(z45.x), d5 = v[e + 5] * gelu_grad(z45.y);
-                        const float d6 = v[e + 6] * gelu_grad(z67.x), d7 = v[e + 7] * gelu_grad(z67.y);
-                        const uint4 pk = make_uint4(pack_bf16x2(d0, d1), pack_bf16x2(d2, d3), pack_bf16x2(d4, d5),
-                                                    pack_bf16x2(d6, d7));
-                        *(uint4 *)(P.out + row * P.N + c0 + e) = pk;
-                        const __nv_bfloat16 *hb = (const __nv_bfloat16 *)&pk;
-#pragma unroll
-                        for (int w = 0; w < 8; ++w) P.outT[(int64_t)(c0 + e + w) * P.ldT + row] = hb[w];
-                    }
-                }
+                for (int e = 0; e < 32; e += 4)
+                    if (c0 + e < P.N) *(float4 *)(dst + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
             }
         }
     }
@@ -757,148 +974,153 @@ bool kmajor_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, i
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-size_t gemm_tc_smem() { return 1024 + STAGES * (G_A_STAGE + W_STAGE_BYTES) + 128; }
-
-int gemm_tc(const GemmP &P0, const void *A, int64_t a_rows, int64_t a_cols, int64_t a_ld, const void *B,
-            int64_t b_ld, int splits, int device, cudaStream_t st)
-{
-    GemmP P = P0;
-    if (P.N < 16 || P.N > MAX_N || P.N % 16 || splits < 1) return -1;
-    CUtensorMap ma, mb;
-    if (!kmajor_map(&ma, A, a_rows, a_cols, a_ld, TILE_M) || !kmajor_map(&mb, B, P.N, a_cols, b_ld, P.N)) return -1;
-    static bool configured = false;
-    if (!configured) {
-        cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_tc_smem());
-        configured = true;
-    }
-    const dim3 grid((unsigned)((P.M + TILE_M - 1) / TILE_M), (unsigned)splits);
-    k_gemm_tc<<<grid, G_THREADS, gemm_tc_smem(), st>>>(ma, mb, P);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
 }  // namespace
 
-// dZ_prev = (dZ * W) . GELU'(Z): A = dZ [rows x K] (ld K), B = W^T [N x K] (ld K),
-// z = Z [rows x N]; writes out [rows x N] and outT [N x ldT].  N <= 256.
-int mlp_dgelu_tc(const void *dZ, const void *WT, const void *z, int64_t rows, int N, int K, void *out, void *outT,
-                 int64_t ldT, unsigned *err, int device, cudaStream_t st)
+// Splits of the batch for the weight gradients of layers with `tiles` 128-row tiles in
+// all: one CTA an SM, at least 4 chunks of 64 samples a split (below that the partial sums
+// cost more than the GEMM), no split without work.
+static int dw_splits(int64_t rows, int tiles, int device, int *kcs)
 {
-    GemmP P;
-    memset(&P, 0, sizeof(P));
-    P.M = (int)((rows + TILE_M - 1) / TILE_M) * TILE_M;
-    P.N = N;
-    P.kchunks = (K + KCHUNK - 1) / KCHUNK;
-    P.kcs = P.kchunks;
-    P.mode = GEMM_DGELU;
-    P.m_valid = rows;
-    P.z = (const __nv_bfloat16 *)z;
-    P.out = (__nv_bfloat16 *)out;
-    P.outT = (__nv_bfloat16 *)outT;
-    P.ldT = ldT;
-    P.err = err;
-    return gemm_tc(P, dZ, rows, K, K, WT, K, 1, device, st);
+    int sms = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    const int kchunks = (int)((rows + KCHUNK - 1) / KCHUNK), most = std::max(1, sms / tiles);
+    *kcs = std::max(4, (kchunks + most - 1) / most);
+    return (kchunks + *kcs - 1) / *kcs;
+}
+static int dw_tiles(int L, const int *pad)
+{
+    int t = 0;
+    for (int l = 0; l < L; ++l) t += (pad[l + 1] + TILE_M - 1) / TILE_M;
+    return t;
+}
+int mlp_dw_splits(int L, const int *pad, int64_t rows, int device)
+{
+    int kcs;
+    return dw_splits(rows, dw_tiles(L, pad), device, &kcs);
 }
 
-// split-K partials of dW = dZ^T H: A = dZ^T [M x rows] (ld ldT), B = H^T [N x rows]
-// (ld ldT); part [splits x M x N] FP32.  Returns the number of splits used
-// (<= 0 on failure).
-int mlp_dw_tc(const void *dZT, const void *HT, int64_t rows, int64_t ldT, int M, int N, float *part, int max_splits,
-              unsigned *err, int device, cudaStream_t st)
+int mlp_dw_tc(int L, const int *pad, void *const *dZT, void *const *HT, int64_t rows, int64_t ldT, float *const *part,
+              float *const *partb, unsigned *err, int device, cudaStream_t st)
 {
-    GemmP P;
-    memset(&P, 0, sizeof(P));
-    P.M = M;
-    P.N = N;
-    P.kchunks = (int)((rows + KCHUNK - 1) / KCHUNK);
-    const int mt = (M + TILE_M - 1) / TILE_M;
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    int splits = std::max(1, std::min(max_splits, sms / std::max(1, mt)));
-    P.kcs = (P.kchunks + splits - 1) / splits;
-    splits = (P.kchunks + P.kcs - 1) / P.kcs;  // no empty split
-    P.mode = GEMM_PARTIAL;
-    P.m_valid = M;
-    P.part = part;
-    P.err = err;
-    return gemm_tc(P, dZT, M, rows, ldT, HT, ldT, splits, device, st) == 0 ? splits : -1;
+    constexpr size_t smem = 1024 + G_STAGES * (G_A_STAGE + W_STAGE_BYTES) + 128;
+    DwArgs A;
+    memset(&A, 0, sizeof(A));
+    A.L = L;
+    A.kchunks = (int)((rows + KCHUNK - 1) / KCHUNK);
+    A.err = err;
+    int tiles = 0;
+    for (int l = 0; l < L; ++l) {
+        DwLayer &Y = A.l[l];
+        Y.M = pad[l + 1];
+        Y.N = pad[l];
+        if (Y.N < 16 || Y.N > MAX_N || Y.N % 16) return -1;
+        Y.tile0 = tiles;
+        tiles += (Y.M + TILE_M - 1) / TILE_M;
+        Y.part = part[l];
+        Y.partb = partb[l];
+        if (!kmajor_map(&Y.ma, dZT[l], Y.M, rows, ldT, TILE_M) || !kmajor_map(&Y.mb, HT[l], Y.N, rows, ldT, Y.N)) return -1;
+    }
+    const int splits = dw_splits(rows, tiles, device, &A.kcs);
+    static bool configured = false;
+    if (!configured) {
+        cudaFuncSetAttribute(k_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        configured = true;
+    }
+    k_dw_tc<<<dim3((unsigned)tiles, (unsigned)splits), G_THREADS, smem, st>>>(A);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 size_t mlp_tc_smem() { return 1024 + 2 * A_BYTES + STAGES * W_STAGE_BYTES + 256; }
 
-// Forward of an MLP whose layers all fit the fused kernel (K, N <= 256).
-// W[l]: padded BF16 weights [pad_out x pad_in] row-major; bias[l]: pad_out
-// floats.  Returns 0 on success, -1 if the shape is unsupported or the tensor
-// maps cannot be made (the caller then uses the mma.sync kernels).
-// Training forward: the same kernel also stores Z[l] (BF16 [rows x pad[l+1]],
-// hidden layers) and HT[l] (BF16 [pad[l] x ldT], every layer's input
-// transposed).  Hidden widths must be multiples of 32.
-int mlp_forward_train_tc(int L, const int *dims, const int *pad, void *const *W, const float *const *bias,
-                         const float *X, int64_t rows, float *Y, void *const *Z, void *const *HT, int64_t ldT,
-                         unsigned *err, int device, cudaStream_t st);
+namespace {
 
-int mlp_forward_tc(int L, const int *dims, const int *pad, void *const *W, const float *const *bias, const float *X,
-                   int64_t rows, float *Y, unsigned *err, int device, cudaStream_t st)
+// Checks and fills what every mode of the fused kernel needs: layer i takes pad[i] columns
+// to pad[i + 1] with the weights W[i] [pad[i + 1] x pad[i]] (BF16, row-major).
+bool fused_setup(int L, const int *pad, void *const *W, int64_t rows, unsigned *err, int device, Maps &maps, Params &P)
 {
-    return mlp_forward_train_tc(L, dims, pad, W, bias, X, rows, Y, nullptr, nullptr, 0, err, device, st);
-}
-
-int mlp_forward_train_tc(int L, const int *dims, const int *pad, void *const *W, const float *const *bias,
-                         const float *X, int64_t rows, float *Y, void *const *Z, void *const *HT, int64_t ldT,
-                         unsigned *err, int device, cudaStream_t st)
-{
-    if (L < 1 || L > MAX_LAYERS || rows < 1) return -1;
+    if (L < 1 || L > MAX_LAYERS || rows < 1) return false;
     for (int l = 0; l < L; ++l)
-        if (pad[l] > MAX_K || pad[l + 1] > MAX_N || pad[l + 1] % 16 != 0) return -1;
-    if (Z)
-        for (int l = 0; l + 1 < L; ++l)
-            if (pad[l + 1] % 32 != 0) return -1;
+        if (pad[l] > MAX_K || pad[l + 1] > MAX_N || pad[l + 1] % 16 != 0) return false;
     int major = 0;
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
-    if (major < 10) return -1;
-    encode_fn_t enc = encoder();
-    if (!enc) return -1;
-    Maps maps;
+    if (major < 10 || !encoder()) return false;
     memset(&maps, 0, sizeof(maps));
-    Params P;
     memset(&P, 0, sizeof(P));
     P.L = L;
     for (int l = 0; l < L; ++l) {
-        const cuuint64_t gdim[2] = {(cuuint64_t)pad[l], (cuuint64_t)pad[l + 1]};
-        const cuuint64_t gstride[1] = {(cuuint64_t)pad[l] * 2};
-        const cuuint32_t box[2] = {(cuuint32_t)KCHUNK, (cuuint32_t)pad[l + 1]};
-        const cuuint32_t estr[2] = {1, 1};
-        if (enc(&maps.m[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W[l], gdim, gstride, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return -1;
+        if (!kmajor_map(&maps.m[l], W[l], pad[l + 1], pad[l], pad[l], pad[l + 1])) return false;
         P.layer[l].K = pad[l];
         P.layer[l].N = pad[l + 1];
         P.layer[l].kchunks = (pad[l] + KCHUNK - 1) / KCHUNK;
-        P.layer[l].bias = bias[l];
     }
-    P.X = X;
-    P.in_cols = dims[0];
-    P.Y = Y;
-    P.out_cols = dims[L];
     P.rows = rows;
     P.err = err;
-    if (Z) {
-        for (int l = 0; l < L; ++l) {
-            P.Z[l] = (l + 1 < L) ? (__nv_bfloat16 *)Z[l] : nullptr;
-            P.HT[l] = (__nv_bfloat16 *)HT[l];
-        }
-        P.ldT = ldT;
-    }
+    return true;
+}
+
+// Returns the number of CTAs, or -1.
+template <int MODE>
+int fused_launch(const Maps &maps, const Params &P, int device, cudaStream_t st)
+{
     const size_t smem = mlp_tc_smem();
     static bool configured = false;
     if (!configured) {
-        cudaFuncSetAttribute(k_mlp_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_mlp_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         configured = true;
     }
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    const int64_t ntiles = (rows + TILE_M - 1) / TILE_M;
+    const int64_t ntiles = (P.rows + TILE_M - 1) / TILE_M;
     const int grid = (int)std::min<int64_t>(ntiles, (int64_t)sms);
-    k_mlp_fwd_tc<<<grid, THREADS, smem, st>>>(maps, P);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    k_mlp_tc<MODE><<<grid, THREADS, smem, st>>>(maps, P);
+    return cudaGetLastError() == cudaSuccess ? grid : -1;
+}
+
+}  // namespace
+
+int mlp_forward_tc(int L, const int *dims, const int *pad, void *const *W, const float *const *bias, const float *X,
+                   int64_t rows, float *Y, const MlpTrain *tr, unsigned *err, int device, cudaStream_t st)
+{
+    Maps maps;
+    Params P;
+    if (!fused_setup(L, pad, W, rows, err, device, maps, P)) return -1;
+    for (int l = 0; l < L; ++l) P.layer[l].bias = bias[l];
+    P.X = X;
+    P.in_cols = dims[0];
+    P.Y = Y;
+    P.out_cols = dims[L];
+    if (!tr) return fused_launch<INFER>(maps, P, device, st);
+    for (int l = 0; l < L; ++l) {
+        if (l + 1 < L && pad[l + 1] % 32 != 0) return -1;
+        P.Z[l] = (l + 1 < L) ? (__nv_bfloat16 *)tr->Z[l] : nullptr;
+        P.HT[l] = (__nv_bfloat16 *)tr->HT[l];
+    }
+    P.ldT = tr->ldT;
+    P.T = tr->T;
+    P.scale = tr->scale;
+    P.dY = (__nv_bfloat16 *)tr->dY;
+    P.dYT = (__nv_bfloat16 *)tr->dYT;
+    P.lpart = tr->lpart;
+    return fused_launch<TRAIN_FWD>(maps, P, device, st);
+}
+
+int mlp_backward_tc(int L, const int *pad, void *const *WT, const MlpTrain *tr, void *const *dZT, int64_t rows,
+                    unsigned *err, int device, cudaStream_t st)
+{
+    if (L < 2) return 0;
+    int rpad[MAX_LAYERS + 1];
+    void *W[MAX_LAYERS];
+    for (int i = 0; i < L; ++i) rpad[i] = pad[L - i];  // layer i: dZ_{L-1-i} [pad[L - i]] -> dZ_{L-2-i} [pad[L - 1 - i]]
+    for (int i = 0; i + 1 < L; ++i) W[i] = WT[L - 1 - i];
+    Maps maps;
+    Params P;
+    if (!fused_setup(L - 1, rpad, W, rows, err, device, maps, P)) return -1;
+    for (int i = 0; i + 1 < L; ++i) {
+        if (rpad[i + 1] % 32 != 0) return -1;
+        P.Z[i] = (__nv_bfloat16 *)tr->Z[L - 2 - i];
+        P.HT[i] = (__nv_bfloat16 *)dZT[L - 2 - i];
+    }
+    P.ldT = tr->ldT;
+    P.dY = (__nv_bfloat16 *)tr->dY;
+    return fused_launch<TRAIN_BWD>(maps, P, device, st);
 }
