@@ -217,8 +217,9 @@ pd_status pd_stable_dt(pd_ctx *ctx, double *dt_crit);
  * force.  Captured and replayed as CUDA graphs.  Blocks until done.  The
  * steps run in segments of 2 graph chunks (up to 128 steps; a chunk is the
  * largest multiple of the rebuild period within graph_chunk); a segment
- * whose contact list went stale or overflowed is rolled back to its own start
- * and rerun with a shorter rebuild period or larger lists.  The contact list is
+ * whose contact list went stale goes on from the step it went stale in, with a
+ * shorter rebuild period, and one whose list overflowed is rolled back to its own
+ * start and rerun with larger lists.  The contact list is
  * rebuilt often enough for the fastest node (or wall) to gain 50% in speed
  * (150% while speeds are growing).  A call of one step rebuilds it only when the
  * list on the device no longer holds for the current state (not built since the
@@ -356,8 +357,9 @@ pd_status pd_set_profiling(pd_ctx *ctx, int on);
 pd_status pd_last_step_stats(pd_ctx *ctx, double *ms_force, double *ms_total, int64_t *launches);
 
 /* Counters since pd_create (each pointer nullable): steps taken, contact-list
- * rebuilds of those steps, and segments rolled back and rerun because the list
- * went stale or overflowed (see pd_step). */
+ * rebuilds of those steps, and interruptions of segments because the list went
+ * stale (taken up again where they stopped) or overflowed (rolled back and rerun;
+ * see pd_step). */
 pd_status pd_step_counters(pd_ctx *ctx, int64_t *steps, int64_t *rebuilds, int64_t *rollbacks);
 
 /* pd_set_state / pd_set_state_packed calls since pd_create (each pointer

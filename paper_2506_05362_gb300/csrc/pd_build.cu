@@ -425,6 +425,8 @@ __global__ void __launch_bounds__(128) k_cand(const int32_t *__restrict__ grain,
                                               unsigned *err, double *disp, int *stale)
 {
     __shared__ unsigned long long s_base;
+    // a segment whose list went stale takes no further step (written by earlier kernels only)
+    if (*(volatile const unsigned *)err & PDE_SKIN) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *disp = 0.0;
         *stale = 0;

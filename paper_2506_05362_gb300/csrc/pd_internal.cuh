@@ -105,7 +105,7 @@ struct StepParams {
     double *partials;              // gridDim.x * PART_STRIDE
     unsigned *counter;
     unsigned *vmax_bits;           // max |v|^2 of the step as FP32 bits (atomicMax)
-    unsigned *err;
+    unsigned *err;                 // error bits; [1]: steps taken since it was cleared
     double *react;                 // nw*3 final wall reactions
     double *impulse;               // nw*3 sum over steps of dt * react (not in MODE_FORCES)
     double beta_d;                 // normal contact damping (0 = none)

@@ -104,12 +104,12 @@ __device__ __forceinline__ double group_sum(double v)
     return v;
 }
 
-// A step whose segment will be rolled back anyway: the contact list went stale in
-// an earlier step (the mark is in *p.stale, or in the error word of an earlier
-// kernel), or a rebuild overflowed the candidate list.  Every block reads values
-// that only earlier kernels wrote (block 0 of k_step adds PDE_SKIN to the error
-// word only when *p.stale is set), so all blocks of a launch agree and return
-// together; the rest of the segment then costs little more than its launches.
+// A step that its segment does not take: the contact list went stale in an earlier step
+// (the mark is in *p.stale, or in the error word of an earlier kernel), or a rebuild
+// overflowed the candidate list.  Every block reads values that only earlier kernels
+// wrote (block 0 of k_step adds PDE_SKIN to the error word only when *p.stale is set), so
+// all blocks of a launch agree and return together; the rest of the segment then costs
+// little more than its launches and leaves the state of the last step taken.
 __device__ __forceinline__ bool segment_doomed(const StepParams &p)
 {
     return (p.contact && *(volatile const int *)p.stale) ||
@@ -1158,6 +1158,7 @@ __device__ __forceinline__ void block_finish(const StepParams &p, double (*s_rea
         }
     }
     if (threadIdx.x == 0) {
+        if (p.mode != MODE_FORCES) ++p.err[1];  // steps taken
         const double vm = (double)__uint_as_float(atomicExch(p.vmax_bits, 0u));  // max |v|^2, reset
         if (p.mode == MODE_FULL) {
             const double dsp = *p.disp + p.dt * sqrt(vm);
@@ -1371,6 +1372,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2)
         s_disp = *pa.disp;
         if (blockIdx.x == 0 && pa.contact && *pa.stale) atomicOr(pa.err, (unsigned)PDE_SKIN);
     }
+    if (segment_doomed(pa)) return;  // uniform over the grid: read before the first barrier
     __syncthreads();
     unsigned nbar = 0;
     int done = 0;
@@ -1392,6 +1394,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2)
     if (blockIdx.x == 0) {
         if ((int)threadIdx.x < ncomp) pa.wall_pos[threadIdx.x] = s_wall[threadIdx.x];
         if (threadIdx.x == 0 && done > 0) {
+            pa.err[1] += done;
             *pa.disp = s_disp;
             if (2.0 * s_disp >= pa.skin) *pa.stale = 1;
         }
@@ -1525,6 +1528,8 @@ __global__ void k_drift(const StepParams p)
 {
     __shared__ float s_m[8];
     __shared__ bool s_last;
+    // a chunk after the one whose list went stale or overflowed; written by earlier kernels only
+    if (*(volatile const unsigned *)p.err & (PDE_SKIN | PDE_CAPACITY)) return;
     const double hdt = 0.5 * p.dt;
     float vm = 0.f;  // largest |v|^2 after the half kick (FP32, as the fused steps keep it)
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n;

@@ -506,7 +506,7 @@ class Context:
         return pd_state_counters(self.h)
 
     def step_counters(self):
-        """(steps, contact-list rebuilds, rolled-back segments) since creation."""
+        """(steps, contact-list rebuilds, interrupted segments) since creation."""
         return pd_step_counters(self.h)
 
     def close(self):
