@@ -582,7 +582,7 @@ static pd_status create_impl(pd_ctx *c, const double *x, const double *vol, cons
     c->blocks_cap = 0;
     for (int g : {4, 8, 16, 32}) c->blocks_cap = std::max(c->blocks_cap, step_blocks(g, c->opt.device, mixed, false, 0));
     ALLOC(c->partials, double, 2 * (int64_t)c->blocks_cap * PART_STRIDE);  // two step parities (multi-step kernel)
-    ALLOC(c->gbar, unsigned, 1);
+    ALLOC(c->gbar, unsigned, 4);
     ALLOC(c->react, double, PD_MAX_WALLS * 3);
     ALLOC(c->disp, double, 1);
     ALLOC(c->wall_pos, double, PD_MAX_WALLS * 9);  // wall points, the wall impulses, the wall normals
@@ -1002,7 +1002,7 @@ static int64_t enqueue_chunk(pd_ctx *c, int steps, int k, int parity, double dt,
             const bool ends = s + run == steps;
             const int full = ends ? run - 1 : run;
             if (full > 1) {
-                cudaMemsetAsync(c->gbar, 0, sizeof(unsigned), c->st);
+                cudaMemsetAsync(c->gbar, 0, 4 * sizeof(unsigned), c->st);
                 StepParams pa = params(c, MODE_FULL, in, dt), pb = params(c, MODE_FULL, in ^ 1, dt);
                 cudaError_t e =
                     launch_persist(pa, pb, full, c->lanes, pgrid, c->gbar, (unsigned)c->opt.barrier_absent, c->st);

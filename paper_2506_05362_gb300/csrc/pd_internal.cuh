@@ -141,7 +141,7 @@ struct StepParams {
     float4 *fup;                   // per row: pass 1's force from the row's own slots
 };
 
-#define PART_STRIDE 20  // 18 reaction components, max|v| (multi-step kernel), spare
+#define PART_STRIDE 20  // 18 reaction components, padded
 #define PD_GL 32        // Gauss-Legendre points of the multi-wall overlap integrals
 
 // Radix sort of (key, value) pairs, LSD 8-bit digits, stable.  bits = number of

@@ -66,6 +66,7 @@ __device__ __forceinline__ void root64(double a, double &l, double &r)
 }
 
 constexpr int STEP_THREADS = 256;
+constexpr unsigned STEP_TOUCH = 0x80000000u;  // beside the error bits of a block: a node of it touches a wall
 // bonds each lane keeps in flight per loop iteration, and the minimum resident
 // blocks per SM the compiler must allow (register budget)
 #ifndef PD_INFLIGHT
@@ -308,6 +309,7 @@ __device__ __forceinline__ unsigned wall_force(const StepParams &p, const double
             }
         }
         ++touching;
+        e |= STEP_TOUCH;
     }
     if (WX && p.wall_overlap && touching >= 2) {
         const double3 o = wall_overlap_terms(wp, p.wall_n, p.gl, p.walls.nw, p.Rc, p.Kn, px, py, pz, vol,
@@ -1146,30 +1148,67 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
 #undef load_u
 }
 
-// Per-block partials and the finish of the step by the last block.  The max |v|
-// bound goes through one atomicMax per block (a max does not depend on order);
-// wall reactions are summed per block in group order, then by the last block
-// with one warp per component, lanes striding over the blocks and a fixed xor
-// butterfly, so the result is bitwise reproducible.  The last block also
-// advances the walls and the skin bookkeeping.
+// A block's part of the step: the wall reactions summed over its groups (a warp per
+// component, lanes striding over the groups, a fixed xor butterfly; zeros if no node
+// touches a wall) to `part`, the largest |v|^2 into *vmax_bits (a max does not depend on
+// order), the error bits.  Adding 64 groups' sums in turn in one thread a component, and as
+// many maxima in another, took a third of a block's fixed cost of 2.8 us.
 template <int GPB>
-__device__ __forceinline__ void block_finish(const StepParams &p, double (*s_react)[PD_MAX_WALLS * 3],
-                                             double *s_vmax, unsigned &s_err, bool &s_last, unsigned err)
+__device__ __forceinline__ void block_partials(const StepParams &p, const double (*s_react)[PD_MAX_WALLS * 3],
+                                               unsigned s_vbits, unsigned s_err, double *part, unsigned *vmax_bits)
 {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ncomp = 3 * p.walls.nw;
+    if (s_err & STEP_TOUCH) {
+        for (int c = warp; c < ncomp; c += STEP_THREADS / 32) {
+            double s = 0.0;
+            for (int g = lane; g < GPB; g += 32) s += s_react[g][c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) part[c] = s;
+        }
+    } else if ((int)threadIdx.x < ncomp) {
+        part[threadIdx.x] = 0.0;
+    }
+    if (threadIdx.x == STEP_THREADS - 1) {
+        if (s_vbits) atomicMax(vmax_bits, s_vbits);
+        if (s_err & ~STEP_TOUCH) atomicOr(p.err, s_err & ~STEP_TOUCH);
+    }
+}
+
+// a lane's largest |v|^2 as FP32 bits (rounded up), and its error bits, into the block's
+template <bool MIXED>
+__device__ __forceinline__ void block_collect(float vmax2f, double vmax2, unsigned err, unsigned &s_vbits,
+                                              unsigned &s_err)
+{
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(MIXED ? vmax2f : __double2float_ru(vmax2)));
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(&s_vbits, m);
     if (err) atomicOr(&s_err, err);
+}
+
+// The wall reactions of one step from the per-block partials: component c in one warp,
+// lanes striding over the blocks (unrolled so that the loads of several blocks' partials
+// are in flight together; the additions keep their order), a fixed xor butterfly, so the
+// result is bitwise reproducible.
+__device__ __forceinline__ void store_reaction(const StepParams &p, int c, double s)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) {
+        p.react[c] = s;
+        if (p.mode != MODE_FORCES) p.impulse[c] = dadd(p.impulse[c], dmul(p.dt, s));
+    }
+}
+
+// The finish of the step by the last block: the wall reactions, the walls' motion and the
+// skin bookkeeping.
+template <int GPB>
+__device__ __forceinline__ void block_finish(const StepParams &p, const double (*s_react)[PD_MAX_WALLS * 3],
+                                             const unsigned &s_vbits, const unsigned &s_err, bool &s_last)
+{
     __syncthreads();
     const int ncomp = 3 * p.walls.nw;
-    double *part = p.partials + (int64_t)blockIdx.x * PART_STRIDE;
-    if ((int)threadIdx.x < ncomp) {
-        double s = 0.0;
-        for (int g = 0; g < GPB; ++g) s += s_react[g][threadIdx.x];
-        part[threadIdx.x] = s;
-    } else if (threadIdx.x == 32) {
-        double m = 0.0;
-        for (int g = 0; g < GPB; ++g) m = fmax(m, s_vmax[g]);
-        if (m > 0.0) atomicMax(p.vmax_bits, __float_as_uint(__double2float_ru(m)));
-        if (s_err) atomicOr(p.err, s_err);
-    }
+    block_partials<GPB>(p, s_react, s_vbits, s_err, p.partials + (int64_t)blockIdx.x * PART_STRIDE, p.vmax_bits);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1180,18 +1219,17 @@ __device__ __forceinline__ void block_finish(const StepParams &p, double (*s_rea
     if (!s_last) return;
     __threadfence();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int c = warp; c < ncomp; c += STEP_THREADS / 32) {
-        double s = 0.0;
-        // unrolled so that the loads of several blocks' partials are in flight
-        // together; the additions keep their order
-#pragma unroll 8
-        for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(p.partials + (int64_t)b * PART_STRIDE + c);
+    constexpr int NW = STEP_THREADS / 32, PER = (3 * PD_MAX_WALLS + NW - 1) / NW;
+    if (warp < ncomp) {
+        double s[PER] = {0.0};
+#pragma unroll 4
+        for (unsigned b = lane; b < gridDim.x; b += 32)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            p.react[c] = s;
-            if (p.mode != MODE_FORCES) p.impulse[c] = dadd(p.impulse[c], dmul(p.dt, s));
-        }
+            for (int q = 0; q < PER; ++q)
+                if (warp + NW * q < ncomp) s[q] += __ldcg(p.partials + (int64_t)b * PART_STRIDE + warp + NW * q);
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (warp + NW * q < ncomp) store_reaction(p, warp + NW * q, s[q]);
     }
     if (threadIdx.x == 0) {
         if (p.mode != MODE_FORCES) ++p.err[1];  // steps taken
@@ -1208,6 +1246,19 @@ __device__ __forceinline__ void block_finish(const StepParams &p, double (*s_rea
     }
 }
 
+// zeros the groups' reactions and the block's maximum and error bits; a barrier must follow
+template <int GPB>
+__device__ __forceinline__ void block_begin(const StepParams &p, double (*s_react)[PD_MAX_WALLS * 3],
+                                            unsigned &s_vbits, unsigned &s_err)
+{
+    if (p.walls.nw)
+        for (int q = threadIdx.x; q < GPB * PD_MAX_WALLS * 3; q += STEP_THREADS) (&s_react[0][0])[q] = 0.0;
+    if (threadIdx.x == 0) {
+        s_vbits = 0u;
+        s_err = 0u;
+    }
+}
+
 // Rows in a grid-stride loop, neighbour records gathered from global memory
 // (FP64 path, and the mixed path without tiles).
 template <int G, bool MIXED, bool WX, bool PAIRS = false>
@@ -1215,19 +1266,13 @@ __global__ void __launch_bounds__(STEP_THREADS, MIXED ? PD_MINB_GLOBAL : 2) k_st
 {
     constexpr int GPB = STEP_THREADS / G;
     __shared__ double s_react[GPB][PD_MAX_WALLS * 3];
-    __shared__ double s_vmax[GPB];
-    __shared__ unsigned s_err;
+    __shared__ unsigned s_vbits, s_err;
     __shared__ bool s_last;
     const int gl = threadIdx.x % G, grp = threadIdx.x / G;
-    if (gl == 0) {
-        for (int q = 0; q < PD_MAX_WALLS * 3; ++q) s_react[grp][q] = 0.0;
-    }
     __shared__ WallF s_wf[PD_MAX_WALLS];
     load_walls_f(p, p.wall_pos, s_wf);
-    if (threadIdx.x == 0) {
-        s_err = 0;
-        if (blockIdx.x == 0 && p.contact && *p.stale) atomicOr(p.err, (unsigned)PDE_SKIN);
-    }
+    block_begin<GPB>(p, s_react, s_vbits, s_err);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && p.contact && *p.stale) atomicOr(p.err, (unsigned)PDE_SKIN);
     if (segment_doomed(p)) return;  // uniform over the grid (see segment_doomed)
     __syncthreads();
     unsigned err = 0;
@@ -1238,8 +1283,8 @@ __global__ void __launch_bounds__(STEP_THREADS, MIXED ? PD_MINB_GLOBAL : 2) k_st
         const int64_t row = r0 + grp;
         process_row<G, MIXED, WX, PAIRS>(p, p.wall_pos, s_wf, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
     }
-    if (gl == 0) s_vmax[grp] = MIXED ? (double)vmax2f : vmax2;
-    block_finish<GPB>(p, s_react, s_vmax, s_err, s_last, err);
+    block_collect<MIXED>(vmax2f, vmax2, err, s_vbits, s_err);
+    block_finish<GPB>(p, s_react, s_vbits, s_err, s_last);
 }
 
 // ---- Several steps in one launch ------------------------------------------------
@@ -1249,8 +1294,8 @@ __global__ void __launch_bounds__(STEP_THREADS, MIXED ? PD_MINB_GLOBAL : 2) k_st
 // so the trajectory is bit for bit that of one launch per step while the launch
 // cost and the gap between launches are paid once per run.  Every block keeps
 // its own copy of the wall positions and of the skin bookkeeping and advances
-// them identically; block 0 alone writes the wall reactions and impulses, and
-// at the end the walls, displacement bound and stale flag.  Even steps use the
+// them identically; the first blocks write the wall reactions and impulses, a
+// component each, block 0 at the end the walls, displacement bound and stale flag.  Even steps use the
 // parameters pa (state buffers in -> out), odd steps pb (out -> in).
 
 constexpr unsigned BAR_ABORT = 0x80000000u;     // set in the barrier word by a block that gave up
@@ -1300,29 +1345,9 @@ __device__ bool grid_barrier(unsigned *bar, unsigned target, unsigned *err, int 
     return *s_ok != 0;
 }
 
-// The wall reactions of one step from the per-block partials (the last-block
-// reduction of block_finish: one warp per component, lanes striding over the
-// blocks, a fixed xor butterfly), written with the impulse by block 0.
-__device__ __forceinline__ void reduce_reactions(const StepParams &p, const double *partials, int nblocks)
-{
-    const int ncomp = 3 * p.walls.nw;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int c = warp; c < ncomp; c += STEP_THREADS / 32) {
-        double s = 0.0;
-#pragma unroll 8
-        for (int b = lane; b < nblocks; b += 32) s += __ldcg(partials + (int64_t)b * PART_STRIDE + c);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            p.react[c] = s;
-            p.impulse[c] = dadd(p.impulse[c], dmul(p.dt, s));
-        }
-    }
-}
-
 template <int G, bool MIXED, bool WX>
 __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsigned *bar, unsigned &nbar, unsigned arrivals,
-                                             double (*s_react)[PD_MAX_WALLS * 3], double *s_vmax, double *s_wall,
+                                             double (*s_react)[PD_MAX_WALLS * 3], double *s_wall, unsigned &s_vbits,
                                              unsigned &s_err, int &s_ok, double &s_disp)
 {
     constexpr int GPB = STEP_THREADS / G;
@@ -1331,11 +1356,9 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
         pair_damping_rows<MIXED>(p, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
         if (!grid_barrier(bar, ++nbar * arrivals, p.err, &s_ok)) return false;
     }
-    if (gl == 0)
-        for (int q = 0; q < PD_MAX_WALLS * 3; ++q) s_react[grp][q] = 0.0;
     __shared__ WallF s_wf[PD_MAX_WALLS];
     load_walls_f(p, s_wall, s_wf);
-    if (threadIdx.x == 0) s_err = 0;
+    block_begin<GPB>(p, s_react, s_vbits, s_err);
     __syncthreads();
     unsigned err = 0;
     double vmax2 = 0.0;
@@ -1345,40 +1368,29 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
         const int64_t row = r0 + grp;
         process_row<G, MIXED, WX, false>(p, s_wall, s_wf, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
     }
-    if (gl == 0) s_vmax[grp] = MIXED ? (double)vmax2f : vmax2;
-    if (err) atomicOr(&s_err, err);
+    block_collect<MIXED>(vmax2f, vmax2, err, s_vbits, s_err);
     __syncthreads();
-    // this block's partials, in the buffer of the step's parity
+    // this block's partials in the buffer of the step's parity, its largest |v|^2 in the
+    // word of the step modulo 3: the next step's word is cleared before this step's barrier,
+    // when every block has read it (two steps ago) and none writes it yet
     double *partials = p.partials + (int64_t)(step & 1) * gridDim.x * PART_STRIDE;
-    double *part = partials + (int64_t)blockIdx.x * PART_STRIDE;
-    const int ncomp = 3 * p.walls.nw;
-    if ((int)threadIdx.x < ncomp) {
-        double sum = 0.0;
-        for (int g = 0; g < GPB; ++g) sum += s_react[g][threadIdx.x];
-        part[threadIdx.x] = sum;
-    } else if (threadIdx.x == 32) {
-        double m = 0.0;
-        for (int g = 0; g < GPB; ++g) m = fmax(m, s_vmax[g]);
-        part[PART_STRIDE - 2] = m > 0.0 ? (double)__double2float_ru(m) : 0.0;
-        if (s_err) atomicOr(p.err, s_err);
-    }
+    unsigned *vmax_bits = bar + 1 + step % 3;
+    block_partials<GPB>(p, s_react, s_vbits, s_err, partials + (int64_t)blockIdx.x * PART_STRIDE, vmax_bits);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile unsigned *)(bar + 1 + (step + 1) % 3) = 0u;
     if (!grid_barrier(bar, ++nbar * arrivals, p.err, &s_ok)) return false;
-    if (blockIdx.x == 0) reduce_reactions(p, partials, gridDim.x);
-    {  // the same bookkeeping in every block: max |v|^2 over the blocks' partials,
-       // read by all threads at once (a max does not depend on the order)
-        double vm = 0.0;
-        for (unsigned b = threadIdx.x; b < gridDim.x; b += STEP_THREADS)
-            vm = fmax(vm, __ldcg(partials + (int64_t)b * PART_STRIDE + PART_STRIDE - 2));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) vm = fmax(vm, __shfl_xor_sync(0xffffffffu, vm, o));
-        if ((threadIdx.x & 31) == 0) s_vmax[threadIdx.x >> 5] = vm;  // s_vmax holds >= 8 entries (G <= 32)
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double m = 0.0;
-            for (int w = 0; w < STEP_THREADS / 32; ++w) m = fmax(m, s_vmax[w]);
-            s_disp = s_disp + p.dt * sqrt(m);
+    const int ncomp = 3 * p.walls.nw;
+    // one block a component, so that none is far behind the others at the next barrier
+    // (block 0 alone took 3 us for twelve of them)
+    if (threadIdx.x < 32)
+        for (int c = blockIdx.x; c < ncomp; c += gridDim.x) {
+            double s = 0.0;
+#pragma unroll 8
+            for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) s += __ldcg(partials + (int64_t)b * PART_STRIDE + c);
+            store_reaction(p, c, s);
         }
-    }
+    // the same bookkeeping in every block
+    if (threadIdx.x == STEP_THREADS - 1)
+        s_disp = s_disp + p.dt * sqrt((double)__uint_as_float(__ldcg(vmax_bits)));
     if ((int)threadIdx.x < ncomp) {
         const int l = threadIdx.x / 3, q = threadIdx.x % 3;
         s_wall[threadIdx.x] = dadd(s_wall[threadIdx.x], dmul(p.dt, p.walls.v[l][q]));
@@ -1397,9 +1409,8 @@ __global__ void __launch_bounds__(STEP_THREADS, 2)
     const unsigned arrivals = gridDim.x + absent;
     constexpr int GPB = STEP_THREADS / G;
     __shared__ double s_react[GPB][PD_MAX_WALLS * 3];
-    __shared__ double s_vmax[GPB];
     __shared__ double s_wall[PD_MAX_WALLS * 3];
-    __shared__ unsigned s_err;
+    __shared__ unsigned s_vbits, s_err;
     __shared__ int s_ok;
     __shared__ double s_disp;
     const int ncomp = 3 * pa.walls.nw;
@@ -1423,7 +1434,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 2)
         // chosen at run time (grid-constant parameters can be addressed)
         const StepParams &p = (st & 1) ? pb : pa;
         const bool ok =
-            persist_step<G, MIXED, WX>(p, st, bar, nbar, arrivals, s_react, s_vmax, s_wall, s_err, s_ok, s_disp);
+            persist_step<G, MIXED, WX>(p, st, bar, nbar, arrivals, s_react, s_wall, s_vbits, s_err, s_ok, s_disp);
         if (!ok) return;
         done = st + 1;
     }
@@ -1449,8 +1460,7 @@ __global__ void __launch_bounds__(STEP_THREADS, PD_MINB_TILED) k_step_tiled(cons
     constexpr int GPB = STEP_THREADS / G;
     extern __shared__ float4 s_rec[];
     __shared__ double s_react[GPB][PD_MAX_WALLS * 3];
-    __shared__ double s_vmax[GPB];
-    __shared__ unsigned s_err;
+    __shared__ unsigned s_vbits, s_err;
     __shared__ bool s_last;
     const int T = p.tile_rows, cap = p.tile_cap;
     float4 *r0s = s_rec, *r1s = r0s + cap, *r2s = r1s + cap, *vhs = r2s + cap, *vls = vhs + T;
@@ -1460,15 +1470,10 @@ __global__ void __launch_bounds__(STEP_THREADS, PD_MINB_TILED) k_step_tiled(cons
     uint16_t *lrs = (uint16_t *)(rps + ((T + 2) & ~1));
     uint16_t *lcs = lrs + ((T + 7) & ~7);
     const int gl = threadIdx.x % G, grp = threadIdx.x / G;
-    if (gl == 0) {
-        for (int q = 0; q < PD_MAX_WALLS * 3; ++q) s_react[grp][q] = 0.0;
-    }
     __shared__ WallF s_wf[PD_MAX_WALLS];
     load_walls_f(p, p.wall_pos, s_wf);
-    if (threadIdx.x == 0) {
-        s_err = 0;
-        if (blockIdx.x == 0 && p.contact && *p.stale) atomicOr(p.err, (unsigned)PDE_SKIN);
-    }
+    block_begin<GPB>(p, s_react, s_vbits, s_err);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && p.contact && *p.stale) atomicOr(p.err, (unsigned)PDE_SKIN);
     if (segment_doomed(p)) return;  // uniform over the grid (see segment_doomed)
     __syncthreads();
     unsigned err = 0;
@@ -1550,8 +1555,8 @@ __global__ void __launch_bounds__(STEP_THREADS, PD_MINB_TILED) k_step_tiled(cons
         }
         __syncthreads();
     }
-    if (gl == 0) s_vmax[grp] = (double)vmax2f;
-    block_finish<GPB>(p, s_react, s_vmax, s_err, s_last, err);
+    block_collect<true>(vmax2f, vmax2, err, s_vbits, s_err);
+    block_finish<GPB>(p, s_react, s_vbits, s_err, s_last);
 }
 
 // First half of a chunk's first step: v += dt/2 a; u^{n+1} = u^n + dt v; walls move.
@@ -1776,7 +1781,7 @@ int persist_blocks(int lanes, int device, bool mixed, bool wx)
 }
 
 // nsteps MODE_FULL steps in one cooperative launch; pa for even steps, pb for odd
-// ones.  bar (one word) must be zero.  Returns the launch status.
+// ones.  bar (four words: the barrier, three maxima) must be zero.  Returns the launch status.
 cudaError_t launch_persist(const StepParams &pa, const StepParams &pb, int nsteps, int lanes, int blocks,
                            unsigned *bar, unsigned absent, cudaStream_t st)
 {
