@@ -665,6 +665,13 @@ static int step_grid(const pd_ctx *c, int lanes)
     return (int)std::min<int64_t>(b, need);
 }
 
+// Whether pd_step runs its steps between rebuilds in one launch of the multi-step
+// kernel: the per-slot global-gather kernels only, not while profiling.
+static bool use_persist(const pd_ctx *c)
+{
+    return c->persist && !c->tiled && !c->pairs && !c->profiling;
+}
+
 static pd_status autotune(pd_ctx *c)
 {
     // time a force evaluation (idempotent at a fixed state) for each lane count of the
@@ -700,7 +707,18 @@ static pd_status autotune(pd_ctx *c)
     // group of fewer lanes shares among more nodes per warp: of the winning kernel,
     // the fewest lanes within 3% of its best force evaluation are taken (on the
     // plate 4 and 8 lanes tie within 0.5% here, and 4 lanes are 4% faster a step).
-    for (int q = 0; q < 4 && cand[q] < bestl; ++q) {
+    // In the mixed multi-step kernel a step of few nodes is one chain of latencies: there
+    // the most lanes whose blocks are all resident are taken, the shortest chain that needs
+    // no second round (us a step at 8 / 16 / 32 lanes; 304 blocks of 256 threads fit: 895
+    // nodes 10.8 / 10.3 / 10.2, 4,139 nodes 12.6 / 10.2 / 11.8, plate of 2,592 11.6 / 8.8 /
+    // 10.2, 7,123 nodes 12.2 / 13.6 / 15.0).  Where only 4 lanes fit, and in FP64, which the
+    // FP64 pipe bounds, the times above decide.
+    int fit = 0;
+    if (mixed && use_persist(c))
+        for (int l : {8, 16, 32})
+            if ((c->n + 256 / l - 1) / (256 / l) <= persist_blocks(l, c->opt.device, mixed, false)) fit = l;
+    if (fit) bestl = fit;
+    for (int q = 0; q < 4 && !fit && cand[q] < bestl; ++q) {
         const double t = c->tune_ms[4 * kind + q];
         if (t > 0 && t <= 1.03 * best) { bestl = cand[q]; break; }
     }
@@ -959,13 +977,6 @@ pd_status pd_stable_dt(pd_ctx *c, double *dt)
 // ---- stepping -------------------------------------------------------------------
 // Enqueues one chunk of `steps` Verlet steps starting from u[parity]; contact
 // lists are rebuilt before the first step and then every k steps.
-// Whether pd_step runs its steps between rebuilds in one launch of the multi-step
-// kernel: the per-slot global-gather kernels only, not while profiling.
-static bool use_persist(const pd_ctx *c)
-{
-    return c->persist && !c->tiled && !c->pairs && !c->profiling;
-}
-
 // Grid of the multi-step kernel: resident blocks, at most one per GPB rows.
 static int persist_grid(const pd_ctx *c)
 {
