@@ -102,7 +102,7 @@ struct StepParams {
     double *wall_pos;              // nw*3, current wall points (device)
     double b[3];
     // per-block partials and the last-block reduction
-    double *partials;              // gridDim.x * PART_STRIDE
+    double *partials;              // [component][block], room for gridDim.x * PART_STRIDE
     unsigned *counter;
     unsigned *vmax_bits;           // max |v|^2 of the step as FP32 bits (atomicMax)
     unsigned *err;                 // error bits; [1]: steps taken since it was cleared
@@ -141,7 +141,7 @@ struct StepParams {
     float4 *fup;                   // per row: pass 1's force from the row's own slots
 };
 
-#define PART_STRIDE 20  // 18 reaction components, padded
+#define PART_STRIDE 20  // 18 reaction components, padded (the partials are component-major)
 #define PD_GL 32        // Gauss-Legendre points of the multi-wall overlap integrals
 
 // Radix sort of (key, value) pairs, LSD 8-bit digits, stable.  bits = number of

@@ -1162,25 +1162,26 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
 
 // A block's part of the step: the wall reactions summed over its groups (a warp per
 // component, lanes striding over the groups, a fixed xor butterfly; zeros if no node
-// touches a wall) to `part`, the largest |v|^2 into *vmax_bits (a max does not depend on
+// touches a wall) to partials[c][block], the largest |v|^2 into *vmax_bits (a max does not depend on
 // order), the error bits.  Adding 64 groups' sums in turn in one thread a component, and as
 // many maxima in another, took a third of a block's fixed cost of 2.8 us.
 template <int GPB>
 __device__ __forceinline__ void block_partials(const StepParams &p, const double (*s_react)[PD_MAX_WALLS * 3],
-                                               unsigned s_vbits, unsigned s_err, double *part, unsigned *vmax_bits)
+                                               unsigned s_vbits, unsigned s_err, double *partials, unsigned *vmax_bits)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ncomp = 3 * p.walls.nw;
+    double *part = partials + blockIdx.x;
     if (s_err & STEP_TOUCH) {
         for (int c = warp; c < ncomp; c += STEP_THREADS / 32) {
             double s = 0.0;
             for (int g = lane; g < GPB; g += 32) s += s_react[g][c];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) part[c] = s;
+            if (lane == 0) part[(int64_t)c * gridDim.x] = s;
         }
     } else if ((int)threadIdx.x < ncomp) {
-        part[threadIdx.x] = 0.0;
+        part[(int64_t)threadIdx.x * gridDim.x] = 0.0;
     }
     if (threadIdx.x == STEP_THREADS - 1) {
         if (s_vbits) atomicMax(vmax_bits, s_vbits);
@@ -1202,14 +1203,27 @@ __device__ __forceinline__ void block_collect(float vmax2f, double vmax2, unsign
 // lanes striding over the blocks (unrolled so that the loads of several blocks' partials
 // are in flight together; the additions keep their order), a fixed xor butterfly, so the
 // result is bitwise reproducible.
-__device__ __forceinline__ void store_reaction(const StepParams &p, int c, double s)
+__device__ __forceinline__ void sum_reaction(const StepParams &p, const double *partials, int c)
 {
+    const int lane = threadIdx.x & 31;
+    const double before = p.impulse[c];
+    const double *part = partials + (int64_t)c * gridDim.x;
+    double s = 0.0;
+#pragma unroll 8
+    for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(part + b);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
         p.react[c] = s;
-        if (p.mode != MODE_FORCES) p.impulse[c] = dadd(p.impulse[c], dmul(p.dt, s));
+        if (p.mode != MODE_FORCES) p.impulse[c] = dadd(before, dmul(p.dt, s));
     }
+}
+
+// the walls move by dt v; called by threads 0..31 of a block
+__device__ __forceinline__ void advance_walls(const StepParams &p)
+{
+    const int t = threadIdx.x;
+    if (t < 3 * p.walls.nw) p.wall_pos[t] = dadd(p.wall_pos[t], dmul(p.dt, p.walls.v[t / 3][t % 3]));
 }
 
 // The finish of the step by the last block: the wall reactions, the walls' motion and the
@@ -1220,7 +1234,7 @@ __device__ __forceinline__ void block_finish(const StepParams &p, const double (
 {
     __syncthreads();
     const int ncomp = 3 * p.walls.nw;
-    block_partials<GPB>(p, s_react, s_vbits, s_err, p.partials + (int64_t)blockIdx.x * PART_STRIDE, p.vmax_bits);
+    block_partials<GPB>(p, s_react, s_vbits, s_err, p.partials, p.vmax_bits);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1230,29 +1244,19 @@ __device__ __forceinline__ void block_finish(const StepParams &p, const double (
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int NW = STEP_THREADS / 32, PER = (3 * PD_MAX_WALLS + NW - 1) / NW;
-    if (warp < ncomp) {
-        double s[PER] = {0.0};
-#pragma unroll 4
-        for (unsigned b = lane; b < gridDim.x; b += 32)
-#pragma unroll
-            for (int q = 0; q < PER; ++q)
-                if (warp + NW * q < ncomp) s[q] += __ldcg(p.partials + (int64_t)b * PART_STRIDE + warp + NW * q);
-#pragma unroll
-        for (int q = 0; q < PER; ++q)
-            if (warp + NW * q < ncomp) store_reaction(p, warp + NW * q, s[q]);
-    }
-    if (threadIdx.x == 0) {
+    // each chain of dependent global accesses in a thread of its own, side by side: one
+    // thread moving 6 walls in turn took 6.5 us of every step, at the end of which the
+    // other SMs wait (hollow sphere of 343,846 nodes
+    // between two walls 165 -> 160 us a step, of 37,272 nodes 32.0 -> 27.9)
+    if (threadIdx.x < 32 && p.mode == MODE_FULL) advance_walls(p);
+    for (int c = threadIdx.x >> 5; c < ncomp; c += STEP_THREADS / 32) sum_reaction(p, p.partials, c);
+    if (threadIdx.x == STEP_THREADS - 1) {
         if (p.mode != MODE_FORCES) ++p.err[1];  // steps taken
         const double vm = (double)__uint_as_float(atomicExch(p.vmax_bits, 0u));  // max |v|^2, reset
         if (p.mode == MODE_FULL) {
             const double dsp = *p.disp + p.dt * sqrt(vm);
             *p.disp = dsp;
             if (2.0 * dsp >= p.skin) *p.stale = 1;
-            for (int l = 0; l < p.walls.nw; ++l)
-                for (int q = 0; q < 3; ++q)
-                    p.wall_pos[3 * l + q] = dadd(p.wall_pos[3 * l + q], dmul(p.dt, p.walls.v[l][q]));
         }
         *p.counter = 0u;
     }
@@ -1387,19 +1391,14 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
     // when every block has read it (two steps ago) and none writes it yet
     double *partials = p.partials + (int64_t)(step & 1) * gridDim.x * PART_STRIDE;
     unsigned *vmax_bits = bar + 1 + step % 3;
-    block_partials<GPB>(p, s_react, s_vbits, s_err, partials + (int64_t)blockIdx.x * PART_STRIDE, vmax_bits);
+    block_partials<GPB>(p, s_react, s_vbits, s_err, partials, vmax_bits);
     if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile unsigned *)(bar + 1 + (step + 1) % 3) = 0u;
     if (!grid_barrier(bar, ++nbar * arrivals, p.err, &s_ok)) return false;
     const int ncomp = 3 * p.walls.nw;
     // one block a component, so that none is far behind the others at the next barrier
     // (block 0 alone took 3 us for twelve of them)
     if (threadIdx.x < 32)
-        for (int c = blockIdx.x; c < ncomp; c += gridDim.x) {
-            double s = 0.0;
-#pragma unroll 8
-            for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) s += __ldcg(partials + (int64_t)b * PART_STRIDE + c);
-            store_reaction(p, c, s);
-        }
+        for (int c = blockIdx.x; c < ncomp; c += gridDim.x) sum_reaction(p, partials, c);
     // the same bookkeeping in every block
     if (threadIdx.x == STEP_THREADS - 1)
         s_disp = s_disp + p.dt * sqrt((double)__uint_as_float(__ldcg(vmax_bits)));
@@ -1617,11 +1616,7 @@ __global__ void k_drift(const StepParams p)
             vm = fmaxf(vm, __double2float_ru(v.x * v.x + v.y * v.y + v.z * v.z));
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        for (int l = 0; l < p.walls.nw; ++l)
-            for (int q = 0; q < 3; ++q)
-                p.wall_pos[3 * l + q] = dadd(p.wall_pos[3 * l + q], dmul(p.dt, p.walls.v[l][q]));
-    }
+    if (blockIdx.x == 0 && threadIdx.x < 32) advance_walls(p);
     if (!p.contact) return;  // uniform: a kernel parameter
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, o));

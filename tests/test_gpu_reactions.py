@@ -43,5 +43,8 @@ def test_reactions_match_the_oracle_and_the_multi_step_kernel(lanes, nw, precisi
         out.append([np.asarray(q).copy() for q in ctx.get_state()[:3]] +
                    [ctx.bulk_stress(areas)[1], ctx.bulk_stress_mean(areas)[1], ctx.get_walls()])
         ctx.close()
-    for a, b in zip(*out):
-        assert np.array_equal(a, b)
+    for k, (a, b) in enumerate(zip(*out)):
+        if k in (3, 4):  # summed over other blocks where the two kernels' grids differ (32 lanes)
+            assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+        else:
+            assert np.array_equal(a, b)
