@@ -54,7 +54,8 @@ __device__ __forceinline__ double2 ld_len(const double2 *a)
 // Newton correction.  The FP64 bond loop is bound by the FP64 pipe (2 lanes a clock an
 // SM): with sqrt and two divisions, and the undeformed length computed again in every
 // step, a directed bond cost some 62 FP64 instructions, with this and the stored
-// lengths (16 bytes a slot) some 30.  Plate cut of 21,240 nodes: 654 -> 354 us a step.
+// lengths (16 bytes a slot) some 30.  Plate cut of 21,240 nodes: 654 -> 354 us a step (321
+// with its rows spread over the SMs, first_row).
 __device__ __forceinline__ void root64(double a, double &l, double &r)
 {
     double x0;
@@ -1275,6 +1276,25 @@ __device__ __forceinline__ void block_begin(const StepParams &p, double (*s_reac
     }
 }
 
+// The first row of a warp, and its group's place among the rows from there.  On the mixed
+// path the rows of a block are adjacent: it lives on the neighbours that they share in L1
+// (the 178,200-node plate 142 us a force evaluation, 150 with the rows of one warp adjacent).
+// On the FP64 path, which the FP64 pipe bounds, those of a warp are, so that work that
+// clusters in the body is spread over the SMs (plate cut of 21,240 nodes 354 -> 321 us a
+// step, plate 2,462 -> 2,382, hollow sphere of 37,272 339 -> 299, packing of 134,592 1,057
+// -> 1,016).
+template <int G, bool MIXED>
+__device__ __forceinline__ int64_t first_row()
+{
+    if (MIXED) return (int64_t)blockIdx.x * (STEP_THREADS / G);
+    return ((int64_t)blockIdx.x + (int64_t)gridDim.x * (threadIdx.x >> 5)) * (32 / G);
+}
+template <int G, bool MIXED>
+__device__ __forceinline__ int row_of_group()
+{
+    return MIXED ? threadIdx.x / G : (threadIdx.x & 31) / G;
+}
+
 // Rows in a grid-stride loop, neighbour records gathered from global memory
 // (FP64 path, and the mixed path without tiles).
 template <int G, bool MIXED, bool WX, bool PAIRS = false>
@@ -1295,8 +1315,8 @@ __global__ void __launch_bounds__(STEP_THREADS, MIXED ? PD_MINB_GLOBAL : 2) k_st
     double vmax2 = 0.0;
     float vmax2f = 0.f;
     const TileView tv{nullptr, nullptr, nullptr, false};
-    for (int64_t r0 = (int64_t)blockIdx.x * GPB; r0 < p.n; r0 += (int64_t)gridDim.x * GPB) {
-        const int64_t row = r0 + grp;
+    for (int64_t r0 = first_row<G, MIXED>(); r0 < p.n; r0 += (int64_t)gridDim.x * GPB) {
+        const int64_t row = r0 + row_of_group<G, MIXED>();
         process_row<G, MIXED, WX, PAIRS>(p, p.wall_pos, s_wf, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
     }
     block_collect<MIXED>(vmax2f, vmax2, err, s_vbits, s_err);
@@ -1380,8 +1400,8 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
     double vmax2 = 0.0;
     float vmax2f = 0.f;
     const TileView tv{nullptr, nullptr, nullptr, false};
-    for (int64_t r0 = (int64_t)blockIdx.x * GPB; r0 < p.n; r0 += (int64_t)gridDim.x * GPB) {
-        const int64_t row = r0 + grp;
+    for (int64_t r0 = first_row<G, MIXED>(); r0 < p.n; r0 += (int64_t)gridDim.x * GPB) {
+        const int64_t row = r0 + row_of_group<G, MIXED>();
         process_row<G, MIXED, WX, false, true>(p, s_wall, s_wf, row, row < p.n, gl, 0, tv, s_react[grp], err, vmax2f, vmax2);
     }
     block_collect<MIXED>(vmax2f, vmax2, err, s_vbits, s_err);
