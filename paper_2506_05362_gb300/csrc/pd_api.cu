@@ -1221,7 +1221,7 @@ static pd_status run_segment(pd_ctx *c, double dt, int64_t left, int64_t *m_out,
     pd_status s = left == 1 ? PD_OK : rebuild_period(c, dt, &k);
     if (s) return s;
     bool carry = left == 1 && c->list_ok && c->opt.contact;
-    // a rollback costs at most one segment of work
+    // a rollback (an overflowed list) costs at most one segment of work
     int64_t m = std::min<int64_t>(left, (int64_t)PD_SEGMENT_CHUNKS * chunk_for(c, k));
     *m_out = m;
     const int cur0 = c->cur;

@@ -1416,7 +1416,7 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
     if (!grid_barrier(bar, ++nbar * arrivals, p.err, &s_ok)) return false;
     const int ncomp = 3 * p.walls.nw;
     // one block a component, so that none is far behind the others at the next barrier
-    // (block 0 alone took 3 us for twelve of them)
+    // (one block doing them all was late by up to 3 us)
     if (threadIdx.x < 32)
         for (int c = blockIdx.x; c < ncomp; c += gridDim.x) sum_reaction(p, partials, c);
     // the same bookkeeping in every block
