@@ -1,9 +1,10 @@
 // Bulk-stress surrogate: MLP with exact GELU, BF16 weights and activations,
 // FP32 accumulation and FP32 master weights, MSE loss, Adam.
 //
-// GEMMs run on the tensor cores (mma.sync m16n8k16 BF16 -> FP32) with
-// cp.async triple buffering and ldmatrix / ldmatrix.trans, so one kernel
-// serves the three operand layouts of training:
+// Networks whose layers all fit the fused tcgen05 kernels run there (pd_mlp_tc.cu; training
+// ends in k_update below).  For the others (and path 1) the GEMMs here run on the tensor
+// cores (mma.sync m16n8k16 BF16 -> FP32) with cp.async triple buffering and ldmatrix /
+// ldmatrix.trans, so one kernel serves the three operand layouts of training:
 //   forward      Z  = H  W^T + b      (A = H  row-major, B = W  row-major)
 //   data grad    dH = dZ W            (A = dZ row-major, B = W  read transposed)
 //   weight grad  dW = dZ^T H          (A = dZ read transposed, B = H read transposed)
