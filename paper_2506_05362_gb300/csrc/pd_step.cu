@@ -686,8 +686,8 @@ __device__ __forceinline__ unsigned epilogue_lanes(const StepParams &p, const do
 // l = sqrt(a), r = 1 / sqrt(a) for any a > 0 (root64 wants a normal number).  A contact
 // evaluation is a chain of dependent FP64 operations in one or two lanes of a warp, the
 // square root and the division half of it before: with this in their place a step of the
-// 47,808-node aggregate takes 62.4 us instead of 65.7 (5,770 touching pairs), its pair
-// damping 12.4 us instead of 14.1.
+// 47,808-node aggregate took 62.4 us instead of 65.7 (5,770 touching pairs; 55.4 with the
+// end of a step split up since), its pair damping 12.4 us instead of 14.1.
 __device__ __forceinline__ void dist64(double a, double &l, double &r)
 {
     if (a > 1e-280) {
