@@ -371,37 +371,41 @@ __global__ void k_colsum(const bf16 *__restrict__ dZ, int64_t rows, int ld, int 
     if (threadIdx.x == 0 && c < n_valid) gb[c] = s[0];
 }
 
+// One parameter's Adam step.  The multiply-adds are written out, so that every kernel
+// rounds alike whatever the compiler would contract.
+__device__ __forceinline__ float adam_step(float w, float g, float &m, float &v, float lr, float b1, float b2, float eps,
+                                           float c1, float c2)
+{
+    m = __fmaf_rn(1.f - b1, g, __fmul_rn(b1, m));
+    v = __fmaf_rn(__fmul_rn(1.f - b2, g), g, __fmul_rn(b2, v));
+    return w - lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+
 __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
                        int64_t n, float lr, float b1, float b2, float eps, float c1, float c2)
 {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        const float gq = g[q];
-        const float mq = b1 * m[q] + (1.f - b1) * gq;
-        const float vq = b2 * v[q] + (1.f - b2) * gq * gq;
-        m[q] = mq;
-        v[q] = vq;
-        w[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + eps);
+        w[q] = adam_step(w[q], g[q], m[q], v[q], lr, b1, b2, eps, c1, c2);
     }
 }
 
-// Everything after the last GEMM of a tcgen05 training step in one launch: the split-K
-// partials of every layer's weight and bias gradients summed in a fixed order into the
-// gradient vector, and, for a training step, Adam on them and the new weights and biases
-// in the layouts the GEMMs read (their padding stays as it was set); block 0 also sums the
-// loss.  A thread takes one parameter, its partials eight loads at a time: bound by the
-// latency of those loads (16 partials of 0.9 MB each, from L2).  16 launches (reductions,
-// bias row sums, Adam, repacking) did this before: 135 us a step of the surrogate at batch
-// 65,536, this 8.9 us; one warp per 32 parameters and part of the splits, as in
-// k_reduce_dw, took 20.
+// Everything after the last GEMM of a tcgen05 training step in one launch: the parts of
+// every layer's weight gradient summed in order into the gradient vector, and, for a
+// training step, Adam on it and the new weights and biases in the layouts the GEMMs read
+// (their padding stays as it was set); block 0 also sums the loss, as k_loss_final does.  A
+// thread takes one parameter, its partials' loads all in flight: bound by their latency (8
+// partials of 0.9 MB each, from L2).  16 launches (reductions, bias row sums, Adam,
+// repacking) did this and the sums beside the GEMMs before: 135 us a step of the surrogate
+// at batch 65,536, this 11 us.
 struct UpdateLayer {
-    const float *part, *partb;  // [splits x N x K], [splits x N]
-    int N, K, k_valid;
+    const float *part, *gb;     // [parts x N x K], [N]
+    int N, K, k_valid, parts;
     int64_t w0, b0;             // offsets of W and b in the parameter vector (b follows W)
     bf16 *Wb, *WT;
     float *bias;
 };
 struct Update {
-    int L, splits;
+    int L;
     int64_t nparams;
     UpdateLayer l[8];
     float *w, *m, *v, *g;
@@ -439,18 +443,14 @@ __global__ void __launch_bounds__(256) k_update(const __grid_constant__ Update U
     const bool isw = p < Y.b0;
     const int q = (int)(p - (isw ? Y.w0 : Y.b0));
     const int r = isw ? q / Y.k_valid : q, c = isw ? q - r * Y.k_valid : 0;
-    const float *src = isw ? Y.part + (size_t)r * Y.K + c : Y.partb + r;
-    const size_t zs = isw ? (size_t)Y.N * Y.K : (size_t)Y.N;
-    float g = 0.f;
-#pragma unroll 8
-    for (int z = 0; z < U.splits; ++z) g += __ldcs(src + (size_t)z * zs);
+    const float *src = isw ? Y.part + (size_t)r * Y.K + c : Y.gb + r;
+    const size_t zs = (size_t)Y.N * Y.K;
+    float g = __ldcs(src);
+#pragma unroll 7
+    for (int z = 1; z < (isw ? Y.parts : 1); ++z) g += __ldcs(src + (size_t)z * zs);
     U.g[p] = g;
     if (!U.adam) return;
-    const float mq = U.b1 * U.m[p] + (1.f - U.b1) * g;
-    const float vq = U.b2 * U.v[p] + (1.f - U.b2) * g * g;
-    U.m[p] = mq;
-    U.v[p] = vq;
-    const float w = U.w[p] - U.lr * (mq / U.c1) / (sqrtf(vq / U.c2) + U.eps);
+    const float w = adam_step(U.w[p], g, U.m[p], U.v[p], U.lr, U.b1, U.b2, U.eps, U.c1, U.c2);
     U.w[p] = w;
     if (isw) {
         const bf16 h = __float2bfloat16_rn(w);
@@ -505,7 +505,8 @@ struct pd_mlp {
     float *part = nullptr;    // split-K partials
     int64_t part_cap = 0;
     float *lpart = nullptr, *dloss = nullptr;
-    unsigned *tc_err = nullptr;  // error word of the tcgen05 forward
+    unsigned *tc_err = nullptr;  // error word of the tcgen05 kernels
+    unsigned *next = nullptr;    // task counter of k_dw_tc
     int path = 0;                // 0: tcgen05 forward when the shapes allow; 1: mma.sync only
     std::vector<void *> owned;
 };
@@ -610,7 +611,7 @@ pd_status forward_dev(pd_mlp *m, const float *X, int64_t rows, float *Y, bool ke
         void *W[8];
         const float *b[8];
         for (int l = 0; l < m->L; ++l) { W[l] = m->Wb[l]; b[l] = m->bias[l]; }
-        if (mlp_forward_tc(m->L, m->dims, m->pad, W, b, X, rows, Y, nullptr, m->tc_err, m->device, m->st) > 0)
+        if (mlp_forward_tc(m->L, m->dims, m->pad, W, b, X, rows, Y, nullptr, m->tc_err, m->device, m->st) == 0)
             return PD_OK;
         if (m->path == 2) return mfail(m, PD_EINVAL, "the tcgen05 forward cannot run this network or GPU");
     }
@@ -680,21 +681,21 @@ int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float l
     tr.Z = Z;
     tr.HT = HT;
     tr.ldT = m->ldT;
+    tr.Y = m->Y;
     tr.T = T;
     tr.scale = 2.0f / (float)(rows * nout);
     tr.dY = m->dZ[L - 1];
     tr.dYT = m->dZT[L - 1];
     tr.lpart = m->lpart;
+    tr.next = m->next;
     // room for every layer's partials
     int64_t need = 0, at[8];
-    const int splits = mlp_dw_splits(L, m->pad, rows, m->device);
     for (int l = 0; l < L; ++l) {
         at[l] = need;
-        need += (int64_t)splits * m->pad[l + 1] * (m->pad[l] + 1);
+        need += (int64_t)m->pad[l + 1] * (mlp_dw_parts(m->pad[l + 1], rows, m->device, nullptr, nullptr) * m->pad[l] + 1);
         need = (need + 31) / 32 * 32;
     }
-    const int nlp = mlp_forward_tc(L, m->dims, m->pad, W, b, X, rows, nullptr, &tr, m->tc_err, m->device, m->st);
-    if (nlp < 0) return -1;
+    if (mlp_forward_tc(L, m->dims, m->pad, W, b, X, rows, nullptr, &tr, m->tc_err, m->device, m->st)) return -1;
     if (ensure_part(m, need)) return -2;
     void *WT[8], *dZT[8];
     for (int l = 0; l < L; ++l) { WT[l] = m->WT[l]; dZT[l] = m->dZT[l]; }
@@ -702,19 +703,20 @@ int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float l
     Update U;
     memset(&U, 0, sizeof(U));
     U.L = L;
-    float *part[8], *partb[8];
+    float *part[8], *gb[8];
     for (int l = 0; l < L; ++l) {
         const int N = m->pad[l + 1], K = m->pad[l];
-        part[l] = m->part + at[l];
-        partb[l] = part[l] + (int64_t)splits * N * K;
         UpdateLayer &Y = U.l[l];
-        Y.part = part[l]; Y.partb = partb[l]; Y.N = N; Y.K = K;
+        Y.parts = mlp_dw_parts(N, rows, m->device, nullptr, nullptr);
+        part[l] = m->part + at[l];
+        gb[l] = part[l] + (int64_t)Y.parts * N * K;
+        Y.part = part[l]; Y.gb = gb[l]; Y.N = N; Y.K = K;
         Y.k_valid = m->dims[l];
         Y.w0 = m->woff[l]; Y.b0 = m->boff[l];
         Y.Wb = m->Wb[l]; Y.WT = m->WT[l]; Y.bias = m->bias[l];
     }
-    if (mlp_dw_tc(L, m->pad, dZT, HT, rows, m->ldT, part, partb, m->tc_err, m->device, m->st)) return -2;
-    U.splits = splits;
+    const int nlp = grid1(rows * m->pad[L]);
+    if (mlp_dw_tc(L, m->dims, m->pad, dZT, HT, rows, tr, nlp, part, gb, m->tc_err, m->device, m->st)) return -2;
     U.nparams = m->nparams;
     U.w = m->master; U.m = m->m; U.v = m->v; U.g = m->grad;
     if (lr > 0) {
@@ -741,7 +743,7 @@ pd_status backward_dev(pd_mlp *m, const float *X, const float *T, int64_t rows, 
     pd_status s = forward_dev(m, X, rows, m->Y, true);
     if (s) return s;
     const int L = m->L, nout = m->dims[L];
-    const int nb = std::min(grid1(rows * m->pad[L]), 8192);
+    const int nb = grid1(rows * m->pad[L]);
     k_loss<<<nb, 256, 0, m->st>>>(m->Y, T, rows, nout, m->pad[L], m->dZ[L - 1], m->lpart);
     k_loss_final<<<1, 256, 0, m->st>>>(m->lpart, nb, rows * nout, m->dloss);
     if (loss2) MCK(cudaMemcpyAsync(loss2, m->dloss, sizeof(float), cudaMemcpyDeviceToDevice, m->st));
@@ -823,7 +825,7 @@ pd_status pd_mlp_create(const int *dims, int nlayers, uint64_t seed, int device,
     pd_status s = PD_OK;
     if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); delete m; return PD_ECUDA; }
     if ((s = malloc_(m, &m->master, off)) || (s = malloc_(m, &m->m, off)) || (s = malloc_(m, &m->v, off)) ||
-        (s = malloc_(m, &m->grad, off)) || (s = malloc_(m, &m->dloss, 4)) || (s = malloc_(m, &m->tc_err, 1))) {
+        (s = malloc_(m, &m->grad, off)) || (s = malloc_(m, &m->dloss, 4)) || (s = malloc_(m, &m->tc_err, 2))) {
         pd_mlp_destroy(m);
         return s;
     }
@@ -835,7 +837,8 @@ pd_status pd_mlp_create(const int *dims, int nlayers, uint64_t seed, int device,
             return s;
         }
     }
-    if (cudaMemsetAsync(m->tc_err, 0, sizeof(unsigned), m->st) != cudaSuccess) {
+    m->next = m->tc_err + 1;
+    if (cudaMemsetAsync(m->tc_err, 0, 2 * sizeof(unsigned), m->st) != cudaSuccess) {
         cudaGetLastError();
         pd_mlp_destroy(m);
         return PD_ECUDA;

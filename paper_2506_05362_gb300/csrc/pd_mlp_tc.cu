@@ -17,7 +17,7 @@
 //               tile in the swizzled layout; the last layer writes FP32 outputs.
 //               They also stage the input tile with coalesced reads.
 // The same kernel runs a training step's forward (it also stores what the backward needs
-// and ends in the loss) and, over the layers in reverse with the transposed weights, its
+// and ends in the loss gradient) and, over the layers in reverse with the transposed weights, its
 // backward: dZ_{l-1} = (dZ_l W_l) GELU'(Z_{l-1}) stays in shared memory from layer to layer
 // and only its transposed copy, the operand of the weight gradient, is stored.  Both are
 // bound by the epilogue's instructions (GELU or GELU', the transposition by lane pairs, the
@@ -70,12 +70,12 @@ struct Params {
     __nv_bfloat16 *Z[MAX_LAYERS];
     __nv_bfloat16 *HT[MAX_LAYERS];
     int64_t ldT;
-    // and the MSE loss: targets [rows x out_cols], dY = scale (Y - T) as BF16 [rows x
-    // N_last] and transposed [N_last x ldT], and one partial sum of (Y - T)^2 a CTA
+    // and the gradient of the MSE loss: targets [rows x out_cols], dY = scale (Y - T) as
+    // BF16 [rows x N_last] and transposed [N_last x ldT]
     const float *T;
     float scale;
     __nv_bfloat16 *dY, *dYT;
-    float *lpart;
+    unsigned *next;   // task counter of k_dw_tc, cleared here
     // backward: the input is dY [rows x K_0]; layer i multiplies by GELU' of Z[i] [rows x
     // N_i] and stores its transposed result to HT[i] [N_i x ldT]
 };
@@ -493,7 +493,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
     uint64_t *done = a_ready + 2;
     uint32_t *tmem_slot = (uint32_t *)(done + 1);
     __shared__ volatile int s_abort;
-    __shared__ float s_loss[EPI_THREADS / 32];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -507,6 +506,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
         }
         mbar_init(done, 1);
         s_abort = 0;
+        if (TRAIN && blockIdx.x == 0) *P.next = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {  // TMEM: two accumulators of 256 columns x 128 lanes (FP32)
@@ -583,7 +583,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
         const int part = (warp - 2) >> 2;  // 0..3
         const int m = q * 32 + lane;       // row of the tile owned by this thread
         const int ew = warp - 2;
-        float loss = 0.f;  // training: this thread's part of the sum of (Y - T)^2
         uint32_t accph[2] = {0u, 0u};
         bool stopped = false;
         for (int b = 0; b < 2 && b < my; ++b) stage_input<MODE>(P, pair_tile(0, b), base + b * A_BYTES, ew, lane);
@@ -702,7 +701,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
                         __syncwarp();  // tcgen05.ld is warp-collective
                         tmem_ld32(tacc + (uint32_t)c0, v);
                         if (TRAIN) {
-                            // the loss and its gradient, row-major and transposed
+                            // the output and the loss gradient, row-major and transposed
 #pragma unroll
                             for (int c8 = 0; c8 < 32; c8 += 8) {
                                 if (c0 + c8 >= Ly.N) break;  // uniform
@@ -714,8 +713,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
                                     for (int u = 0; u < 2; ++u) {
                                         const int c = c0 + c8 + e + u;
                                         if (c < P.out_cols && row < P.rows) {
-                                            d[u] = (v[c8 + e + u] + __ldg(Ly.bias + c)) - __ldg(P.T + row * P.out_cols + c);
-                                            loss += d[u] * d[u];
+                                            const float y = v[c8 + e + u] + __ldg(Ly.bias + c);
+                                            P.Y[row * P.out_cols + c] = y;
+                                            d[u] = y - __ldg(P.T + row * P.out_cols + c);
                                         }
                                     }
                                     pk[e / 2] = pack_bf16x2(d[0] * P.scale, d[1] * P.scale);
@@ -756,19 +756,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
                         mbar_arrive(a_ready + b);
                     }
                 }
-        if (TRAIN) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-            if (lane == 0) s_loss[ew] = loss;
-        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (TRAIN && threadIdx.x == 0) {
-        float sum = 0.f;
-        for (int w = 0; w < EPI_THREADS / 32; ++w) sum += s_loss[w];
-        P.lpart[blockIdx.x] = sum;
-    }
     __syncwarp();
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * MAX_N));
 }
@@ -796,75 +786,193 @@ encode_fn_t encoder()
 }  // namespace
 
 // ---- weight gradients: C[M x N] = A[M x K] * B[N x K]^T over the batch K ----------
-// Both operands K-major and fed by TMA (same 128-byte swizzle as above).  All layers in
-// one launch: blockIdx.x is one 128-row tile of one layer's C (N <= 256), blockIdx.y one
-// split of the batch, and the splits are as many as give every SM one CTA, so that a
-// layer's FP32 partial sums part[split][m][n] are few (16 splits for the five layers of
-// the surrogate; a launch a layer wanted 76 to fill the SMs, 80 MB of partials to write and
-// read again).  The row sums of A over the split (the bias gradient) go to partb[split][m]:
-// the epilogue warps, idle until the end, read them from the stages.  Bound by the 290 MB
-// of operands it reads at batch 65,536: 52 us, 5.6 TB/s (12 us at batch 4,096).  The nine
-// GEMM launches of the data and weight gradients and the row sums took 348 us (129 us)
-// before; this and the fused data gradients take 181 us (52 us).
+// Both operands K-major and fed by TMA (same 128-byte swizzle as above), all layers in one
+// launch.  The batch is cut into splits as many as give every SM a CTA of a layer's 128-row
+// tiles; a split's sum is one accumulator in TMEM, and the splits are added in FP32 in the
+// order of k_reduce_dw: z = p, p + 8, p + 16, ... to part p, the parts in turn (k_update).
+// (The grouping is part of the result: Adam divides small gradients by their own size, so
+// that sums grouped otherwise are other weights after some steps.)  A CTA takes one 128 x
+// 128 tile of one layer's C and one part: its splits go through two TMEM accumulators in
+// turn, and the epilogue warps add one to the part, in registers, while the other fills.
+// So the eight parts go to memory and not the 74 splits of the surrogate's hidden layers at
+// batch 65,536 (67 MB a step).  Tiles of 128 columns, since with 256 the surrogate's eight
+// parts are 72 CTAs for 152 SMs; they read A twice, 670 MB with the row sums: 74 us, 9.1
+// TB/s out of L2 (19 us at batch 4,096).  The nine GEMM launches of the data and weight
+// gradients and the row sums took 348 us (129 us) before; this and the fused data gradients
+// take 203 us (59 us).
+//
+// The first CTAs of the grid, and the others once their tile is done, take the sums that
+// need no tensor cores, from a common counter, a warp each: the rows of dZ^T (the bias
+// gradients) and the loss.
 namespace {
 
 constexpr int G_EPI = 256;  // 8 epilogue warps, 2 per TMEM lane quarter
 constexpr int G_THREADS = 64 + G_EPI;
-constexpr int G_A_STAGE = TILE_M * KCHUNK * 2;  // 16 KiB
-constexpr int G_STAGES = 4;
-constexpr int G_SUM_WARPS = 4;                  // warps that also read the A stages
+constexpr int G_STAGE = TILE_M * KCHUNK * 2;  // 16 KiB of either operand
+constexpr int G_STAGES = 6;
+constexpr int G_COLS = 128;                   // columns of a tile of C
+constexpr int DW_PARTS = 8;                   // = RD_PARTS of k_reduce_dw
 
 struct DwLayer {
     CUtensorMap ma, mb;
     int M, N;            // rows of C that exist, columns
-    int tile0;           // the layer's first tile of 128 rows
-    float *part, *partb;
+    int tile0, nt;       // the layer's first tile, its tiles beside one another
+    int kcs, splits;     // K chunks per split, splits
+    float *part;
+    const __nv_bfloat16 *dZT;
+    float *gb;           // bias gradient
+    int row0;            // the layer's first row among those to be summed
 };
 struct DwArgs {
     DwLayer l[MAX_LAYERS];
-    int L, kchunks, kcs;  // kcs: K chunks per split
+    int L, kchunks, free_ctas;
+    int64_t rows, ldT;
+    int sum_rows;        // of all layers
+    const float *Y, *T;  // [rows x nout]
+    int nout, ldo, nlp;
+    float *lpart;
+    unsigned *next;      // task counter, zero
     unsigned *err;
 };
+
+// One row of dZ^T summed as a block of 1024 threads would: thread t adds the 16-byte words
+// t, t + 1024, ... two elements at a time, those beyond the last whole word go to the first
+// threads, and a tree halves the threads.  Lane l is threads l, l + 32, ..., 32 loads in
+// flight.
+__device__ __forceinline__ float row_sum(const __nv_bfloat16 *r, int64_t rows, int lane)
+{
+    float acc[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) acc[j] = 0.f;
+    const int64_t r8 = rows / 8;
+    for (int64_t q0 = lane; q0 < r8; q0 += 1024) {
+        uint4 w[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            w[j] = q0 + 32 * j < r8 ? __ldcs((const uint4 *)r + q0 + 32 * j) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const uint32_t h[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 f = __bfloat1622float2(*(const __nv_bfloat162 *)&h[e]);
+                acc[j] += f.x + f.y;
+            }
+        }
+    }
+    if (8 * r8 + lane < rows) acc[0] += __bfloat162float(r[8 * r8 + lane]);  // fewer than 8
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int j = 0; j < o; ++j) acc[j] += acc[j + o];
+    float s = acc[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// Block b of 256 threads of k_loss: thread t adds the squares of elements 256 b + t, + 256
+// nlp, ... of the padded output, then a tree; lane l is threads l, l + 32, ...
+__device__ __forceinline__ float loss_sum(const DwArgs &A, int b, int lane)
+{
+    float acc[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+    const int64_t total = A.rows * A.ldo;
+    for (int64_t q = (int64_t)b * 256; q < total; q += (int64_t)A.nlp * 256) {
+        const int64_t r0 = q / A.ldo;
+        const unsigned c0 = (unsigned)(q - r0 * A.ldo);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const unsigned x = c0 + 32u * j + lane, c = x % (unsigned)A.ldo;
+            const int64_t r = r0 + x / (unsigned)A.ldo;
+            if (r < A.rows && (int)c < A.nout) {
+                const float d = __ldg(A.Y + r * A.nout + c) - __ldg(A.T + r * A.nout + c);
+                acc[j] = fmaf(d, d, acc[j]);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int j = 0; j < o; ++j) acc[j] += acc[j + o];
+    float s = acc[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// Takes the remaining sums, a warp each: the rows first, then the blocks of the loss.
+__device__ __forceinline__ void take_sums(const DwArgs &A, int lane)
+{
+    const unsigned tasks = (unsigned)(A.sum_rows + A.nlp);
+    for (;;) {
+        unsigned i = 0;
+        if (lane == 0) i = atomicAdd(A.next, 1u);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= tasks) return;
+        if (i < (unsigned)A.sum_rows) {
+            int l = 0;
+            while (l + 1 < A.L && (int)i >= A.l[l + 1].row0) ++l;
+            const int64_t row = (int)i - A.l[l].row0;
+            const float s = row_sum(A.l[l].dZT + row * A.ldT, A.rows, lane);
+            if (lane == 0) A.l[l].gb[row] = s;
+        } else {
+            const int b = (int)i - A.sum_rows;
+            const float s = loss_sum(A, b, lane);
+            if (lane == 0) A.lpart[b] = s;
+        }
+    }
+}
 
 __global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ DwArgs A)
 {
     constexpr int S = G_STAGES;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = ((int)blockIdx.x - A.free_ctas) / DW_PARTS, p = ((int)blockIdx.x - A.free_ctas) % DW_PARTS;
     int layer = 0;
-    while (layer + 1 < A.L && (int)blockIdx.x >= A.l[layer + 1].tile0) ++layer;
+    while (layer + 1 < A.L && tile >= A.l[layer + 1].tile0) ++layer;
     const DwLayer &P = A.l[layer];
+    if ((int)blockIdx.x < A.free_ctas || p >= P.splits) {
+        take_sums(A, lane);
+        return;
+    }
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *sA = base;                      // S x 16 KiB
-    unsigned char *sB = base + S * G_A_STAGE;      // S x 32 KiB
-    uint64_t *full = (uint64_t *)(sB + S * W_STAGE_BYTES);
+    unsigned char *sB = base + S * G_STAGE;        // S x 16 KiB
+    uint64_t *full = (uint64_t *)(sB + S * G_STAGE);
     uint64_t *empty = full + S;
-    uint64_t *acc_full = empty + S;
-    uint64_t *done = acc_full + 1;
+    uint64_t *acc_full = empty + S;   // [2], per accumulator
+    uint64_t *acc_free = acc_full + 2;
+    uint64_t *done = acc_free + 2;
     uint32_t *tmem_slot = (uint32_t *)(done + 1);
     __shared__ volatile int s_abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int q = 0; q < S; ++q) {
             mbar_init(full + q, 1);
-            mbar_init(empty + q, 1 + G_SUM_WARPS);
+            mbar_init(empty + q, 1);
         }
-        mbar_init(acc_full, 1);
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(acc_full + q, 1);
+            mbar_init(acc_free + q, G_EPI);
+        }
         mbar_init(done, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(MAX_N));
+                     "r"(2 * G_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
-    const int m0 = ((int)blockIdx.x - P.tile0) * TILE_M;
-    const int kc0 = blockIdx.y * A.kcs, kc1 = min(A.kchunks, kc0 + A.kcs);
+    const int m0 = (tile - P.tile0) / P.nt * TILE_M, n0 = (tile - P.tile0) % P.nt * G_COLS;
+    const int cols = min(G_COLS, P.N - n0);
 
     if (warp == 0) {
         if (lane == 0) {
@@ -872,92 +980,94 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ 
             uint32_t ph = 0;
             int last_ph[S];
             for (int q = 0; q < S; ++q) last_ph[q] = -1;
-            for (int kc = kc0; kc < kc1 && !s_abort; ++kc) {
-                if (!mbar_wait(empty + s, ph ^ 1)) { atomicOr(A.err, 1u); s_abort = 1; break; }
-                mbar_expect_tx(full + s, (uint32_t)(G_A_STAGE + P.N * KCHUNK * 2));
-                tma_load_2d(sA + s * G_A_STAGE, &P.ma, full + s, kc * KCHUNK, m0);
-                tma_load_2d(sB + s * W_STAGE_BYTES, &P.mb, full + s, kc * KCHUNK, 0);
-                last_ph[s] = (int)ph;
-                if (++s == S) { s = 0; ph ^= 1; }
+            // a box of B has min(N, 128) rows; those beyond N arrive as zeros
+            const uint32_t bytes = (uint32_t)(G_STAGE + min(P.N, G_COLS) * KCHUNK * 2);
+            for (int z = p; z < P.splits && !s_abort; z += DW_PARTS) {
+                const int kc1 = min(A.kchunks, (z + 1) * P.kcs);
+                for (int kc = z * P.kcs; kc < kc1 && !s_abort; ++kc) {
+                    if (!mbar_wait(empty + s, ph ^ 1)) { atomicOr(A.err, 1u); s_abort = 1; break; }
+                    mbar_expect_tx(full + s, bytes);
+                    tma_load_2d(sA + s * G_STAGE, &P.ma, full + s, kc * KCHUNK, m0);
+                    tma_load_2d(sB + s * G_STAGE, &P.mb, full + s, kc * KCHUNK, n0);
+                    last_ph[s] = (int)ph;
+                    if (++s == S) { s = 0; ph ^= 1; }
+                }
             }
             for (int q = 0; q < S; ++q)
                 if (last_ph[q] >= 0 && !mbar_wait(full + q, (uint32_t)last_ph[q])) atomicOr(A.err, 1u);
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
-            const uint32_t idesc = idesc_bf16(TILE_M, P.N);
-            for (int kc = kc0; kc < kc1 && !s_abort; ++kc) {
-                if (!mbar_wait(full + s, ph)) { atomicOr(A.err, 1u); s_abort = 1; break; }
+            int s = 0, b = 0;
+            uint32_t ph = 0, fph = 1;  // both accumulators are free at the start
+            const uint32_t idesc = idesc_bf16(TILE_M, cols);
+            for (int z = p; z < P.splits && !s_abort; z += DW_PARTS) {
+                if (!mbar_wait(acc_free + b, fph)) { atomicOr(A.err, 1u); s_abort = 1; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a0 = smem_u32(sA + s * G_A_STAGE);
-                const uint32_t b0 = smem_u32(sB + s * W_STAGE_BYTES);
+                const uint32_t d = tmem + (uint32_t)(b * G_COLS);
+                const int kc0 = z * P.kcs, kc1 = min(A.kchunks, kc0 + P.kcs);
+                for (int kc = kc0; kc < kc1; ++kc) {
+                    if (!mbar_wait(full + s, ph)) { atomicOr(A.err, 1u); s_abort = 1; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t a0 = smem_u32(sA + s * G_STAGE);
+                    const uint32_t b0 = smem_u32(sB + s * G_STAGE);
 #pragma unroll
-                for (int kk = 0; kk < KCHUNK / 16; ++kk)
-                    mma_bf16(tmem, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), idesc, (kc != kc0 || kk != 0));
-                mma_commit(empty + s);
-                if (++s == S) { s = 0; ph ^= 1; }
+                    for (int kk = 0; kk < KCHUNK / 16; ++kk)
+                        mma_bf16(d, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), idesc, (kc != kc0 || kk != 0));
+                    mma_commit(empty + s);
+                    if (++s == S) { s = 0; ph ^= 1; }
+                }
+                mma_commit(acc_full + b);
+                b ^= 1;
+                if (b == 0) fph ^= 1;
             }
-            mma_commit(acc_full);
             mma_commit(done);
             if (!mbar_wait(done, 0)) atomicOr(A.err, 1u);
         }
     } else {
         const int q = warp & 3;
-        const int part = (warp - 2) >> 2;  // 0..1
-        const int m = q * 32 + lane;
-        const int64_t row = (int64_t)m0 + m;
-        if (part == 0) {
-            // row sums of A: this thread's row of every stage (128 swizzled bytes)
-            int s = 0;
-            uint32_t ph = 0;
-            float sum = 0.f;
-            for (int kc = kc0; kc < kc1; ++kc) {
-                const bool ok = mbar_wait(full + s, ph);
-                if (!ok) { atomicOr(A.err, 1u); s_abort = 1; }
-                if (__any_sync(0xffffffffu, !ok || s_abort)) break;
-                const unsigned char *a = sA + s * G_A_STAGE + (m >> 3) * 1024 + (m & 7) * 128;
+        const int c0 = (warp - 2) / 4 * 64;  // this warp's first column
+        const int64_t row = (int64_t)m0 + q * 32 + lane;
+        float acc[64];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint4 w = *(const uint4 *)(a + ((c ^ (m & 7)) << 4));
-                    const uint32_t h[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 f = __bfloat1622float2(*(const __nv_bfloat162 *)&h[e]);
-                        sum += f.x + f.y;
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(empty + s);
-                if (++s == S) { s = 0; ph ^= 1; }
-            }
-            if (row < P.M) P.partb[(int64_t)blockIdx.y * P.M + row] = sum;
-        }
-        __syncwarp();
-        const bool ok = mbar_wait(acc_full, 0);
-        if (!ok) { atomicOr(A.err, 1u); s_abort = 1; }
-        if (!__any_sync(0xffffffffu, !ok || s_abort)) {
+        for (int e = 0; e < 64; ++e) acc[e] = 0.f;
+        int b = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int z = p; z < P.splits; z += DW_PARTS) {
+            __syncwarp();
+            ok = mbar_wait(acc_full + b, ph);
+            if (!ok) { atomicOr(A.err, 1u); s_abort = 1; }
+            ok = !__any_sync(0xffffffffu, !ok || s_abort);
+            if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int hw = ((P.N / 2 + 31) / 32) * 32;
-            const int cend = min(P.N, (part + 1) * hw);
-            const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16);
-            for (int c0 = part * hw; c0 < cend; c0 += 32) {
-                float v[32];
-                __syncwarp();
-                tmem_ld32(tacc + (uint32_t)c0, v);
-                if (row >= P.M) continue;
-                float *dst = P.part + ((int64_t)blockIdx.y * P.M + row) * P.N + c0;
+            const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * G_COLS + c0);
 #pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    if (c0 + e < P.N) *(float4 *)(dst + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-            }
+            for (int h = 0; h < 64; h += 32)
+                if (c0 + h < cols) {  // uniform in the warp
+                    float v[32];
+                    tmem_ld32(tacc + (uint32_t)h, v);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) acc[h + e] += v[e];
+                }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(acc_free + b);
+            b ^= 1;
+            if (b == 0) ph ^= 1;
+        }
+        if (ok && row < P.M) {
+            float *dst = P.part + ((int64_t)p * P.M + row) * P.N + n0 + c0;
+#pragma unroll
+            for (int e = 0; e < 64; e += 4)
+                if (c0 + e < cols) *(float4 *)(dst + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     __syncwarp();
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(MAX_N));
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * G_COLS));
+    take_sums(A, lane);
 }
 
 // K-major BF16 tensor map: rows x cols (cols = K, contiguous), row stride ld elements
@@ -976,57 +1086,65 @@ bool kmajor_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, i
 
 }  // namespace
 
-// Splits of the batch for the weight gradients of layers with `tiles` 128-row tiles in
-// all: one CTA an SM, at least 4 chunks of 64 samples a split (below that the partial sums
-// cost more than the GEMM), no split without work.
-static int dw_splits(int64_t rows, int tiles, int device, int *kcs)
+int mlp_dw_parts(int pad_out, int64_t rows, int device, int *kcs, int *splits)
 {
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    const int kchunks = (int)((rows + KCHUNK - 1) / KCHUNK), most = std::max(1, sms / tiles);
-    *kcs = std::max(4, (kchunks + most - 1) / most);
-    return (kchunks + *kcs - 1) / *kcs;
-}
-static int dw_tiles(int L, const int *pad)
-{
-    int t = 0;
-    for (int l = 0; l < L; ++l) t += (pad[l + 1] + TILE_M - 1) / TILE_M;
-    return t;
-}
-int mlp_dw_splits(int L, const int *pad, int64_t rows, int device)
-{
-    int kcs;
-    return dw_splits(rows, dw_tiles(L, pad), device, &kcs);
+    const int kchunks = (int)((rows + KCHUNK - 1) / KCHUNK), mt = (pad_out + TILE_M - 1) / TILE_M;
+    const int most = std::max(1, std::min(128, sms / mt));
+    const int k = (kchunks + most - 1) / most, n = (kchunks + k - 1) / k;  // no split without work
+    if (kcs) *kcs = k;
+    if (splits) *splits = n;
+    return std::min(n, DW_PARTS);
 }
 
-int mlp_dw_tc(int L, const int *pad, void *const *dZT, void *const *HT, int64_t rows, int64_t ldT, float *const *part,
-              float *const *partb, unsigned *err, int device, cudaStream_t st)
+int mlp_dw_tc(int L, const int *dims, const int *pad, void *const *dZT, void *const *HT, int64_t rows, const MlpTrain &tr,
+              int nlp, float *const *part, float *const *gb, unsigned *err, int device, cudaStream_t st)
 {
-    constexpr size_t smem = 1024 + G_STAGES * (G_A_STAGE + W_STAGE_BYTES) + 128;
+    constexpr size_t smem = 1024 + 2 * G_STAGES * G_STAGE + 256;
     DwArgs A;
     memset(&A, 0, sizeof(A));
     A.L = L;
     A.kchunks = (int)((rows + KCHUNK - 1) / KCHUNK);
+    A.rows = rows;
+    A.ldT = tr.ldT;
+    A.Y = tr.Y;
+    A.T = tr.T;
+    A.nout = dims[L];
+    A.ldo = pad[L];
+    A.nlp = nlp;
+    A.lpart = tr.lpart;
+    A.next = tr.next;
     A.err = err;
     int tiles = 0;
     for (int l = 0; l < L; ++l) {
         DwLayer &Y = A.l[l];
         Y.M = pad[l + 1];
         Y.N = pad[l];
-        if (Y.N < 16 || Y.N > MAX_N || Y.N % 16) return -1;
+        if (Y.N < 16 || Y.N > 2 * G_COLS || Y.N % 16) return -1;
         Y.tile0 = tiles;
-        tiles += (Y.M + TILE_M - 1) / TILE_M;
+        Y.nt = (Y.N + G_COLS - 1) / G_COLS;
+        tiles += (Y.M + TILE_M - 1) / TILE_M * Y.nt;
+        mlp_dw_parts(Y.M, rows, device, &Y.kcs, &Y.splits);
         Y.part = part[l];
-        Y.partb = partb[l];
-        if (!kmajor_map(&Y.ma, dZT[l], Y.M, rows, ldT, TILE_M) || !kmajor_map(&Y.mb, HT[l], Y.N, rows, ldT, Y.N)) return -1;
+        Y.dZT = (const __nv_bfloat16 *)dZT[l];
+        Y.gb = gb[l];
+        Y.row0 = A.sum_rows;
+        A.sum_rows += dims[l + 1];
+        if (!kmajor_map(&Y.ma, dZT[l], Y.M, rows, tr.ldT, TILE_M) ||
+            !kmajor_map(&Y.mb, HT[l], Y.N, rows, tr.ldT, std::min(Y.N, G_COLS)))
+            return -1;
     }
-    const int splits = dw_splits(rows, tiles, device, &A.kcs);
+    // the sums start at once on the SMs that the tiles leave over
+    int sms = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    A.free_ctas = std::max(0, sms - tiles * DW_PARTS);
     static bool configured = false;
     if (!configured) {
         cudaFuncSetAttribute(k_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         configured = true;
     }
-    k_dw_tc<<<dim3((unsigned)tiles, (unsigned)splits), G_THREADS, smem, st>>>(A);
+    k_dw_tc<<<(unsigned)(A.free_ctas + tiles * DW_PARTS), G_THREADS, smem, st>>>(A);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1058,7 +1176,6 @@ bool fused_setup(int L, const int *pad, void *const *W, int64_t rows, unsigned *
     return true;
 }
 
-// Returns the number of CTAs, or -1.
 template <int MODE>
 int fused_launch(const Maps &maps, const Params &P, int device, cudaStream_t st)
 {
@@ -1073,7 +1190,7 @@ int fused_launch(const Maps &maps, const Params &P, int device, cudaStream_t st)
     const int64_t ntiles = (P.rows + TILE_M - 1) / TILE_M;
     const int grid = (int)std::min<int64_t>(ntiles, (int64_t)sms);
     k_mlp_tc<MODE><<<grid, THREADS, smem, st>>>(maps, P);
-    return cudaGetLastError() == cudaSuccess ? grid : -1;
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace
@@ -1087,7 +1204,7 @@ int mlp_forward_tc(int L, const int *dims, const int *pad, void *const *W, const
     for (int l = 0; l < L; ++l) P.layer[l].bias = bias[l];
     P.X = X;
     P.in_cols = dims[0];
-    P.Y = Y;
+    P.Y = tr ? tr->Y : Y;
     P.out_cols = dims[L];
     if (!tr) return fused_launch<INFER>(maps, P, device, st);
     for (int l = 0; l < L; ++l) {
@@ -1100,7 +1217,7 @@ int mlp_forward_tc(int L, const int *dims, const int *pad, void *const *W, const
     P.scale = tr->scale;
     P.dY = (__nv_bfloat16 *)tr->dY;
     P.dYT = (__nv_bfloat16 *)tr->dYT;
-    P.lpart = tr->lpart;
+    P.next = tr->next;
     return fused_launch<TRAIN_FWD>(maps, P, device, st);
 }
 
