@@ -234,47 +234,14 @@ __device__ __forceinline__ float rcp_approx(float x)
     return y;
 }
 
-// GELU of two values at once on packed FP32x2 instructions.  With a = |z|:
-//   GELU(z) = max(z, 0) - a Phi(-a),   Phi(-a) = erfc(a / sqrt 2) / 2 = 2^(-1 - R(a)),
-// where R(a) = -log2 erfc(a / sqrt 2) is smooth and zero at 0: a polynomial of degree 8
-// without a constant term, fitted here by linear programming to the smallest largest
-// error of erf over a <= 5.6 (5.9e-8); its leading coefficient is positive, so that it
-// keeps growing beyond.  One special-function instruction an element (ex2) where the
-// Abramowitz-Stegun form of gelu() needs two, (65,536 rows 68.9 -> 65.0 us, 49
-// rows 28.0 -> 26.0 us).
-// Error of GELU over |z| <= 12: at most 2.5e-7, RMS 2.0e-8 for normal z (3.8e-7 and
-// 4.0e-8 before).  n = -min(a, 2^15) keeps the product finite for infinite z; a NaN
-// goes through.
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float y;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-    return y;
-}
-__device__ __forceinline__ float2 gelu2(float2 z)
-{
-    const float2 n = make_float2(max_nan(-fabsf(z.x), -32768.f), max_nan(-fabsf(z.y), -32768.f));
-    // -1 - R as a polynomial in n = -a
-    float2 q = __ffma2_rn(make_float2(-1.33944366e-06f, -1.33944366e-06f), n, make_float2(-2.22031613e-05f, -2.22031613e-05f));
-    q = __ffma2_rn(q, n, make_float2(-0.000109909415f, -0.000109909415f));
-    q = __ffma2_rn(q, n, make_float2(0.000304504327f, 0.000304504327f));
-    q = __ffma2_rn(q, n, make_float2(0.00725635746f, 0.00725635746f));
-    q = __ffma2_rn(q, n, make_float2(0.0526092798f, 0.0526092798f));
-    q = __ffma2_rn(q, n, make_float2(-0.459178358f, -0.459178358f));
-    q = __ffma2_rn(q, n, make_float2(1.15110767f, 1.15110767f));
-    q = __ffma2_rn(q, n, make_float2(-1.0f, -1.0f));
-    const float2 phi = make_float2(ex2_approx(q.x), ex2_approx(q.y));
-    return __ffma2_rn(n, phi, make_float2(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f)));
-}
-
-// The training forward's GELU: the function whose derivative gelu_grad() takes, in the
-// same form (the special-function unit does not bound that epilogue).  Same method as
+// GELU of two values at once on packed FP32x2 instructions, in inference and in training
+// (a training step's loss is that of the network inference evaluates).  Same method as
 // gelu() below (Abramowitz & Stegun eq. 7.1.26 for erf, odd extension):
 //   x = |z|/sqrt2, t = 1/(1 + p x), e = erf(x) = 1 - t P(t) exp(-x^2),
 //   GELU = z/2 (1 + sign(z) e); the Horner coefficients carry the minus sign so
 //   that e is one fused multiply-add, and sign(z) e is e with z's sign bit
 //   (e >= 0).  exp(-x^2) = 2^(-x^2 log2 e) on the hardware ex2.
-__device__ __forceinline__ float2 gelu2_train(float2 z)
+__device__ __forceinline__ float2 gelu2(float2 z)
 {
     const float2 c = make_float2(0.70710678118654752f, 0.70710678118654752f);
     float2 x = __fmul2_rn(z, c);
@@ -392,7 +359,7 @@ __device__ __forceinline__ void epi_train8(const float (&bb)[8], const uint32_t 
         const float2 zz = __fadd2_rn(make_float2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])),
                                      make_float2(bb[e], bb[e + 1]));
         z[e / 2] = pack_bf16x2(zz.x, zz.y);
-        const float2 g2 = gelu2_train(zz);
+        const float2 g2 = gelu2(zz);
         pk[e / 2] = pack_bf16x2(g2.x, g2.y);
         store_pair_T(P.HT[l + 1], P.ldT, c + e, row, (row & ~(int64_t)1) < P.rows, pk[e / 2]);
     }

@@ -102,3 +102,17 @@ def test_sums_over_the_batch_keep_their_order(dims, rows):
     assert loss == loss_sum(-T, pad[1])
     assert np.array_equal(g[dims[0] * dims[1]:], bias_sum(z))
     assert np.array_equal(g[:dims[0] * dims[1]].reshape(dims[1], dims[0]), weight_sum(z, X, size))
+
+
+@pytest.mark.parametrize("rows", [3, 129, 4099])
+@pytest.mark.parametrize("dims", [(109, 256, 256, 6), (30, 64, 3), (256, 128, 256, 20)])
+def test_the_training_loss_is_that_of_the_inference_output(dims, rows):
+    from paper_2506_05362_gb300 import pd
+    rng = np.random.default_rng(rows)
+    net = pd.MLP(dims, seed=rows)
+    net.set_forward_path(2)
+    X = rng.normal(0, 2, (rows, dims[0])).astype(f32)
+    T = rng.normal(0, 1, (rows, dims[-1])).astype(f32)
+    loss, _ = net.grad(X, T)
+    assert loss == loss_sum(net.forward(X) - T, -(-dims[-1] // 16) * 16)
+    net.close()
