@@ -711,6 +711,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
                         }
                     }
                     if (!last) {
+                        // The next layer's MMAs read whole chunks of 64 columns.  Those past N
+                        // meet zero weights, but zero times what an earlier kernel or tile left
+                        // there (an infinity, a NaN) is not zero: they are cleared.
+                        const int cz = (Ly.N + 31) & ~31;  // up to here columns are written above
+                        if (cz & 32) *(uint4 *)(sA + sw128_offset(m, cz + 8 * part)) = make_uint4(0u, 0u, 0u, 0u);
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         mbar_arrive(a_ready + b);
