@@ -543,12 +543,14 @@ pd_status malloc_(pd_mlp *m, T **p, int64_t count)
     return PD_OK;
 }
 
-void mfree(pd_mlp *m, void *p)
+template <typename T>
+void mfree(pd_mlp *m, T *&p)
 {
     if (!p) return;
     for (size_t q = 0; q < m->owned.size(); ++q)
         if (m->owned[q] == p) { m->owned.erase(m->owned.begin() + q); break; }
     cudaFree(p);
+    p = nullptr;
 }
 
 int grid1(int64_t n)
@@ -576,13 +578,23 @@ pd_status pack_all(pd_mlp *m)
     return PD_OK;
 }
 
+// Whether the buffers of training are there (a larger forward takes them away).
+bool can_train(const pd_mlp *m)
+{
+    for (int l = 0; l < m->L; ++l)
+        if (!m->dZ[l] || !m->HT[l] || !m->dZT[l] || (l + 1 < m->L && !m->Z[l])) return false;
+    return true;
+}
+
+// Buffers for batches of `rows` rows.  None is left behind half made: while they are being
+// replaced the capacity is zero.
 pd_status ensure_cap(pd_mlp *m, int64_t rows, bool train)
 {
-    if (rows <= m->cap && (!train || m->Z[0] || m->L == 1)) return PD_OK;
-    int64_t cap = std::max<int64_t>(rows, m->cap);
-    for (int l = 0; l <= m->L; ++l) { mfree(m, m->H[l]); m->H[l] = nullptr; mfree(m, m->dZ[l]); m->dZ[l] = nullptr; }
-    for (int l = 0; l < m->L; ++l) { mfree(m, m->HT[l]); m->HT[l] = nullptr; mfree(m, m->dZT[l]); m->dZT[l] = nullptr; }
-    for (int l = 0; l < m->L; ++l) { mfree(m, m->Z[l]); m->Z[l] = nullptr; }
+    if (rows <= m->cap && (!train || can_train(m))) return PD_OK;
+    const int64_t cap = std::max<int64_t>(rows, m->cap);
+    m->cap = 0;
+    for (int l = 0; l <= m->L; ++l) { mfree(m, m->H[l]); mfree(m, m->dZ[l]); }
+    for (int l = 0; l < m->L; ++l) { mfree(m, m->HT[l]); mfree(m, m->dZT[l]); mfree(m, m->Z[l]); }
     mfree(m, m->Y); mfree(m, m->Xf); mfree(m, m->Tf); mfree(m, m->lpart);
     pd_status s;
     for (int l = 0; l < m->L; ++l)
@@ -654,8 +666,8 @@ void adam_constants(pd_mlp *m, float *b1, float *b2, float *eps, float *c1, floa
 pd_status ensure_part(pd_mlp *m, int64_t need)
 {
     if (need <= m->part_cap) return PD_OK;
+    m->part_cap = 0;
     mfree(m, m->part);
-    m->part = nullptr;
     pd_status s = malloc_(m, &m->part, need);
     if (s) return s;
     m->part_cap = need;
@@ -753,13 +765,7 @@ pd_status backward_dev(pd_mlp *m, const float *X, const float *T, int64_t rows, 
         int splits = (int)std::max<int64_t>(1, std::min<int64_t>(128, rows / 512));
         int64_t ks = ((rows + splits - 1) / splits + BK - 1) / BK * BK;
         splits = (int)((rows + ks - 1) / ks);
-        int64_t need = (int64_t)splits * N * K;
-        if (need > m->part_cap) {
-            mfree(m, m->part);
-            m->part = nullptr;
-            if ((s = malloc_(m, &m->part, need))) return s;
-            m->part_cap = need;
-        }
+        if ((s = ensure_part(m, (int64_t)splits * N * K))) return s;
         GemmArgs g;
         memset(&g, 0, sizeof(g));
         g.M = N; g.N = K; g.K = (int)rows;
@@ -942,6 +948,7 @@ static pd_status grad_impl(pd_mlp *m, const float *Xd, const float *Td, int64_t 
 {
     pd_status s = ensure_cap(m, batch, true);
     if (s) return s;
+    if (batch > m->cap || !can_train(m)) return mfail(m, PD_ECUDA, "the training buffers are missing");
     return backward_dev(m, Xd, Td, batch, lr, loss2);
 }
 
