@@ -40,6 +40,24 @@ __device__ __forceinline__ int32_t ld_slot(const int32_t *a)
     return v;
 }
 
+// LIVE: memory that the same launch also writes (the displacement records and the flagged
+// neighbour indices in the multi-step kernel), which the read-only path may not load:
+// ordinary loads, ordered by the grid barrier between the steps (the 4,139-node sphere 2.81 ->
+// 2.84 ms for 200 steps).
+template <bool LIVE>
+__device__ __forceinline__ float4 ld_u(const float4 *a)
+{
+    return LIVE ? *a : __ldg(a);
+}
+template <bool LIVE>
+__device__ __forceinline__ int32_t ld_colf(const int32_t *a)
+{
+    if (!LIVE) return ld_slot(a);
+    int32_t v;
+    asm volatile("ld.global.L1::no_allocate.b32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+    return v;
+}
+
 // a slot's bond lengths on the FP64 path: streamed once per step, past L1
 __device__ __forceinline__ double2 ld_len(const double2 *a)
 {
@@ -360,24 +378,31 @@ __device__ __forceinline__ void xl_unpack(float w1, float w2, float *xl)
 
 // The three record slots of neighbour j (mixed path), in the layout PD_PLANES
 // selects: (x_hi, c V), (u_hi, x_lo.xy packed), (u_lo, x_lo.z packed).
+template <bool LIVE = false>
 __device__ __forceinline__ void gather_record(const StepParams &p, int32_t j, float4 &a0, float4 &a1, float4 &a2)
 {
 #if PD_PLANES == 2
     a0 = __ldg(p.xh4 + j);
     // the node's u pair is 32-byte aligned (u0 even): one 256-bit read-only load
     const float4 *q = p.uh_in + 2 * (int64_t)j;
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a1.x), "=f"(a1.y), "=f"(a1.z), "=f"(a1.w), "=f"(a2.x), "=f"(a2.y), "=f"(a2.z), "=f"(a2.w)
-        : "l"(q));
+    if (LIVE)
+        asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(a1.x), "=f"(a1.y), "=f"(a1.z), "=f"(a1.w), "=f"(a2.x), "=f"(a2.y), "=f"(a2.z), "=f"(a2.w)
+                     : "l"(q)
+                     : "memory");
+    else
+        asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(a1.x), "=f"(a1.y), "=f"(a1.z), "=f"(a1.w), "=f"(a2.x), "=f"(a2.y), "=f"(a2.z), "=f"(a2.w)
+            : "l"(q));
 #elif PD_PLANES == 1
     a0 = __ldg(p.xh4 + j);
-    a1 = __ldg(p.uh_in + j);
-    a2 = __ldg(p.ul_in + j);
+    a1 = ld_u<LIVE>(p.uh_in + j);
+    a2 = ld_u<LIVE>(p.ul_in + j);
 #else
     const float4 *r = p.xh4 + 3 * (int64_t)j;  // one 48-byte record
     a0 = __ldg(r);
-    a1 = __ldg(r + 1);
-    a2 = __ldg(r + 2);
+    a1 = ld_u<LIVE>(r + 1);
+    a2 = ld_u<LIVE>(r + 2);
 #endif
 }
 
@@ -711,9 +736,10 @@ __device__ __forceinline__ void undeformed(const StepParams &p, const dbl4 &ox, 
 // In FP32, whether the row's node (records o0, o1) and node j are too far apart to touch.
 // Each difference of the records' high halves is off by at most 2^-24 of itself, and the low
 // halves left out are at most 2^-24 of x and u; the margins below are four times that.
+template <bool LIVE>
 __device__ __forceinline__ bool clearly_apart(const StepParams &p, const float4 &o0, const float4 &o1, int j)
 {
-    const float4 a0 = __ldg(p.xh4 + RECX * (int64_t)j), a1 = __ldg(p.uh_in + REC * (int64_t)j);
+    const float4 a0 = __ldg(p.xh4 + RECX * (int64_t)j), a1 = ld_u<LIVE>(p.uh_in + REC * (int64_t)j);
     const float x0 = a0.x - o0.x, x1 = a0.y - o0.y, x2 = a0.z - o0.z;
     const float u0 = a1.x - o1.x, u1 = a1.y - o1.y, u2 = a1.z - o1.z;
     const float ex = x0 + u0, ey = x1 + u1, ez = x2 + u2;
@@ -727,7 +753,7 @@ __device__ __forceinline__ bool clearly_apart(const StepParams &p, const float4 
 // normal damping of Sec. 3.3): false when the pair does not touch or is still
 // bonded; otherwise (gx, gy, gz) = its force density on i.  The predicate is
 // evaluated in FP64 without FMA, so contact pair sets are exact.
-template <bool MIXED>
+template <bool MIXED, bool LIVE>
 __device__ __forceinline__ bool contact_term(const StepParams &p, int64_t q, const float4 &o0, const float4 &o1,
                                              const dbl4 &ox, double pix, double piy, double piz, int gi, double R2,
                                              double &gx, double &gy, double &gz)
@@ -740,7 +766,7 @@ __device__ __forceinline__ bool contact_term(const StepParams &p, int64_t q, con
     }
     if (MIXED) {
         // FP32 first: a pair that is clearly apart needs no FP64 (that pipe is narrow)
-        if (clearly_apart(p, o0, o1, j)) return false;
+        if (clearly_apart<LIVE>(p, o0, o1, j)) return false;
     }
     const dbl4 xj = p.x4[j], uj = load_u_t<MIXED>(p, j);
     const double dx = dadd(xj.x, uj.x) - pix;
@@ -782,7 +808,7 @@ __device__ __forceinline__ bool contact_term(const StepParams &p, int64_t q, con
 // touching pairs alone in ascending partner order: an evaluation at a given state
 // gives the same bits whichever rebuild (and skin superset) made the list.  All
 // lanes of the warp call it (inactive rows with active = false).
-template <int G, bool MIXED>
+template <int G, bool MIXED, bool LIVE>
 __device__ __forceinline__ void contact_sum(const StepParams &p, int64_t row, bool active, int gl, double &cx,
                                             double &cy, double &cz)
 {
@@ -803,7 +829,7 @@ __device__ __forceinline__ void contact_sum(const StepParams &p, int64_t row, bo
     if (nch > 0) {
         if (MIXED) {
             o0 = __ldg(p.xh4 + RECX * row);
-            o1 = __ldg(p.uh_in + REC * row);
+            o1 = ld_u<LIVE>(p.uh_in + REC * row);
         }
         ox = p.x4[row];
         const dbl4 ou = load_u_t<MIXED>(p, row);
@@ -814,7 +840,7 @@ __device__ __forceinline__ void contact_sum(const StepParams &p, int64_t row, bo
     for (int t = 0; t < nmax; ++t) {
         const int64_t q = c0 + (int64_t)t * G + gl;
         double gx = 0.0, gy = 0.0, gz = 0.0;
-        const bool touch = q < c1 && contact_term<MIXED>(p, q, o0, o1, ox, pix, piy, piz, gi, R2, gx, gy, gz);
+        const bool touch = q < c1 && contact_term<MIXED, LIVE>(p, q, o0, o1, ox, pix, piy, piz, gi, R2, gx, gy, gz);
         if (!touch) gx = gy = gz = 0.0;
         // in ascending order, passing over the places where no group of the warp touches
         // (adding their zeros changes nothing)
@@ -856,7 +882,7 @@ __device__ __forceinline__ void load_v_t(const StepParams &p, int64_t i, double 
 // step kernel (which updates v in place) reads a consistent half-step velocity
 // field.  Candidates that do not touch are left out: the step kernel reads the term only
 // of pairs that do, by the same test.
-template <bool MIXED>
+template <bool MIXED, bool LIVE>
 __device__ __forceinline__ void pair_damping_rows(const StepParams &p, int64_t first, int64_t stride)
 {
     const double R2 = dmul(p.Rc, p.Rc);
@@ -876,7 +902,7 @@ __device__ __forceinline__ void pair_damping_rows(const StepParams &p, int64_t f
         load_v_t<MIXED>(p, i, vix, viy, viz);
         for (int64_t q = c0; q < c1; ++q) {
             const int j = p.cand[q].x;
-            if (MIXED && clearly_apart(p, o0, o1, j)) continue;
+            if (MIXED && clearly_apart<LIVE>(p, o0, o1, j)) continue;
             const dbl4 xj = p.x4[j], uj = load_u_t<MIXED>(p, j);
             const double dx = dadd(xj.x, uj.x) - pix;
             const double dy = dadd(xj.y, uj.y) - piy;
@@ -932,7 +958,7 @@ __device__ __forceinline__ void pair_damping_rows(const StepParams &p, int64_t f
 template <bool MIXED>
 __global__ void k_pair_damping(const StepParams p)
 {
-    pair_damping_rows<MIXED>(p, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+    pair_damping_rows<MIXED, false>(p, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // Tile staging of the mixed path: the records of the nodes a tile touches.
@@ -942,8 +968,9 @@ struct TileView {
 };
 
 // Steps 1-4 for one row owned by a group of G lanes (all lanes call; inactive
-// groups pass active = false and still join the shuffles).
-template <int G, bool MIXED, bool WX = false, bool PAIRS = false, bool EARLY = false>
+// groups pass active = false and still join the shuffles).  LIVE: the multi-step kernel,
+// which also loads the row's velocity at the start of the row.
+template <int G, bool MIXED, bool WX = false, bool PAIRS = false, bool LIVE = false>
 __device__ __forceinline__ void process_row(const StepParams &p, const double *wp, const WallF *wf, int64_t row, bool active, int gl,
                                             int lrow,
                                             const TileView &tv, double *react, unsigned &err, float &vmax2f,
@@ -954,7 +981,7 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
     float fbx = 0.f, fby = 0.f, fbz = 0.f;
     double fdx = 0.0, fdy = 0.0, fdz = 0.0;
     float4 ovh = make_float4(0.f, 0.f, 0.f, 0.f), ovl = ovh;
-    if (EARLY && MIXED && active && (gl < 3 || p.walls.nw)) {
+    if (LIVE && MIXED && active && (gl < 3 || p.walls.nw)) {
         ovh = p.vh[row];
         ovl = p.vl[row];
     }
@@ -995,7 +1022,8 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                 }
             }
         } else if (MIXED) {
-            const float4 o0 = __ldg(p.xh4 + RECX * row), o1 = __ldg(p.uh_in + REC * row), o2 = __ldg(p.ul_in + REC * row);
+            const float4 o0 = __ldg(p.xh4 + RECX * row), o1 = ld_u<LIVE>(p.uh_in + REC * row),
+                         o2 = ld_u<LIVE>(p.ul_in + REC * row);
             float ol[3];
             xl_unpack(o1.w, o2.w, ol);
             const int i0 = (int)k0, i1 = (int)k1;
@@ -1011,7 +1039,7 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                 for (int q = 0; q < PD_INFLIGHT_PF; ++q) {
                     // a slot past the row end gathers the first slot's node, flagged
                     const int kq = k + q * G;
-                    raw[q] = kq < i1 ? ld_slot(p.colf + kq)
+                    raw[q] = kq < i1 ? ld_colf<LIVE>(p.colf + kq)
                                      : (q == 0 ? (int32_t)0x80000000u : (int32_t)((uint32_t)raw[0] | 0x80000000u));
                 }
             }
@@ -1019,7 +1047,7 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                 float4 a0[PD_INFLIGHT_PF], a1[PD_INFLIGHT_PF], a2[PD_INFLIGHT_PF];
 #pragma unroll
                 for (int q = 0; q < PD_INFLIGHT_PF; ++q) {
-                    gather_record(p, raw[q] & 0x7fffffff, a0[q], a1[q], a2[q]);
+                    gather_record<LIVE>(p, raw[q] & 0x7fffffff, a0[q], a1[q], a2[q]);
                 }
                 int32_t nxt[PD_INFLIGHT_PF];
 #pragma unroll
@@ -1027,7 +1055,7 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                     // a slot past the row end gathers this batch's first node (a
                     // neighbour of the row), flagged: no force
                     const int kq = k + (PD_INFLIGHT_PF + q) * G;
-                    nxt[q] = kq < i1 ? ld_slot(p.colf + kq) : (int32_t)((uint32_t)raw[0] | 0x80000000u);
+                    nxt[q] = kq < i1 ? ld_colf<LIVE>(p.colf + kq) : (int32_t)((uint32_t)raw[0] | 0x80000000u);
                 }
 #pragma unroll
                 for (int q = 0; q < PD_INFLIGHT_PF; ++q)
@@ -1042,13 +1070,13 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                 for (int q = 0; q < PD_INFLIGHT; ++q) {
                     // a slot past the row end reuses the first slot's node, flagged
                     const int kq = k + q * G;
-                    raw[q] = q == 0 ? ld_slot(p.colf + kq)
-                                    : (kq < i1 ? ld_slot(p.colf + kq) : (int32_t)((uint32_t)raw[0] | 0x80000000u));
+                    raw[q] = q == 0 ? ld_colf<LIVE>(p.colf + kq)
+                                    : (kq < i1 ? ld_colf<LIVE>(p.colf + kq) : (int32_t)((uint32_t)raw[0] | 0x80000000u));
                 }
                 float4 a0[PD_INFLIGHT], a1[PD_INFLIGHT], a2[PD_INFLIGHT];
 #pragma unroll
                 for (int q = 0; q < PD_INFLIGHT; ++q) {
-                    gather_record(p, raw[q] & 0x7fffffff, a0[q], a1[q], a2[q]);
+                    gather_record<LIVE>(p, raw[q] & 0x7fffffff, a0[q], a1[q], a2[q]);
                 }
 #pragma unroll
                 for (int q = 0; q < PD_INFLIGHT; ++q)
@@ -1084,7 +1112,7 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
     __syncwarp();
     // ---- 2. contact candidates (FP64, exact predicate, ordered sum)
     double cx, cy, cz;
-    contact_sum<G, MIXED>(p, row, active, gl, cx, cy, cz);
+    contact_sum<G, MIXED, LIVE>(p, row, active, gl, cx, cy, cz);
     // ---- 3. combine the group, then add pass 1's part (each bond once) and the contact sum
     if (MIXED) {
         fbx = group_sum<G>(fbx);
@@ -1108,8 +1136,10 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
     if (MIXED) {
         float4 oxh = make_float4(0.f, 0.f, 0.f, 0.f), ouh = oxh, oul = oxh;
         if (active && (gl < 3 || p.walls.nw)) {
-            oxh = __ldg(p.xh4 + RECX * row); ouh = __ldg(p.uh_in + REC * row); oul = __ldg(p.ul_in + REC * row);
-            if (!EARLY) {
+            oxh = __ldg(p.xh4 + RECX * row);
+            ouh = ld_u<LIVE>(p.uh_in + REC * row);
+            oul = ld_u<LIVE>(p.ul_in + REC * row);
+            if (!LIVE) {
                 ovh = p.vh[row];
                 ovl = p.vl[row];
             }
@@ -1389,7 +1419,7 @@ __device__ __forceinline__ bool persist_step(const StepParams &p, int step, unsi
     constexpr int GPB = STEP_THREADS / G;
     const int gl = threadIdx.x % G, grp = threadIdx.x / G;
     if (p.pair_diss && p.contact && p.cand_fd) {  // damping and friction of the candidates first
-        pair_damping_rows<MIXED>(p, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+        pair_damping_rows<MIXED, true>(p, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
         if (!grid_barrier(bar, ++nbar * arrivals, p.err, &s_ok)) return false;
     }
     __shared__ WallF s_wf[PD_MAX_WALLS];
@@ -1575,7 +1605,7 @@ __global__ void __launch_bounds__(STEP_THREADS, PD_MINB_TILED) k_step_tiled(cons
             __syncwarp();
             // contact candidates (rare; FP64 from global memory, ordered sum)
             double cx, cy, cz;
-            contact_sum<G, true>(p, row, active, gl, cx, cy, cz);
+            contact_sum<G, true, false>(p, row, active, gl, cx, cy, cz);
             fbx = group_sum<G>(fbx) + (float)cx;
             fby = group_sum<G>(fby) + (float)cy;
             fbz = group_sum<G>(fbz) + (float)cz;
