@@ -416,8 +416,11 @@ pd_status pd_mlp_create(const int *dims, int nlayers, uint64_t seed, int device,
 /* Y (batch x dims[nlayers], FP32) = MLP(X); X (batch x dims[0], FP32) is
  * rounded to BF16 (nearest-even). Host pointers. */
 pd_status pd_mlp_forward(pd_mlp *m, const float *X, int64_t batch, float *Y);
-/* Same with device pointers (no copies, no synchronisation; a tensor-core
- * wait that gave up is reported by the next pd_mlp_forward). */
+/* Same with device pointers (no copies, no synchronisation).  A wait of a
+ * tensor-core kernel that gave up, here or in pd_mlp_train_step_device, is
+ * reported as PD_ETIMEOUT by the next pd_mlp_forward, pd_mlp_grad,
+ * pd_mlp_train_step or pd_mlp_get_params, once; until then Adam steps leave the
+ * weights as they are (a device loss is NaN), and results are void. */
 pd_status pd_mlp_forward_device(pd_mlp *m, const float *X, int64_t batch, float *Y);
 /* Forward kernels: 0 (default) = the fused tcgen05 kernel (TMA-fed weights,
  * TMEM accumulators, activations kept in shared memory across layers) when
@@ -429,6 +432,9 @@ pd_status pd_mlp_forward_device(pd_mlp *m, const float *X, int64_t batch, float 
  * tcgen05 GEMMs, hidden widths multiples of 32), 1 on the mma.sync GEMMs.
  * PD_EINVAL for any other value. */
 pd_status pd_mlp_set_forward_path(pd_mlp *m, int path);
+/* Test aid: marks a wait as given up (see pd_mlp_forward_device), which makes the
+ * next reporting call fail without one. */
+pd_status pd_mlp_mark_timeout(pd_mlp *m);
 /* One Adam step on the MSE loss of (X, T); *loss receives the loss before the
  * update (nullable).  Host pointers. */
 pd_status pd_mlp_train_step(pd_mlp *m, const float *X, const float *T, int64_t batch, float lr,

@@ -381,9 +381,19 @@ __device__ __forceinline__ float adam_step(float w, float g, float &m, float &v,
     return w - lr * (m / c1) / (sqrtf(v / c2) + eps);
 }
 
-__global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
-                       int64_t n, float lr, float b1, float b2, float eps, float c1, float c2)
+// A step whose sums are not all there (err[0]: a wait of a tensor-core kernel gave up) leaves
+// weights and moments as they are and is counted in err[2].
+__device__ __forceinline__ bool step_is_void(unsigned *err)
 {
+    if (!*err) return false;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ++err[2];
+    return true;
+}
+
+__global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
+                       int64_t n, float lr, float b1, float b2, float eps, float c1, float c2, unsigned *err)
+{
+    if (step_is_void(err)) return;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
         w[q] = adam_step(w[q], g[q], m[q], v[q], lr, b1, b2, eps, c1, c2);
     }
@@ -415,6 +425,7 @@ struct Update {
     int nlp;
     int64_t lcount;
     float *loss, *loss2;        // loss2 nullable
+    unsigned *err;
 };
 
 __global__ void __launch_bounds__(256) k_update(const __grid_constant__ Update U)
@@ -430,11 +441,12 @@ __global__ void __launch_bounds__(256) k_update(const __grid_constant__ Update U
             __syncthreads();
         }
         if (threadIdx.x == 0) {
-            const float loss = (float)(sd[0] / (double)U.lcount);
+            const float loss = *U.err ? NAN : (float)(sd[0] / (double)U.lcount);
             *U.loss = loss;
             if (U.loss2) *U.loss2 = loss;
         }
     }
+    if (U.adam && step_is_void(U.err)) return;
     const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (p >= U.nparams) return;
     int l = 0;
@@ -506,7 +518,7 @@ struct pd_mlp {
     int64_t part_cap = 0;
     float *lpart = nullptr, *dloss = nullptr;
     unsigned *tc_err = nullptr;  // error word of the tcgen05 kernels
-    unsigned *next = nullptr;    // task counter of k_dw_tc
+    unsigned *next = nullptr;    // task counter of k_dw_tc, = tc_err + 1; tc_err[2]: void Adam steps
     int path = 0;                // 0: tcgen05 forward when the shapes allow; 1: mma.sync only
     std::vector<void *> owned;
 };
@@ -663,6 +675,19 @@ void adam_constants(pd_mlp *m, float *b1, float *b2, float *eps, float *c1, floa
     *c2 = (float)(1.0 - pow(0.999, (double)m->t));
 }
 
+// Waits for the stream.  A wait of a tensor-core kernel that gave up since the last such call
+// is reported here, once: the results since then are void, the Adam steps not taken.
+pd_status finish(pd_mlp *m)
+{
+    unsigned e[3] = {0, 0, 0};
+    MCK(cudaMemcpyAsync(e, m->tc_err, sizeof(e), cudaMemcpyDeviceToHost, m->st));
+    MCK(cudaStreamSynchronize(m->st));
+    if (!e[0]) return PD_OK;
+    m->t -= e[2];
+    MCK(cudaMemsetAsync(m->tc_err, 0, sizeof(e), m->st));
+    return mfail(m, PD_ETIMEOUT, "a bounded wait of a tensor-core kernel gave up");
+}
+
 pd_status ensure_part(pd_mlp *m, int64_t need)
 {
     if (need <= m->part_cap) return PD_OK;
@@ -738,6 +763,7 @@ int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float l
     }
     U.lpart = m->lpart; U.nlp = nlp; U.lcount = rows * nout;
     U.loss = m->dloss; U.loss2 = loss2;
+    U.err = m->tc_err;
     k_update<<<(unsigned)((m->nparams + 255) / 256), 256, 0, m->st>>>(U);
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
@@ -796,7 +822,7 @@ pd_status backward_dev(pd_mlp *m, const float *X, const float *T, int64_t rows, 
         float b1, b2, eps, c1, c2;
         adam_constants(m, &b1, &b2, &eps, &c1, &c2);
         k_adam<<<grid1(m->nparams), 256, 0, m->st>>>(m->master, m->grad, m->m, m->v, m->nparams, lr, b1, b2, eps, c1,
-                                                     c2);
+                                                     c2, m->tc_err);
         return pack_all(m);
     }
     return PD_OK;
@@ -831,7 +857,7 @@ pd_status pd_mlp_create(const int *dims, int nlayers, uint64_t seed, int device,
     pd_status s = PD_OK;
     if (cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); delete m; return PD_ECUDA; }
     if ((s = malloc_(m, &m->master, off)) || (s = malloc_(m, &m->m, off)) || (s = malloc_(m, &m->v, off)) ||
-        (s = malloc_(m, &m->grad, off)) || (s = malloc_(m, &m->dloss, 4)) || (s = malloc_(m, &m->tc_err, 2))) {
+        (s = malloc_(m, &m->grad, off)) || (s = malloc_(m, &m->dloss, 4)) || (s = malloc_(m, &m->tc_err, 3))) {
         pd_mlp_destroy(m);
         return s;
     }
@@ -844,7 +870,7 @@ pd_status pd_mlp_create(const int *dims, int nlayers, uint64_t seed, int device,
         }
     }
     m->next = m->tc_err + 1;
-    if (cudaMemsetAsync(m->tc_err, 0, 2 * sizeof(unsigned), m->st) != cudaSuccess) {
+    if (cudaMemsetAsync(m->tc_err, 0, 3 * sizeof(unsigned), m->st) != cudaSuccess) {
         cudaGetLastError();
         pd_mlp_destroy(m);
         return PD_ECUDA;
@@ -892,6 +918,7 @@ pd_status pd_mlp_set_params(pd_mlp *m, const float *w)
     MCK(cudaMemcpyAsync(m->master, w, sizeof(float) * m->nparams, cudaMemcpyHostToDevice, m->st));
     MCK(cudaMemsetAsync(m->m, 0, sizeof(float) * m->nparams, m->st));
     MCK(cudaMemsetAsync(m->v, 0, sizeof(float) * m->nparams, m->st));
+    MCK(cudaMemsetAsync(m->tc_err + 2, 0, sizeof(unsigned), m->st));  // the steps counted there are of the old weights
     m->t = 0;
     pd_status s = pack_all(m);
     if (s) return s;
@@ -904,8 +931,7 @@ pd_status pd_mlp_get_params(pd_mlp *m, float *w)
     if (!m || !w) return PD_EINVAL;
     MCK(cudaSetDevice(m->device));
     MCK(cudaMemcpyAsync(w, m->master, sizeof(float) * m->nparams, cudaMemcpyDeviceToHost, m->st));
-    MCK(cudaStreamSynchronize(m->st));
-    return PD_OK;
+    return finish(m);
 }
 
 pd_status pd_mlp_forward_device(pd_mlp *m, const float *X, int64_t batch, float *Y)
@@ -927,13 +953,14 @@ pd_status pd_mlp_forward(pd_mlp *m, const float *X, int64_t batch, float *Y)
     s = forward_dev(m, m->Xf, batch, m->Y, false);
     if (s) return s;
     MCK(cudaMemcpyAsync(Y, m->Y, sizeof(float) * batch * m->dims[m->L], cudaMemcpyDeviceToHost, m->st));
-    unsigned e = 0;
-    MCK(cudaMemcpyAsync(&e, m->tc_err, sizeof(unsigned), cudaMemcpyDeviceToHost, m->st));
-    MCK(cudaStreamSynchronize(m->st));
-    if (e) {
-        cudaMemsetAsync(m->tc_err, 0, sizeof(unsigned), m->st);
-        return mfail(m, PD_ETIMEOUT, "a bounded wait of the tensor-core forward gave up");
-    }
+    return finish(m);
+}
+
+pd_status pd_mlp_mark_timeout(pd_mlp *m)
+{
+    if (!m) return PD_EINVAL;
+    MCK(cudaSetDevice(m->device));
+    MCK(cudaMemsetAsync(m->tc_err, 1, 1, m->st));
     return PD_OK;
 }
 
@@ -964,8 +991,7 @@ pd_status pd_mlp_grad(pd_mlp *m, const float *X, const float *T, int64_t batch, 
     if (s) return s;
     MCK(cudaMemcpyAsync(grad, m->grad, sizeof(float) * m->nparams, cudaMemcpyDeviceToHost, m->st));
     if (loss) MCK(cudaMemcpyAsync(loss, m->dloss, sizeof(float), cudaMemcpyDeviceToHost, m->st));
-    MCK(cudaStreamSynchronize(m->st));
-    return PD_OK;
+    return finish(m);
 }
 
 pd_status pd_mlp_train_step_device(pd_mlp *m, const float *X, const float *T, int64_t batch, float lr, float *loss)
@@ -986,8 +1012,7 @@ pd_status pd_mlp_train_step(pd_mlp *m, const float *X, const float *T, int64_t b
     s = grad_impl(m, m->Xf, m->Tf, batch, lr, nullptr);
     if (s) return s;
     if (loss) MCK(cudaMemcpyAsync(loss, m->dloss, sizeof(float), cudaMemcpyDeviceToHost, m->st));
-    MCK(cudaStreamSynchronize(m->st));
-    return PD_OK;
+    return finish(m);
 }
 
 }  // extern "C"

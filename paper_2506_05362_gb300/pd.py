@@ -119,6 +119,7 @@ def lib():
                 "pd_mlp_last_error": (ctypes.c_char_p, [P]),
                 "pd_mlp_destroy": (None, [P]),
                 "pd_mlp_set_forward_path": (i32, [P, i32]),
+                "pd_mlp_mark_timeout": (i32, [P]),
             }
             for name, (res, args) in sig.items():
                 if not hasattr(L, name):
