@@ -67,7 +67,7 @@ __device__ __forceinline__ double2 ld_len(const double2 *a)
 }
 
 // l = sqrt(a) and r = 1 / sqrt(a) from one approximate reciprocal root x0 (relative
-// error e0 below 2^-20): with e = 1 - a x0^2, 1 / sqrt(a) = x0 (1 - e)^(-1/2), and the
+// error e0 below 2^-20), a a normal number: with e = 1 - a x0^2, 1 / sqrt(a) = x0 (1 - e)^(-1/2), and the
 // binomial series to second order leaves 5/16 e^3, below 2^-58; l = a r then takes one
 // Newton correction.  The FP64 bond loop is bound by the FP64 pipe (2 lanes a clock an
 // SM): with sqrt and two divisions, and the undeformed length computed again in every
@@ -82,6 +82,24 @@ __device__ __forceinline__ void root64(double a, double &l, double &r)
     r = fma(x0 * e, fma(0.375, e, 0.5), x0);
     l = a * r;
     l = fma(fma(-l, l, a), 0.5 * r, l);
+}
+
+// The same for any a >= 0, infinity included, and NaN: outside 2^-900 .. 2^1024, where root64
+// has no approximate root or its corrections underflow, CUDA's root and division (a bond
+// whose ends meet has l = 0, r = infinity).  The range is told by the exponent's bits, off the
+// FP64 pipe.  A contact evaluation is a chain of dependent FP64 operations in one or two lanes
+// of a warp, the square root and the division half of it before: with this in their place a
+// step of the 47,808-node aggregate took 62.4 us instead of 65.7 (5,770 touching pairs; 55.4
+// with the end of a step split up since), its pair damping 12.4 us instead of 14.1.
+__device__ __forceinline__ void dist64(double a, double &l, double &r)
+{
+    constexpr unsigned LO = (unsigned)(1023 - 900) << 20, INF = 0x7ff00000u;
+    if ((unsigned)__double2hiint(a) - LO < INF - LO) {
+        root64(a, l, r);
+    } else {
+        l = sqrt(a);
+        r = 1.0 / l;
+    }
 }
 
 constexpr int STEP_THREADS = 256;
@@ -708,21 +726,6 @@ __device__ __forceinline__ unsigned epilogue_lanes(const StepParams &p, const do
     return err;
 }
 
-// l = sqrt(a), r = 1 / sqrt(a) for any a > 0 (root64 wants a normal number).  A contact
-// evaluation is a chain of dependent FP64 operations in one or two lanes of a warp, the
-// square root and the division half of it before: with this in their place a step of the
-// 47,808-node aggregate took 62.4 us instead of 65.7 (5,770 touching pairs; 55.4 with the
-// end of a step split up since), its pair damping 12.4 us instead of 14.1.
-__device__ __forceinline__ void dist64(double a, double &l, double &r)
-{
-    if (a > 1e-280) {
-        root64(a, l, r);
-    } else {
-        l = sqrt(a);
-        r = 1.0 / l;
-    }
-}
-
 // The undeformed distance of two nodes and its reciprocal.  Comparing it with R_c selects
 // the contact law, so beside R_c it is the correctly rounded root.
 __device__ __forceinline__ void undeformed(const StepParams &p, const dbl4 &ox, const dbl4 &xj, double &L, double &rL)
@@ -1095,7 +1098,7 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                              yz = (a.z - ox.z) + (c.z - ou.z);
                 const double l2 = fma(yx, yx, fma(yy, yy, yz * yz));
                 double l, rl;
-                root64(l2, l, rl);
+                dist64(l2, l, rl);
                 const double s = (l - len.x) * len.y;
                 const bool brk = p.break_mode ? (fabs(s) > p.s0) : (s > p.s0);
                 if (brk) {
