@@ -695,21 +695,6 @@ __global__ void k_sync_colf_flags(const uint32_t *__restrict__ brk, const int32_
         colf[k] = (int32_t)((uint32_t)col[k] | (((brk[k >> 5] >> (k & 31)) & 1u) << 31));
 }
 
-// |xi| and 1 / |xi| of every slot; a warp takes a row
-__global__ void k_bond_lengths(const dbl4 *__restrict__ x4, const int64_t *__restrict__ rowptr,
-                               const int32_t *__restrict__ col, int64_t n, double2 *len)
-{
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nwarps) {
-        const dbl4 a = x4[i];
-        for (int64_t k = rowptr[i] + (threadIdx.x & 31); k < rowptr[i + 1]; k += 32) {
-            const dbl4 b = x4[col[k]];
-            const double L = sqrt(sq3(dsub(b.x, a.x), dsub(b.y, a.y), dsub(b.z, a.z)));
-            len[k] = make_double2(L, 1.0 / L);
-        }
-    }
-}
-
 // Index arrays of the each-bond-once passes: split[i] = first slot of row i whose
 // neighbour index exceeds i (rows are sorted ascending); for each such slot k
 // (bond i -> j), mir[k] = the slot of i in row j, and mir of that slot = k.  A
@@ -1052,11 +1037,6 @@ void pair_index(const int64_t *rowptr, const int32_t *col, int64_t n, int32_t *s
                 cudaStream_t st)
 {
     k_pair_index<<<grid_of(n), 256, 0, st>>>(rowptr, col, n, split, mir, bad);
-}
-
-void bond_lengths(const dbl4 *x4, const int64_t *rowptr, const int32_t *col, int64_t n, double2 *len, cudaStream_t st)
-{
-    k_bond_lengths<<<grid_of(32 * n), 256, 0, st>>>(x4, rowptr, col, n, len);
 }
 
 void sync_colf_flags(const uint32_t *brk, const int32_t *col, int64_t B, int32_t *colf, cudaStream_t st)

@@ -184,6 +184,8 @@ int persist_blocks(int lanes, int device, bool mixed, bool wx);
 cudaError_t launch_persist(const StepParams &pa, const StepParams &pb, int nsteps, int lanes, int blocks,
                            unsigned *bar, unsigned absent, cudaStream_t st);
 void launch_drift(const StepParams &p, cudaStream_t st);
+// per slot (|xi|, 1 / |xi|) for the FP64 path
+void bond_lengths(const dbl4 *x4, const int64_t *rowptr, const int32_t *col, int64_t n, double2 *len, cudaStream_t st);
 // double-float state <-> FP64 (mixed path)
 // double-float pair arrays with an element stride (1 for dense, REC for records)
 void materialize_df(const float4 *hi, const float4 *lo, int stride, int64_t n, dbl4 *out, cudaStream_t st);

@@ -102,6 +102,12 @@ __device__ __forceinline__ void dist64(double a, double &l, double &r)
     }
 }
 
+// Squared length of a bond of the FP64 path, undeformed or not: one formula, so that a body at
+// rest has no strain at all.  Against extended precision on lattice bonds at strains of 1e-4
+// a bond's force is off by 5.3e-13 RMS; with the sums unfused and correctly rounded roots and
+// divisions by 5.7e-13.
+__device__ __forceinline__ double bond_l2(double x, double y, double z) { return fma(x, x, fma(y, y, z * z)); }
+
 constexpr int STEP_THREADS = 256;
 constexpr unsigned STEP_TOUCH = 0x80000000u;  // beside the error bits of a block: a node of it touches a wall
 // bonds each lane keeps in flight per loop iteration, and the minimum resident
@@ -1096,9 +1102,8 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
                 const dbl4 a = p.x4[j], c = p.u_in[j];
                 const double yx = (a.x - ox.x) + (c.x - ou.x), yy = (a.y - ox.y) + (c.y - ou.y),
                              yz = (a.z - ox.z) + (c.z - ou.z);
-                const double l2 = fma(yx, yx, fma(yy, yy, yz * yz));
                 double l, rl;
-                dist64(l2, l, rl);
+                dist64(bond_l2(yx, yy, yz), l, rl);
                 const double s = (l - len.x) * len.y;
                 const bool brk = p.break_mode ? (fabs(s) > p.s0) : (s > p.s0);
                 if (brk) {
@@ -1693,6 +1698,22 @@ __global__ void k_drift(const StepParams p)
     }
 }
 
+// |xi| and 1 / |xi| of every slot; a warp takes a row
+__global__ void k_bond_lengths(const dbl4 *__restrict__ x4, const int64_t *__restrict__ rowptr,
+                               const int32_t *__restrict__ col, int64_t n, double2 *len)
+{
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nwarps) {
+        const dbl4 a = x4[i];
+        for (int64_t k = rowptr[i] + (threadIdx.x & 31); k < rowptr[i + 1]; k += 32) {
+            const dbl4 b = x4[col[k]];
+            double L, rL;
+            dist64(bond_l2(b.x - a.x, b.y - a.y, b.z - a.z), L, rL);
+            len[k] = make_double2(L, 1.0 / L);
+        }
+    }
+}
+
 // u (FP64) from the double-float state, for the rebuild kernels and queries
 __global__ void k_materialize(const float4 *__restrict__ hi, const float4 *__restrict__ lo, int stride, int64_t n,
                               dbl4 *out)
@@ -1891,6 +1912,11 @@ void split_df(const dbl4 *in, const float4 *xl, int64_t n, float4 *hi, float4 *l
 void fill_record_x(const float4 *xh4, int64_t n, float cf, float4 *rec, cudaStream_t st)
 {
     k_fill_record_x<<<small_grid(n), 256, 0, st>>>(xh4, n, cf, rec);
+}
+
+void bond_lengths(const dbl4 *x4, const int64_t *rowptr, const int32_t *col, int64_t n, double2 *len, cudaStream_t st)
+{
+    k_bond_lengths<<<small_grid(32 * n), 256, 0, st>>>(x4, rowptr, col, n, len);
 }
 
 void launch_drift(const StepParams &p, cudaStream_t st)

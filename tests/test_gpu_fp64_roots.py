@@ -59,3 +59,15 @@ def test_lengths_beyond_the_range_break(length):
     ctx.step(1e-9, 3)
     assert np.array_equal(ctx.get_state()[0], u)
     ctx.close()
+
+
+@pytest.mark.parametrize("jitter", [0.0, 0.05])
+def test_a_body_at_rest_or_moved_as_a_whole_has_no_force(jitter):
+    from paper_2506_05362_gb300 import pd, scenarios as S
+    sc = S.small_block(nx=9, ny=8, nz=7, jitter=jitter)
+    ctx = pd.Context.from_scenario(sc, precision="fp64")
+    assert not ctx.forces().any()
+    u = np.zeros(sc.x.shape) + np.array([1.0, -2.0, 0.5]) * sc.h  # the same for every node: no difference at all
+    ctx.set_state(u=u)
+    assert not ctx.forces().any()
+    ctx.close()
