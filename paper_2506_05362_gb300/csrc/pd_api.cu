@@ -83,7 +83,7 @@ struct pd_ctx {
     int32_t *split = nullptr, *mir = nullptr;
     float *tb = nullptr;
     float4 *fup = nullptr;
-    bool pairs_ok = false, pairs = false;
+    bool pairs = false;
     // several steps per launch (cooperative multi-step kernel of the global kernels)
     unsigned *gbar = nullptr;
     bool persist = false;
@@ -748,7 +748,7 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
     release(c, c->rowptr); release(c, c->col); release(c, c->brk); release(c, c->kc_of);
     release(c, c->crow); release(c, c->snap_brk); release(c, c->stage_b); release(c, c->stage_bits);
     release(c, c->split); release(c, c->mir); release(c, c->tb); release(c, c->fup);
-    c->pairs_ok = c->pairs = false;
+    c->pairs = false;
     c->delta = horizon;
     constants(c);
     const int64_t n = c->n;
@@ -882,7 +882,7 @@ pd_status pd_build_bonds(pd_ctx *c, double horizon, int nfilt, const pd_bond_fil
         s = sync(c);
         if (s) return s;
         if (bad) return fail(c, PD_ECUDA, "bond list is not symmetric");
-        c->pairs_ok = c->pairs = true;
+        c->pairs = true;
     }
     CK(cudaGetLastError());
     s = sync(c);

@@ -151,8 +151,6 @@ int radix_blocks(int64_t n);
 int64_t radix_tmp_size(int64_t n);
 void radix_sort_u64(uint64_t **k, uint64_t **kalt, uint32_t **v, uint32_t **valt, int64_t n, int bits,
                     int64_t *hist, cudaStream_t st);
-void radix_sort_u32(uint32_t **k, uint32_t **kalt, uint32_t **v, uint32_t **valt, int64_t n, int bits,
-                    int64_t *hist, cudaStream_t st);
 // Fragments (pd_frag.cu): connected components over intact bonds.  label and
 // is_label are in caller order; parent and minc are n-element scratch.
 void fragments_device(const int64_t *rowptr, const int32_t *col, const uint32_t *brk, const int32_t *perm,

@@ -512,7 +512,6 @@ struct pd_mlp {
     // dZ[l] transposed [pad[l+1] x ldT]
     bf16 *HT[8] = {nullptr}, *dZT[8] = {nullptr};
     int64_t ldT = 0;
-    int tc_train = -1;        // -1: untried; 1: tcgen05 training works here; 0: mma.sync
     float *Y = nullptr, *Xf = nullptr, *Tf = nullptr;
     float *part = nullptr;    // split-K partials
     int64_t part_cap = 0;

@@ -207,12 +207,6 @@ void radix_sort_u64(uint64_t **k, uint64_t **kalt, uint32_t **v, uint32_t **valt
     radix_impl<uint64_t>(k, kalt, v, valt, n, bits, hist, st);
 }
 
-void radix_sort_u32(uint32_t **k, uint32_t **kalt, uint32_t **v, uint32_t **valt, int64_t n, int bits,
-                    int64_t *hist, cudaStream_t st)
-{
-    radix_impl<uint32_t>(k, kalt, v, valt, n, bits, hist, st);
-}
-
 void scan_exclusive_i64(const int64_t *in, int64_t *out, int64_t n, int64_t *tmp, cudaStream_t st)
 {
     scan_impl<int64_t>(in, out, n, tmp, st);
