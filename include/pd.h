@@ -137,7 +137,9 @@ typedef struct {
                                             is PD_EINVAL */
     int persistent;                      /* pd_step runs the steps between two contact-list
                                             rebuilds in one cooperative launch (a grid-wide
-                                            barrier between steps; same results bit for bit):
+                                            barrier between steps; the same trajectory bit for
+                                            bit, wall reactions and impulses up to the order of
+                                            their FP64 sums):
                                             1 = on, -1 = off, 0 = chosen by the library.  Applies
                                             to the per-slot global-gather kernels; ignored while
                                             profiling. */

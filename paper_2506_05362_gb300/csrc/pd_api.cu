@@ -975,8 +975,6 @@ pd_status pd_stable_dt(pd_ctx *c, double *dt)
 }
 
 // ---- stepping -------------------------------------------------------------------
-// Enqueues one chunk of `steps` Verlet steps starting from u[parity]; contact
-// lists are rebuilt before the first step and then every k steps.
 // Grid of the multi-step kernel: resident blocks, at most one per GPB rows.
 static int persist_grid(const pd_ctx *c)
 {
@@ -989,7 +987,9 @@ static int persist_grid(const pd_ctx *c)
     return b;
 }
 
-// resume: the rest of a chunk that a stale list interrupted, u[parity] being drifted already.
+// Enqueues one chunk of `steps` Verlet steps starting from u[parity]; contact lists are
+// rebuilt before the first step (unless skip0) and then every k steps.  resume: the rest of a
+// chunk that a stale list interrupted, u[parity] being drifted already.
 static int64_t enqueue_chunk(pd_ctx *c, int steps, int k, int parity, double dt, bool skip0 = false,
                              bool resume = false)
 {
@@ -1207,9 +1207,9 @@ static int64_t chunk_len(const pd_ctx *c, int64_t m, int head, int k, int64_t at
 // was, so a rebuild and the rest of the steps follow, with the period that the list
 // lasted.  (It was rolled back to its start and run again before, up to twice the work:
 // records of 64 steps of the 47,808-node aggregate between moving walls, where every
-// other record's first period is too long, 9.2 ms on average, 6.8 ms now.)  A segment
-// whose list outgrew its capacity, or
-// that saw any other error, is rolled back to its own start, and run again for the former.
+// other record's first period is too long, 9.2 ms on average, 6.8 ms now.)  A segment whose
+// list outgrew its capacity, or that saw any other error, is rolled back to its own start, and
+// run again for the former.
 static pd_status run_segment(pd_ctx *c, double dt, int64_t left, int64_t *m_out, int64_t *launches, double *ms_out,
                              double *force_ms_out)
 {

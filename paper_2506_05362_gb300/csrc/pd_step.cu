@@ -1201,8 +1201,8 @@ __device__ __forceinline__ void process_row(const StepParams &p, const double *w
 
 // A block's part of the step: the wall reactions summed over its groups (a warp per
 // component, lanes striding over the groups, a fixed xor butterfly; zeros if no node
-// touches a wall) to partials[c][block], the largest |v|^2 into *vmax_bits (a max does not depend on
-// order), the error bits.  Adding 64 groups' sums in turn in one thread a component, and as
+// touches a wall) to partials[c][block], the largest |v|^2 into *vmax_bits (a max does not
+// depend on order), the error bits.  Adding 64 groups' sums in turn in one thread a component, and as
 // many maxima in another, took a third of a block's fixed cost of 2.8 us.
 template <int GPB>
 __device__ __forceinline__ void block_partials(const StepParams &p, const double (*s_react)[PD_MAX_WALLS * 3],
@@ -1284,9 +1284,9 @@ __device__ __forceinline__ void block_finish(const StepParams &p, const double (
     if (!s_last) return;
     __threadfence();
     // each chain of dependent global accesses in a thread of its own, side by side: one
-    // thread moving 6 walls in turn took 6.5 us of every step, at the end of which the
-    // other SMs wait (hollow sphere of 343,846 nodes
-    // between two walls 165 -> 160 us a step, of 37,272 nodes 32.0 -> 27.9)
+    // thread moving 6 walls in turn took 6.5 us of every step, at the end of which the other
+    // SMs wait (hollow sphere of 343,846 nodes between two walls 165 -> 160 us a step, of
+    // 37,272 nodes 32.0 -> 27.9)
     if (threadIdx.x < 32 && p.mode == MODE_FULL) advance_walls(p);
     for (int c = threadIdx.x >> 5; c < ncomp; c += STEP_THREADS / 32) sum_reaction(p, p.partials, c);
     if (threadIdx.x == STEP_THREADS - 1) {
@@ -1364,12 +1364,14 @@ __global__ void __launch_bounds__(STEP_THREADS, MIXED ? PD_MINB_GLOBAL : 2) k_st
 // ---- Several steps in one launch ------------------------------------------------
 // A run of MODE_FULL steps between two contact-list rebuilds in one cooperative
 // launch: each step does what one k_step launch does (the same rows, the same
-// arithmetic, the same fixed-order reductions), separated by a grid-wide barrier,
-// so the trajectory is bit for bit that of one launch per step while the launch
-// cost and the gap between launches are paid once per run.  Every block keeps
-// its own copy of the wall positions and of the skin bookkeeping and advances
-// them identically; the first blocks write the wall reactions and impulses, a
-// component each, block 0 at the end the walls, displacement bound and stale flag.  Even steps use the
+// arithmetic), separated by a grid-wide barrier, so the trajectory is bit for bit
+// that of one launch per step while the launch cost and the gap between launches
+// are paid once per run.  The wall reactions and impulses, which no step reads, are
+// summed in a fixed order too, but over this kernel's grid: where it has other
+// blocks than k_step's they differ in the last bits.  Every block keeps its own copy
+// of the wall positions and of the skin bookkeeping and advances them identically;
+// the first blocks write the wall reactions and impulses, a component each, block 0
+// at the end the walls, displacement bound and stale flag.  Even steps use the
 // parameters pa (state buffers in -> out), odd steps pb (out -> in).
 
 constexpr unsigned BAR_ABORT = 0x80000000u;     // set in the barrier word by a block that gave up
