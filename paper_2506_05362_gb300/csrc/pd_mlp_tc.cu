@@ -52,6 +52,7 @@ struct Layer {
     int K;        // padded input width (multiple of 16)
     int N;        // padded output width (multiple of 16, <= 256)
     int kchunks;  // ceil(K / 64)
+    int clear;    // first of the 32 columns that the epilogue clears in the next layer's tile, or 0
     const float *bias;  // N_pad floats
 };
 
@@ -329,11 +330,13 @@ __device__ __forceinline__ void load_bias(const float *bias, float (&b)[N])
     }
 }
 
-// bias + GELU + BF16 of the N accumulator columns [c, c + N) of row m, written to the next
-// layer's swizzled A tile
+// bias (of column c on) + GELU + BF16 of the N accumulator columns [c, c + N) of row m, written
+// to the next layer's swizzled A tile
 template <int N>
-__device__ __forceinline__ void epi_hidden(const float (&bb)[N], const uint32_t (&r)[N], int c, unsigned char *sA, int m)
+__device__ __forceinline__ void epi_hidden(const float *bias, const uint32_t (&r)[N], int c, unsigned char *sA, int m)
 {
+    float bb[N];
+    load_bias(bias, bb);
 #pragma unroll
     for (int c8 = 0; c8 < N; c8 += 8) {
         uint32_t pk[4];
@@ -575,8 +578,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
                     const int cend = min(Ly.N, (part + 1) * hw);
                     const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * MAX_N);
                     // hidden layers of whole 32-column chunks (training has no others): the
-                    // TMEM load and the biases of the next 16 columns are in flight while
-                    // the current 16 go through GELU
+                    // TMEM load of the next 16 columns is in flight while the current 16 go
+                    // through GELU (in training also their biases, 8 columns at a time; in
+                    // inference that spills: 65,536 rows 69.1 us, 69.7 by 8 columns, and 66.4
+                    // with the biases loaded where they are added)
                     const bool piped = MODE == TRAIN_BWD || (!last && (TRAIN || (Ly.N % 32) == 0));
                     if (MODE == TRAIN_BWD) {  // as below, with the pre-activations instead of the biases
                         if (part * hw < cend) {
@@ -642,24 +647,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
                         }
                     } else if (piped && part * hw < cend) {
                         uint32_t ra[16], rb[16];
-                        float ba[16], bb[16];
                         __syncwarp();  // tcgen05.ld is warp-collective
                         tmem_ld16_issue(tacc + (uint32_t)(part * hw), ra);
-                        load_bias(Ly.bias + part * hw, ba);
                         tmem_wait16(ra);
                         for (int c0 = part * hw; c0 < cend; c0 += 32) {  // bounds uniform in the warp
                             __syncwarp();
                             tmem_ld16_issue(tacc + (uint32_t)(c0 + 16), rb);
-                            load_bias(Ly.bias + c0 + 16, bb);
-                            epi_hidden(ba, ra, c0, sA, m);
+                            epi_hidden(Ly.bias + c0, ra, c0, sA, m);
                             tmem_wait16(rb);
                             const bool more = c0 + 32 < cend;
                             if (more) {
                                 __syncwarp();
                                 tmem_ld16_issue(tacc + (uint32_t)(c0 + 32), ra);
-                                load_bias(Ly.bias + c0 + 32, ba);
                             }
-                            epi_hidden(bb, rb, c0 + 16, sA, m);
+                            epi_hidden(Ly.bias + c0 + 16, rb, c0 + 16, sA, m);
                             if (more) tmem_wait16(ra);
                         }
                     }
@@ -711,11 +712,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_tc(const __grid_constant__ M
                         }
                     }
                     if (!last) {
-                        // The next layer's MMAs read whole chunks of 64 columns.  Those past N
-                        // meet zero weights, but zero times what an earlier kernel or tile left
-                        // there (an infinity, a NaN) is not zero: they are cleared.
-                        const int cz = (Ly.N + 31) & ~31;  // up to here columns are written above
-                        if (cz & 32) *(uint4 *)(sA + sw128_offset(m, cz + 8 * part)) = make_uint4(0u, 0u, 0u, 0u);
+                        if (Ly.clear) *(uint4 *)(sA + sw128_offset(m, Ly.clear + 8 * part)) = make_uint4(0u, 0u, 0u, 0u);
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         mbar_arrive(a_ready + b);
@@ -1142,6 +1139,11 @@ bool fused_setup(int L, const int *pad, void *const *W, int64_t rows, unsigned *
         P.layer[l].K = pad[l];
         P.layer[l].N = pad[l + 1];
         P.layer[l].kchunks = (pad[l] + KCHUNK - 1) / KCHUNK;
+        // The next layer's MMAs read whole chunks of 64 columns.  Those past N meet zero weights,
+        // but zero times what an earlier kernel or tile left there (an infinity, a NaN) is not
+        // zero: they are cleared.  Up to the next multiple of 32 the epilogue writes them anyway.
+        const int written = (pad[l + 1] + 31) / 32 * 32;
+        P.layer[l].clear = written % 64 ? written : 0;
     }
     P.rows = rows;
     P.err = err;
