@@ -62,12 +62,16 @@ __global__ void k_frag_union(const int64_t *__restrict__ rowptr, const int32_t *
     }
 }
 
-// full compression, then the smallest caller index of each root's set
+// Full compression, then the smallest caller index of each root's set.  A thread writes its
+// own node's parent only: with path halving here, one that read a node's parent before the
+// node's thread stored the root could store an older ancestor over it after.
 __global__ void k_frag_compress(int32_t *parent, const int32_t *__restrict__ perm, int32_t *minc, int64_t n)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t r = rep(parent, (int32_t)i);
-        parent[i] = r;
+        volatile int32_t *vp = parent;
+        int32_t r = vp[i], next;
+        while ((next = vp[r]) != r) r = next;
+        vp[i] = r;
         atomicMin(minc + r, perm[i]);
     }
 }
