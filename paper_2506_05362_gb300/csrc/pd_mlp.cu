@@ -399,8 +399,8 @@ __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float
     }
 }
 
-// Everything after the last GEMM of a tcgen05 training step in one launch: the parts of
-// every layer's weight gradient summed in order into the gradient vector, and, for a
+// Everything after the last GEMM of a tcgen05 training step in one launch: the partial sums of
+// every layer's weight gradient added in order into the gradient vector, and, for a
 // training step, Adam on it and the new weights and biases in the layouts the GEMMs read
 // (their padding stays as it was set); block 0 also sums the loss, as k_loss_final does.  A
 // thread takes one parameter, its partials' loads all in flight: bound by their latency (8
@@ -457,9 +457,34 @@ __global__ void __launch_bounds__(256) k_update(const __grid_constant__ Update U
     const int r = isw ? q / Y.k_valid : q, c = isw ? q - r * Y.k_valid : 0;
     const float *src = isw ? Y.part + (size_t)r * Y.K + c : Y.gb + r;
     const size_t zs = (size_t)Y.N * Y.K;
-    float g = __ldcs(src);
+    float g;
+    if (!isw || Y.parts <= RD_PARTS) {  // one sum a class
+        g = __ldcs(src);
 #pragma unroll 7
-    for (int z = 1; z < (isw ? Y.parts : 1); ++z) g += __ldcs(src + (size_t)z * zs);
+        for (int z = 1; z < (isw ? Y.parts : 1); ++z) g += __ldcs(src + (size_t)z * zs);
+    } else {  // one a split: the splits of a class in turn, then the classes
+        constexpr int AHEAD = 4;  // 32 loads in flight; those past the end add zero
+        float cls[RD_PARTS];
+#pragma unroll
+        for (int w = 0; w < RD_PARTS; ++w) cls[w] = 0.f;
+        for (int z0 = 0; z0 < Y.parts; z0 += AHEAD * RD_PARTS) {
+            float v[AHEAD][RD_PARTS];
+#pragma unroll
+            for (int a = 0; a < AHEAD; ++a)
+#pragma unroll
+                for (int w = 0; w < RD_PARTS; ++w) {
+                    const int z = z0 + a * RD_PARTS + w;
+                    v[a][w] = z < Y.parts ? __ldcs(src + (size_t)z * zs) : 0.f;
+                }
+#pragma unroll
+            for (int a = 0; a < AHEAD; ++a)
+#pragma unroll
+                for (int w = 0; w < RD_PARTS; ++w) cls[w] += v[a][w];
+        }
+        g = cls[0];
+#pragma unroll
+        for (int w = 1; w < RD_PARTS; ++w) g += cls[w];
+    }
     U.g[p] = g;
     if (!U.adam) return;
     const float w = adam_step(U.w[p], g, U.m[p], U.v[p], U.lr, U.b1, U.b2, U.eps, U.c1, U.c2);
@@ -728,7 +753,7 @@ int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float l
     int64_t need = 0, at[8];
     for (int l = 0; l < L; ++l) {
         at[l] = need;
-        need += (int64_t)m->pad[l + 1] * (mlp_dw_parts(m->pad[l + 1], rows, m->device, nullptr, nullptr) * m->pad[l] + 1);
+        need += (int64_t)m->pad[l + 1] * (mlp_dw_parts(L, m->pad, l, rows, m->device, nullptr, nullptr) * m->pad[l] + 1);
         need = (need + 31) / 32 * 32;
     }
     if (mlp_forward_tc(L, m->dims, m->pad, W, b, X, rows, nullptr, &tr, m->tc_err, m->device, m->st)) return -1;
@@ -743,7 +768,7 @@ int backward_tc(pd_mlp *m, const float *X, const float *T, int64_t rows, float l
     for (int l = 0; l < L; ++l) {
         const int N = m->pad[l + 1], K = m->pad[l];
         UpdateLayer &Y = U.l[l];
-        Y.parts = mlp_dw_parts(N, rows, m->device, nullptr, nullptr);
+        Y.parts = mlp_dw_parts(L, m->pad, l, rows, m->device, nullptr, nullptr);
         part[l] = m->part + at[l];
         gb[l] = part[l] + (int64_t)Y.parts * N * K;
         Y.part = part[l]; Y.gb = gb[l]; Y.N = N; Y.K = K;

@@ -26,9 +26,9 @@ int mlp_forward_tc(int L, const int *dims, const int *pad, void *const *W, const
 // negative number if it cannot run.
 int mlp_backward_tc(int L, const int *pad, void *const *WT, const MlpTrain *tr, void *const *dZT, int64_t rows,
                     unsigned *err, int device, cudaStream_t st);
-// Partial sums (at most 8) that mlp_dw_tc leaves of a layer's weight gradient; kcs, splits
-// (nullable): 64-row chunks per split of the batch, splits.
-int mlp_dw_parts(int pad_out, int64_t rows, int device, int *kcs, int *splits);
+// Partial sums that mlp_dw_tc leaves of layer l's weight gradient: of at most 8 classes of
+// splits, or of every split; kcs, splits (nullable): 64-row chunks per split, splits.
+int mlp_dw_parts(int L, const int *pad, int l, int64_t rows, int device, int *kcs, int *splits);
 // Sums of a training step over the batch: of every layer the partial weight gradients
 // part[l] [parts x pad[l+1] x pad[l]] of dW = dZ^T H and the bias gradient gb[l]
 // [dims[l+1]], and the nlp partial sums tr.lpart of (Y - T)^2, all FP32; dZT[l] [pad[l+1] x

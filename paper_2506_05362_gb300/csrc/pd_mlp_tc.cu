@@ -758,17 +758,21 @@ encode_fn_t encoder()
 // Both operands K-major and fed by TMA (same 128-byte swizzle as above), all layers in one
 // launch.  The batch is cut into splits as many as give every SM a CTA of a layer's 128-row
 // tiles; a split's sum is one accumulator in TMEM, and the splits are added in FP32 in the
-// order of k_reduce_dw: z = p, p + 8, p + 16, ... to part p, the parts in turn (k_update).
+// order of k_reduce_dw: z = p, p + 8, p + 16, ... to class p, the classes in turn.
 // (The grouping is part of the result: Adam divides small gradients by their own size, so
 // that sums grouped otherwise are other weights after some steps.)  A CTA takes one 128 x
-// 128 tile of one layer's C and one part: its splits go through two TMEM accumulators in
-// turn, and the epilogue warps add one to the part, in registers, while the other fills.
-// So the eight parts go to memory and not the 74 splits of the surrogate's hidden layers at
+// 128 tile of one layer's C and one class: its splits go through two TMEM accumulators in
+// turn, and the epilogue warps add one to the sum, in registers, while the other fills.
+// So eight partial sums go to memory and not the 74 splits of the surrogate's hidden layers at
 // batch 65,536 (67 MB a step).  Tiles of 128 columns, since with 256 the surrogate's eight
 // parts are 72 CTAs for 152 SMs; they read A twice, 670 MB with the row sums: 74 us, 9.1
 // TB/s out of L2 (19 us at batch 4,096).  The nine GEMM launches of the data and weight
 // gradients and the row sums took 348 us (129 us) before; this and the fused data gradients
-// take 203 us (59 us).
+// take 203 us (59 us).  Where the layers have so few tiles that eight CTAs each would take
+// less than a sixth of the SMs, a CTA takes one split and k_update adds the splits class by
+// class (a training step of the 7-2 network, 1 tile, at batch 262,144 206 -> 92 us, at 4,096
+// 24 -> 22; 1-64-32-1, 3 tiles, 382 -> 296, at 4,096 41 -> 43; 256-256, 4 tiles, would go
+// from 1,249 to 1,268 and from 88 to 98).
 //
 // The first CTAs of the grid, and the others once their tile is done, take the sums that
 // need no tensor cores, from a common counter, a warp each: the rows of dZ^T (the bias
@@ -780,13 +784,14 @@ constexpr int G_THREADS = 64 + G_EPI;
 constexpr int G_STAGE = TILE_M * KCHUNK * 2;  // 16 KiB of either operand
 constexpr int G_STAGES = 6;
 constexpr int G_COLS = 128;                   // columns of a tile of C
-constexpr int DW_PARTS = 8;                   // = RD_PARTS of k_reduce_dw
+constexpr int DW_CLASSES = 8;                 // = RD_PARTS of k_reduce_dw
 
 struct DwLayer {
     CUtensorMap ma, mb;
     int M, N;            // rows of C that exist, columns
-    int tile0, nt;       // the layer's first tile, its tiles beside one another
+    int cta0, nt;        // the layer's first CTA, its tiles beside one another
     int kcs, splits;     // K chunks per split, splits
+    int parts;           // CTAs, and partial sums, a tile: CTA p takes splits p, p + parts, ...
     float *part;
     const __nv_bfloat16 *dZT;
     float *gb;           // bias gradient
@@ -796,7 +801,7 @@ struct DwArgs {
     DwLayer l[MAX_LAYERS];
     int L, kchunks, free_ctas;
     int64_t rows, ldT;
-    int sum_rows;        // of all layers
+    int sum_rows;        // of all layers (0: summed by k_rowsum)
     const float *Y, *T;  // [rows x nout]
     int nout, ldo, nlp;
     float *lpart;
@@ -898,14 +903,15 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ 
 {
     constexpr int S = G_STAGES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tile = ((int)blockIdx.x - A.free_ctas) / DW_PARTS, p = ((int)blockIdx.x - A.free_ctas) % DW_PARTS;
-    int layer = 0;
-    while (layer + 1 < A.L && tile >= A.l[layer + 1].tile0) ++layer;
-    const DwLayer &P = A.l[layer];
-    if ((int)blockIdx.x < A.free_ctas || p >= P.splits) {
+    const int cta = (int)blockIdx.x - A.free_ctas;
+    if (cta < 0) {
         take_sums(A, lane);
         return;
     }
+    int layer = 0;
+    while (layer + 1 < A.L && cta >= A.l[layer + 1].cta0) ++layer;
+    const DwLayer &P = A.l[layer];
+    const int tile = (cta - P.cta0) / P.parts, p = (cta - P.cta0) % P.parts;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *sA = base;                      // S x 16 KiB
@@ -940,7 +946,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ 
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
-    const int m0 = (tile - P.tile0) / P.nt * TILE_M, n0 = (tile - P.tile0) % P.nt * G_COLS;
+    const int m0 = tile / P.nt * TILE_M, n0 = tile % P.nt * G_COLS;
     const int cols = min(G_COLS, P.N - n0);
 
     if (warp == 0) {
@@ -951,7 +957,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ 
             for (int q = 0; q < S; ++q) last_ph[q] = -1;
             // a box of B has min(N, 128) rows; those beyond N arrive as zeros
             const uint32_t bytes = (uint32_t)(G_STAGE + min(P.N, G_COLS) * KCHUNK * 2);
-            for (int z = p; z < P.splits && !s_abort; z += DW_PARTS) {
+            for (int z = p; z < P.splits && !s_abort; z += P.parts) {
                 const int kc1 = min(A.kchunks, (z + 1) * P.kcs);
                 for (int kc = z * P.kcs; kc < kc1 && !s_abort; ++kc) {
                     if (!mbar_wait(empty + s, ph ^ 1)) { atomicOr(A.err, 1u); s_abort = 1; break; }
@@ -970,7 +976,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ 
             int s = 0, b = 0;
             uint32_t ph = 0, fph = 1;  // both accumulators are free at the start
             const uint32_t idesc = idesc_bf16(TILE_M, cols);
-            for (int z = p; z < P.splits && !s_abort; z += DW_PARTS) {
+            for (int z = p; z < P.splits && !s_abort; z += P.parts) {
                 if (!mbar_wait(acc_free + b, fph)) { atomicOr(A.err, 1u); s_abort = 1; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d = tmem + (uint32_t)(b * G_COLS);
@@ -1003,7 +1009,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_dw_tc(const __grid_constant__ 
         int b = 0;
         uint32_t ph = 0;
         bool ok = true;
-        for (int z = p; z < P.splits; z += DW_PARTS) {
+        for (int z = p; z < P.splits; z += P.parts) {
             __syncwarp();
             ok = mbar_wait(acc_full + b, ph);
             if (!ok) { atomicOr(A.err, 1u); s_abort = 1; }
@@ -1055,16 +1061,62 @@ bool kmajor_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, i
 
 }  // namespace
 
-int mlp_dw_parts(int pad_out, int64_t rows, int device, int *kcs, int *splits)
+// Row sums of a layer's dZ^T as row_sum() adds them, one block a row of any layer: for few
+// long rows, of which a warp each would be one chain of loads.
+constexpr int RS_THREADS = 1024;
+__global__ void __launch_bounds__(RS_THREADS) k_rowsum(const __grid_constant__ DwArgs A)
 {
-    int sms = 1;
+    __shared__ float s[RS_THREADS];
+    int l = 0;
+    while (l + 1 < A.L && (int)blockIdx.x >= A.l[l + 1].row0) ++l;
+    const int64_t row = (int)blockIdx.x - A.l[l].row0;
+    const __nv_bfloat16 *r = A.l[l].dZT + row * A.ldT;
+    const int64_t r8 = A.rows / 8;
+    float acc = 0.f;
+    constexpr int BATCH = 8;  // loads in flight
+    for (int64_t q0 = threadIdx.x; q0 < r8; q0 += (int64_t)BATCH * RS_THREADS) {
+        uint4 w[BATCH];
+#pragma unroll
+        for (int b = 0; b < BATCH; ++b) {
+            const int64_t q = q0 + (int64_t)b * RS_THREADS;
+            w[b] = q < r8 ? __ldcs((const uint4 *)r + q) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int b = 0; b < BATCH; ++b) {
+            const uint32_t h[4] = {w[b].x, w[b].y, w[b].z, w[b].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 f = __bfloat1622float2(*(const __nv_bfloat162 *)&h[e]);
+                acc += f.x + f.y;
+            }
+        }
+    }
+    if (8 * r8 + threadIdx.x < A.rows) acc += __bfloat162float(r[8 * r8 + threadIdx.x]);  // fewer than 8
+    s[threadIdx.x] = acc;
+    __syncthreads();
+    for (int o = RS_THREADS / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) A.l[l].gb[row] = s[0];
+}
+
+static int layer_tiles(const int *pad, int l)
+{
+    return (pad[l + 1] + TILE_M - 1) / TILE_M * ((pad[l] + G_COLS - 1) / G_COLS);
+}
+
+int mlp_dw_parts(int L, const int *pad, int l, int64_t rows, int device, int *kcs, int *splits)
+{
+    int sms = 1, tiles = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    const int kchunks = (int)((rows + KCHUNK - 1) / KCHUNK), mt = (pad_out + TILE_M - 1) / TILE_M;
+    for (int i = 0; i < L; ++i) tiles += layer_tiles(pad, i);
+    const int kchunks = (int)((rows + KCHUNK - 1) / KCHUNK), mt = (pad[l + 1] + TILE_M - 1) / TILE_M;
     const int most = std::max(1, std::min(128, sms / mt));
     const int k = (kchunks + most - 1) / most, n = (kchunks + k - 1) / k;  // no split without work
     if (kcs) *kcs = k;
     if (splits) *splits = n;
-    return std::min(n, DW_PARTS);
+    return 6 * DW_CLASSES * tiles < sms ? n : std::min(n, DW_CLASSES);
 }
 
 int mlp_dw_tc(int L, const int *dims, const int *pad, void *const *dZT, void *const *HT, int64_t rows, const MlpTrain &tr,
@@ -1085,16 +1137,16 @@ int mlp_dw_tc(int L, const int *dims, const int *pad, void *const *dZT, void *co
     A.lpart = tr.lpart;
     A.next = tr.next;
     A.err = err;
-    int tiles = 0;
+    int ctas = 0;
     for (int l = 0; l < L; ++l) {
         DwLayer &Y = A.l[l];
         Y.M = pad[l + 1];
         Y.N = pad[l];
         if (Y.N < 16 || Y.N > 2 * G_COLS || Y.N % 16) return -1;
-        Y.tile0 = tiles;
         Y.nt = (Y.N + G_COLS - 1) / G_COLS;
-        tiles += (Y.M + TILE_M - 1) / TILE_M * Y.nt;
-        mlp_dw_parts(Y.M, rows, device, &Y.kcs, &Y.splits);
+        Y.parts = mlp_dw_parts(L, pad, l, rows, device, &Y.kcs, &Y.splits);
+        Y.cta0 = ctas;
+        ctas += layer_tiles(pad, l) * Y.parts;
         Y.part = part[l];
         Y.dZT = (const __nv_bfloat16 *)dZT[l];
         Y.gb = gb[l];
@@ -1104,16 +1156,22 @@ int mlp_dw_tc(int L, const int *dims, const int *pad, void *const *dZT, void *co
             !kmajor_map(&Y.mb, HT[l], Y.N, rows, tr.ldT, std::min(Y.N, G_COLS)))
             return -1;
     }
-    // the sums start at once on the SMs that the tiles leave over
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    A.free_ctas = std::max(0, sms - tiles * DW_PARTS);
+    // few rows (less than one an SM) of which each would be a chain of four rounds of loads or
+    // more in a warp have a launch of their own (7-2 at batch 65,536 6 us)
+    if (rows >= 32768 && A.sum_rows < sms) {
+        k_rowsum<<<(unsigned)A.sum_rows, RS_THREADS, 0, st>>>(A);
+        A.sum_rows = 0;
+    }
+    // the sums start at once on the SMs that the tiles leave over
+    A.free_ctas = std::max(0, sms - ctas);
     static bool configured = false;
     if (!configured) {
         cudaFuncSetAttribute(k_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         configured = true;
     }
-    k_dw_tc<<<(unsigned)(A.free_ctas + tiles * DW_PARTS), G_THREADS, smem, st>>>(A);
+    k_dw_tc<<<(unsigned)(A.free_ctas + ctas), G_THREADS, smem, st>>>(A);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
