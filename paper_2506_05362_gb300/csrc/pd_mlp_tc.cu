@@ -408,44 +408,54 @@ struct Maps {
 // epilogue warps finish the other slot's previous item.
 __device__ __forceinline__ int64_t pair_tile(int64_t r, int b) { return blockIdx.x + (2 * r + b) * (int64_t)gridDim.x; }
 
-// input tile -> BF16 swizzled A tile (zero beyond the input width and the batch).  A warp
-// takes 16 rows of 64 columns, a lane two neighbouring columns (coalesced reads); in
-// training the lane's 16 rows of a column are 32 consecutive bytes of the transposed
-// input that the first weight gradient reads.
+// input tile -> BF16 swizzled A tile (zero beyond the input width and the batch), R rows m0 ..
+// of two neighbouring columns k, k + 1 a lane (coalesced reads); in training the lane's rows
+// of a column are consecutive bytes of the transposed input that the first weight gradient
+// reads.
+template <int MODE, int R>
+__device__ __forceinline__ void stage_rows(const Params &P, int64_t t, unsigned char *sA, int m0, int k)
+{
+    const int64_t r0 = t * TILE_M + m0;
+    uint32_t w[R];
+    const float *x = P.X + r0 * P.in_cols + k;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const bool in = r0 + i < P.rows;
+        if (MODE == TRAIN_BWD) {  // the loss gradient as it is (its width is a multiple of 16)
+            w[i] = in && k < P.layer[0].K ? *(const uint32_t *)(P.dY + (r0 + i) * P.layer[0].K + k) : 0u;
+            continue;
+        }
+        const float a = in && k < P.in_cols ? __ldg(x + (int64_t)i * P.in_cols) : 0.f;
+        const float b = in && k + 1 < P.in_cols ? __ldg(x + (int64_t)i * P.in_cols + 1) : 0.f;
+        w[i] = pack_bf16x2(a, b);
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) *(uint32_t *)(sA + sw128_offset(m0 + i, k)) = w[i];
+    if (MODE == TRAIN_FWD && k < P.layer[0].K && r0 < P.rows) {  // K is a multiple of 16: both columns exist
+        __nv_bfloat16 *h = P.HT[0] + (int64_t)k * P.ldT + r0;
+#pragma unroll
+        for (int c = 0; c < 2; ++c, h += P.ldT)
+#pragma unroll
+            for (int i = 0; i < R; i += 8)
+                if (i == 0 || r0 + i < P.ldT)  // ldT is the batch rounded up to 8 rows at least
+                    *(uint4 *)(h + i) = make_uint4(__byte_perm(w[i], w[i + 1], c ? 0x7632 : 0x5410),
+                                                   __byte_perm(w[i + 2], w[i + 3], c ? 0x7632 : 0x5410),
+                                                   __byte_perm(w[i + 4], w[i + 5], c ? 0x7632 : 0x5410),
+                                                   __byte_perm(w[i + 6], w[i + 7], c ? 0x7632 : 0x5410));
+    }
+}
+
+// A warp takes 16 rows of every other 64 columns, or, of inputs of one 64-column chunk, 8 rows
+// (half of the warps would be idle).
 template <int MODE>
 __device__ __forceinline__ void stage_input(const Params &P, int64_t t, unsigned char *sA, int warp, int lane)
 {
-    const int m0 = (warp >> 1) * 16;
-    const int64_t r0 = t * TILE_M + m0;
-    for (int k = 64 * (warp & 1) + 2 * lane; k < P.layer[0].kchunks * KCHUNK; k += 128) {
-        uint32_t w[16];
-        const float *x = P.X + r0 * P.in_cols + k;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const bool in = r0 + i < P.rows;
-            if (MODE == TRAIN_BWD) {  // the loss gradient as it is (its width is a multiple of 16)
-                w[i] = in && k < P.layer[0].K ? *(const uint32_t *)(P.dY + (r0 + i) * P.layer[0].K + k) : 0u;
-                continue;
-            }
-            const float a = in && k < P.in_cols ? __ldg(x + (int64_t)i * P.in_cols) : 0.f;
-            const float b = in && k + 1 < P.in_cols ? __ldg(x + (int64_t)i * P.in_cols + 1) : 0.f;
-            w[i] = pack_bf16x2(a, b);
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) *(uint32_t *)(sA + sw128_offset(m0 + i, k)) = w[i];
-        if (MODE == TRAIN_FWD && k < P.layer[0].K && r0 < P.rows) {  // K is a multiple of 16: both columns exist
-            __nv_bfloat16 *h = P.HT[0] + (int64_t)k * P.ldT + r0;
-#pragma unroll
-            for (int c = 0; c < 2; ++c, h += P.ldT) {
-                uint32_t v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = __byte_perm(w[2 * i], w[2 * i + 1], c ? 0x7632 : 0x5410);
-                *(uint4 *)h = make_uint4(v[0], v[1], v[2], v[3]);
-                // ldT is the batch rounded up to 8 rows at least
-                if (r0 + 8 < P.ldT) *((uint4 *)h + 1) = make_uint4(v[4], v[5], v[6], v[7]);
-            }
-        }
+    if (P.layer[0].kchunks == 1) {
+        stage_rows<MODE, 8>(P, t, sA, warp * 8, 2 * lane);
+        return;
     }
+    for (int k = 64 * (warp & 1) + 2 * lane; k < P.layer[0].kchunks * KCHUNK; k += 128)
+        stage_rows<MODE, 16>(P, t, sA, (warp >> 1) * 16, k);
 }
 
 template <int MODE>
