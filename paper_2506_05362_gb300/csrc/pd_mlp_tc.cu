@@ -775,10 +775,10 @@ encode_fn_t encoder()
 // turn, and the epilogue warps add one to the sum, in registers, while the other fills.
 // So eight partial sums go to memory and not the 74 splits of the surrogate's hidden layers at
 // batch 65,536 (67 MB a step).  Tiles of 128 columns, since with 256 the surrogate's eight
-// parts are 72 CTAs for 152 SMs; they read A twice, 670 MB with the row sums: 74 us, 9.1
+// parts are 72 CTAs for 152 SMs; they read A twice, 670 MB with the row sums: 71 us, 9.4
 // TB/s out of L2 (19 us at batch 4,096).  The nine GEMM launches of the data and weight
 // gradients and the row sums took 348 us (129 us) before; this and the fused data gradients
-// take 203 us (59 us).  Where the layers have so few tiles that eight CTAs each would take
+// take 196 us (59 us).  Where the layers have so few tiles that eight CTAs each would take
 // less than a sixth of the SMs, a CTA takes one split and k_update adds the splits class by
 // class (a training step of the 7-2 network, 1 tile, at batch 262,144 206 -> 92 us, at 4,096
 // 24 -> 22; 1-64-32-1, 3 tiles, 382 -> 296, at 4,096 41 -> 43; 256-256, 4 tiles, would go
